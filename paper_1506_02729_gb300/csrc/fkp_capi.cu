@@ -342,19 +342,19 @@ static int tune_schedule(Plan* P) {
     float bx = 1e30f, by = 1e30f, bz = 1e30f;
     for (int xm : {1, 2, 4, 8}) {
       const float t = timed([&] { return launch_xpass(P->d_grid, nullptr, P->g, P->mt, P->fp, P->d_tw, P->d_S1,
-                                                      P->ctx->nsm, s, xm); }, "x-pass");
+                                                      P->ctx->nsm, s, P->reach, xm); }, "x-pass");
       if (t < bx) { bx = t; best.x_mult = xm; }
     }
     for (int nt : {256, 512}) {
       const float t = timed([&] { return launch_ypass(P->d_S1, P->d_grid, nullptr, P->g, P->mt, P->fp, P->d_tw,
-                                                      P->d_S2, P->d_err + 1, s, nt); }, "y-pass");
+                                                      P->d_S2, P->d_err + 1, s, P->reach, nt); }, "y-pass");
       if (t < by) { by = t; best.y_threads = nt; }
     }
     // the z-pass block shape sets the partition of each k_z column into the
     // FP32 runs of the bin sums, so it is fixed per grid rather than tuned:
     // results then do not depend on the tuning (bit for bit)
     best.z_threads = z_threads_for(N);
-    bz = timed([&] { return launch_zpass(P->d_S2, P->g, P->mt, P->fp, P->d_tw, zp, P->d_zpart, P->d_zpartc,
+    bz = timed([&] { return launch_zpass(P->d_S2, P->g, P->mt, P->fp, P->d_tw, zp, P->reach, P->d_zpart, P->d_zpartc,
                                          P->d_err + 1, s, P->ctx->nsm, best.z_threads); }, "z-pass");
     best.ms[0] = bx;
     best.ms[1] = by;
@@ -508,6 +508,16 @@ extern "C" int fkp_plan_create(void* vctx, const fkp_geometry_t* geom, const fkp
     }
   }
   P->min_edge_gap = min_gap;
+  // the modes the passes carry: every bin's, and every shell's
+  int r2 = 0, r2w = 0;
+  for (int n2 = 1; n2 <= n2max; ++n2)
+    if (lut[n2] >= 0) r2 = n2;
+  if (wantB) {
+    const double hmax = bs->first + (bs->nshells - 1) * (double)bs->step + 0.5 * bs->width;
+    r2w = (int)std::ceil(hmax * hmax) - 1;  // n^2 < hmax^2
+    r2 = std::max(r2, r2w);
+  }
+  const std::vector<int> zt = reach_tiles(N, r2, P->reach), ztw = reach_tiles(N, r2w, P->reach_w);
   std::vector<float2> tw(N);
   for (int m = 0; m < N; ++m) {
     const double a = 2.0 * M_PI * (double)m / (double)N;
@@ -549,6 +559,9 @@ extern "C" int fkp_plan_create(void* vctx, const fkp_geometry_t* geom, const fkp
   P->d_tw = (float2*)A(sizeof(float2) * N);
   P->d_lut = (short*)A(sizeof(short) * (n2max + 1));
   P->d_winv = (float*)A(sizeof(float) * 3 * N);
+  int* d_ztiles = (int*)A(sizeof(int) * (zt.size() + ztw.size()));
+  P->reach.ztiles = d_ztiles;
+  P->reach_w.ztiles = d_ztiles + zt.size();
   P->d_scpart = (double*)A(sizeof(double) * SC_NSUM * 2 * P->nblk_cat);
   P->d_labpart = (double*)A(sizeof(double) * LAB_NSUM * P->nblk_cat);
   P->d_ds = (double*)A(sizeof(double) * (DS_COUNT + LAB_NSUM + 8));
@@ -582,6 +595,8 @@ extern "C" int fkp_plan_create(void* vctx, const fkp_geometry_t* geom, const fkp
   CK(cudaMemcpy(P->d_tw, tw.data(), sizeof(float2) * N, cudaMemcpyHostToDevice));
   CK(cudaMemcpy(P->d_lut, lut.data(), sizeof(short) * (n2max + 1), cudaMemcpyHostToDevice));
   CK(cudaMemcpy(P->d_winv, winv.data(), sizeof(float) * 3 * N, cudaMemcpyHostToDevice));
+  CK(cudaMemcpy(d_ztiles, zt.data(), sizeof(int) * zt.size(), cudaMemcpyHostToDevice));
+  CK(cudaMemcpy(d_ztiles + zt.size(), ztw.data(), sizeof(int) * ztw.size(), cudaMemcpyHostToDevice));
   CK(cudaMemcpy(P->d_hph, hph.data(), sizeof(float2) * N, cudaMemcpyHostToDevice));
   const size_t hbytes = sizeof(double) * (BQ_N * pb->nbins + pb->nbins + DS_COUNT + LAB_NSUM + 8) + 64;
   CK(cudaMallocHost(&P->h_pinned, hbytes));
@@ -879,17 +894,19 @@ ZParams fkp::zparams(const Plan* P, int mode) {
 }
 
 int fkp::enqueue_xy(Plan* P, const unsigned long long* gq, const unsigned long long* gq2, const float* gf,
-                    cudaStream_t s, bool events) {
-  CK(launch_xpass(gq, gf, P->g, P->mt, P->fp, P->d_tw, P->d_S1, P->ctx->nsm, s, P->sched.x_mult, MockBatch(),
+                    cudaStream_t s, const PassReach& pr, bool events) {
+  CK(launch_xpass(gq, gf, P->g, P->mt, P->fp, P->d_tw, P->d_S1, P->ctx->nsm, s, pr, P->sched.x_mult, MockBatch(),
                   P->per_object));
   if (events) CK(record_stage(P->ev[3], s));
-  CK(launch_ypass(P->d_S1, gq, gf, P->g, P->mt, P->fp, P->d_tw, P->d_S2, P->d_err + 1, s, P->sched.y_threads));
+  CK(launch_ypass(P->d_S1, gq, gf, P->g, P->mt, P->fp, P->d_tw, P->d_S2, P->d_err + 1, s, pr,
+                  P->sched.y_threads));
   if (P->interlace) {
     // the second grid's groups follow the first's; the z-pass applies its
     // half-cell phase e^{-i pi (n_x + n_y + n_z)/N}
     float2* S2b = P->d_S2 + field_elems(P->g.N) * P->mt.ngroups;
-    CK(launch_xpass(gq2, nullptr, P->g2, P->mt, P->fp, P->d_tw, P->d_S1, P->ctx->nsm, s, P->sched.x_mult));
-    CK(launch_ypass(P->d_S1, gq2, nullptr, P->g2, P->mt, P->fp, P->d_tw, S2b, P->d_err + 1, s, P->sched.y_threads));
+    CK(launch_xpass(gq2, nullptr, P->g2, P->mt, P->fp, P->d_tw, P->d_S1, P->ctx->nsm, s, pr, P->sched.x_mult));
+    CK(launch_ypass(P->d_S1, gq2, nullptr, P->g2, P->mt, P->fp, P->d_tw, S2b, P->d_err + 1, s, pr,
+                    P->sched.y_threads));
   }
   if (events) CK(record_stage(P->ev[4], s));
   return FKP_OK;
@@ -898,12 +915,12 @@ int fkp::enqueue_xy(Plan* P, const unsigned long long* gq, const unsigned long l
 // Enqueues the three FFT passes, recombination and binning of one base grid
 // (of the interlaced pair d_grid, d_grid2 when the plan interlaces).
 int fkp::enqueue_fft_bin(Plan* P, const unsigned long long* gq, const float* gf, cudaStream_t s) {
-  const int rc = enqueue_xy(P, gq, P->d_grid2, gf, s, true);
+  const int rc = enqueue_xy(P, gq, P->d_grid2, gf, s, P->reach, true);
   if (rc) return rc;
   const ZParams zp = zparams(P, 0);
-  CK(launch_zpass(P->d_S2, P->g, P->mt, P->fp, P->d_tw, zp, P->d_zpart, P->d_zpartc, P->d_err + 1, s,
+  CK(launch_zpass(P->d_S2, P->g, P->mt, P->fp, P->d_tw, zp, P->reach, P->d_zpart, P->d_zpartc, P->d_err + 1, s,
                   P->ctx->nsm, P->sched.z_threads));
-  CK(launch_reduce_bins(P->d_zpart, P->d_zpartc, zpass_blocks(P->g.N, P->sched.z_threads, P->ctx->nsm),
+  CK(launch_reduce_bins(P->d_zpart, P->d_zpartc, zpass_blocks(P->reach, P->sched.z_threads, P->ctx->nsm),
                         P->pb.nbins, P->d_bins, P->d_binc, s));
   CK(record_stage(P->ev[5], s));
   return FKP_OK;
@@ -1196,19 +1213,20 @@ extern "C" int fkp_power_batch(void* plan, int nmock, const fkp_catalog_t* gals,
   int* perr = P->b_err + 1;
   MockBatch mx;
   mx.n = nmock; mx.in = (long long)z.grid; mx.out = (long long)z.s1;
-  CK(launch_xpass(P->b_grid, nullptr, P->g, P->mt, P->fp, P->d_tw, P->b_S1, P->ctx->nsm, s, P->sched.x_mult, mx));
+  CK(launch_xpass(P->b_grid, nullptr, P->g, P->mt, P->fp, P->d_tw, P->b_S1, P->ctx->nsm, s, P->reach, P->sched.x_mult,
+                  mx));
   CK(cudaEventRecord(P->ev[3], s));
   MockBatch my;
   my.n = nmock; my.in = (long long)z.s1; my.in2 = (long long)z.grid; my.out = (long long)z.s2;
-  CK(launch_ypass(P->b_S1, P->b_grid, nullptr, P->g, P->mt, P->fp, P->d_tw, P->b_S2, perr, s, P->sched.y_threads,
-                  my));
+  CK(launch_ypass(P->b_S1, P->b_grid, nullptr, P->g, P->mt, P->fp, P->d_tw, P->b_S2, perr, s, P->reach,
+                  P->sched.y_threads, my));
   CK(cudaEventRecord(P->ev[4], s));
   const ZParams zp = zparams(P, 0);
   MockBatch mz;
   mz.n = nmock; mz.in = (long long)z.s2; mz.out = (long long)z.zpart; mz.out2 = (long long)z.zpartc;
-  CK(launch_zpass(P->b_S2, P->g, P->mt, P->fp, P->d_tw, zp, P->b_zpart, P->b_zpartc, perr, s, P->ctx->nsm,
+  CK(launch_zpass(P->b_S2, P->g, P->mt, P->fp, P->d_tw, zp, P->reach, P->b_zpart, P->b_zpartc, perr, s, P->ctx->nsm,
                   P->sched.z_threads, mz));
-  CK(launch_reduce_bins(P->b_zpart, P->b_zpartc, zpass_blocks(P->g.N, P->sched.z_threads, P->ctx->nsm), P->pb.nbins,
+  CK(launch_reduce_bins(P->b_zpart, P->b_zpartc, zpass_blocks(P->reach, P->sched.z_threads, P->ctx->nsm), P->pb.nbins,
                         P->b_bins, P->b_binc, s, nmock, (long long)z.zpart, (long long)z.zpartc));
   CK(cudaEventRecord(P->ev[5], s));
   // bins and scalars back, mock by mock

@@ -43,6 +43,7 @@ struct Plan {
   int lmax = 0;
   MomentTable mt{};
   PassSchedule sched{};
+  PassReach reach, reach_w;  // modes of the F passes (P bins and shells) and of the F^w passes (shells)
   FftPlan fp{};
   GeomDev g{};
   double min_edge_gap = 0;
@@ -145,7 +146,7 @@ int enqueue_fft_bin(Plan* P, const unsigned long long* gq, const float* gf, cuda
 // x- and y-passes of a field into the plan's S2: of the fixed-point grid gq
 // (and, interlaced, of gq2 on the second grid) or of the FP32 field gf.
 int enqueue_xy(Plan* P, const unsigned long long* gq, const unsigned long long* gq2, const float* gf,
-               cudaStream_t s, bool events);
+               cudaStream_t s, const PassReach& pr, bool events);
 ZParams zparams(const Plan* P, int mode);
 int finish_power(Plan* P, cudaStream_t s, fkp_power_out* out, bool have_scalars, double I22, double N0);
 int bisp_plan_init(Plan* P);
@@ -189,18 +190,21 @@ cudaError_t launch_wait_selftest(unsigned polls, int* flag, cudaStream_t s);
 // (N^3 each); the x-pass transforms them instead of forming the moments at
 // the nodes.
 cudaError_t launch_xpass(const unsigned long long* gq, const float* gf, const GeomDev& g, const MomentTable& mt,
-                         const FftPlan& fp, const float2* tw, float2* S1, int nsm, cudaStream_t s, int xm = 2,
-                         MockBatch mb = MockBatch(), bool per_object = false);
+                         const FftPlan& fp, const float2* tw, float2* S1, int nsm, cudaStream_t s,
+                         const PassReach& pr, int xm = 2, MockBatch mb = MockBatch(), bool per_object = false);
 cudaError_t launch_ypass(const float2* S1, const unsigned long long* gq, const float* gf, const GeomDev& g,
                          const MomentTable& mt, const FftPlan& fp,
-                         const float2* tw, float2* S2, int* err, cudaStream_t s, int nt = 256,
-                         MockBatch mb = MockBatch());
-// The z-pass is persistent: zpass_blocks(N, nt, nsm) blocks, each writing
+                         const float2* tw, float2* S2, int* err, cudaStream_t s,
+                         const PassReach& pr, int nt = 256, MockBatch mb = MockBatch());
+// The z-pass is persistent: zpass_blocks(pr, nt, nsm) blocks, each writing
 // one column of the partial bins (part[key][block]); reduce over that count.
 cudaError_t launch_zpass(const float2* S2, const GeomDev& g, const MomentTable& mt, const FftPlan& fp,
-                         const float2* tw, const ZParams& zp, double* part, int* partc, int* err, cudaStream_t s,
-                         int nsm, int nt = 512, MockBatch mb = MockBatch());
-int zpass_blocks(int N, int nt, int nsm);
+                         const float2* tw, const ZParams& zp, const PassReach& pr, double* part, int* partc, int* err,
+                         cudaStream_t s, int nsm, int nt = 512, MockBatch mb = MockBatch());
+int zpass_blocks(const PassReach& pr, int nt, int nsm);
+// The k_x tiles and (k_x tile, k_y) pencils of the modes |n|^2 <= r2, none on
+// a Nyquist plane (at least one of each, so that every launch has blocks).
+std::vector<int> reach_tiles(int N, int r2, PassReach& pr);
 cudaError_t launch_reduce_bins(const double* part, const int* partc, int nblk, int nbins, double* out,
                                long long* outc, cudaStream_t s, int nmock = 1, long long pstride = 0,
                                long long pcstride = 0);

@@ -736,20 +736,21 @@ static int enqueue_bisp(Plan* P, const CatDev& g, const CatDev& r, int contracti
   zp.E = st->d_E;
   zp.mm = mm;
   // F: P bins and export on the shells
-  rc = enqueue_xy(P, P->d_grid, P->d_grid2, nullptr, s, true);
+  rc = enqueue_xy(P, P->d_grid, P->d_grid2, nullptr, s, P->reach, true);
   if (rc) return rc;
-  const int nbz = zpass_blocks(N, P->sched.z_threads, P->ctx->nsm);
-  BCK(launch_zpass(P->d_S2, P->g, P->mt, P->fp, P->d_tw, zp, P->d_zpart, P->d_zpartc, P->d_err + 1, s,
+  const int nbz = zpass_blocks(P->reach, P->sched.z_threads, P->ctx->nsm);
+  const int nbw = zpass_blocks(P->reach_w, P->sched.z_threads, P->ctx->nsm);
+  BCK(launch_zpass(P->d_S2, P->g, P->mt, P->fp, P->d_tw, zp, P->reach, P->d_zpart, P->d_zpartc, P->d_err + 1, s,
                    P->ctx->nsm, P->sched.z_threads));
   BCK(launch_reduce_bins(P->d_zpart, P->d_zpartc, nbz, P->pb.nbins, P->d_bins, P->d_binc, s));
   BCK(record_stage(P->ev[5], s));
   // F^w: shell sums against the exported F_l
-  rc = enqueue_xy(P, P->d_gridw, P->d_gridw2, nullptr, s, false);
+  rc = enqueue_xy(P, P->d_gridw, P->d_gridw2, nullptr, s, P->reach_w, false);
   if (rc) return rc;
   zp.mode = 2;
-  BCK(launch_zpass(P->d_S2, P->g, P->mt, P->fp, P->d_tw, zp, st->d_spart, st->d_spartc, P->d_err + 1, s,
+  BCK(launch_zpass(P->d_S2, P->g, P->mt, P->fp, P->d_tw, zp, P->reach_w, st->d_spart, st->d_spartc, P->d_err + 1, s,
                    P->ctx->nsm, P->sched.z_threads));
-  BCK(launch_reduce_bins(st->d_spart, st->d_spartc, nbz, S, st->d_shell, st->d_shellc, s));
+  BCK(launch_reduce_bins(st->d_spart, st->d_spartc, nbw, S, st->d_shell, st->d_shellc, s));
   BCK(record_stage(P->ev[6], s));
   // shell IFFTs
   const long long N3 = (long long)N * N * N;

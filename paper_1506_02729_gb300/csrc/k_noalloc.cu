@@ -46,7 +46,8 @@ constexpr size_t kOffPartc = kOffPart + align256(sizeof(double) * BQ_N * kNaMaxB
 constexpr size_t kOffBins = kOffPartc + align256(sizeof(int) * kNaMaxBins * kNaBlkZ);
 constexpr size_t kOffBinc = kOffBins + align256(sizeof(double) * BQ_N * kNaMaxBins);
 constexpr size_t kOffErr = kOffBinc + align256(sizeof(long long) * kNaMaxBins);
-constexpr size_t kNaBytes = kOffErr + 256;  // about 42 MB
+constexpr size_t kOffTiles = kOffErr + 256;
+constexpr size_t kNaBytes = kOffTiles + align256(sizeof(int) * kNaBlkZ);  // about 42 MB
 
 }  // namespace
 
@@ -167,6 +168,11 @@ extern "C" int fkp_power_from_grid_noalloc(const fkp_geometry_t* geom, const fkp
     while (b < pb->nbins && b >= -1 && k >= pb->kmin + pb->dk * (b + 1)) ++b;
     if (b >= 0 && b < pb->nbins) lut[n2] = (short)b;
   }
+  int r2 = 0;
+  for (int n2 = 1; n2 <= n2max; ++n2)
+    if (lut[n2] >= 0) r2 = n2;
+  PassReach pr;
+  const std::vector<int> zt = reach_tiles(N, r2, pr);
   std::vector<float2> tw(N);
   for (int m = 0; m < N; ++m) {
     const double a = 2.0 * M_PI * (double)m / (double)N;
@@ -191,6 +197,9 @@ extern "C" int fkp_power_from_grid_noalloc(const fkp_geometry_t* geom, const fkp
   double* d_bins = reinterpret_cast<double*>(base + kOffBins);
   long long* d_binc = reinterpret_cast<long long*>(base + kOffBinc);
   int* d_err = reinterpret_cast<int*>(base + kOffErr);
+  int* d_tiles = reinterpret_cast<int*>(base + kOffTiles);
+  pr.ztiles = d_tiles;
+  NCK(cudaMemcpyAsync(d_tiles, zt.data(), sizeof(int) * zt.size(), cudaMemcpyHostToDevice, s));
   NCK(cudaMemcpyAsync(d_tw, tw.data(), sizeof(float2) * N, cudaMemcpyHostToDevice, s));
   NCK(cudaMemcpyAsync(d_lut, lut.data(), sizeof(short) * (n2max + 1), cudaMemcpyHostToDevice, s));
   NCK(cudaMemcpyAsync(d_winv, winv.data(), sizeof(float) * 3 * N, cudaMemcpyHostToDevice, s));
@@ -198,8 +207,8 @@ extern "C" int fkp_power_from_grid_noalloc(const fkp_geometry_t* geom, const fkp
 
   int dsm = 1;
   NCK(cudaDeviceGetAttribute(&dsm, cudaDevAttrMultiProcessorCount, dev));
-  NCK(launch_xpass(nullptr, F, g, mt, fp, d_tw, S1, dsm, s));
-  NCK(launch_ypass(S1, nullptr, F, g, mt, fp, d_tw, S2, d_err + 1, s));
+  NCK(launch_xpass(nullptr, F, g, mt, fp, d_tw, S1, dsm, s, pr));
+  NCK(launch_ypass(S1, nullptr, F, g, mt, fp, d_tw, S2, d_err + 1, s, pr));
   ZParams zp;
   zp.nbins = pb->nbins;
   zp.lmax = 4;
@@ -213,8 +222,8 @@ extern "C" int fkp_power_from_grid_noalloc(const fkp_geometry_t* geom, const fkp
   zp.E = nullptr;
   zp.mm = 0;
   zp.split68 = 1;
-  NCK(launch_zpass(S2, g, mt, fp, d_tw, zp, d_part, d_partc, d_err + 1, s, dsm, z_threads_for(N)));
-  NCK(launch_reduce_bins(d_part, d_partc, zpass_blocks(N, z_threads_for(N), dsm), pb->nbins, d_bins, d_binc, s));
+  NCK(launch_zpass(S2, g, mt, fp, d_tw, zp, pr, d_part, d_partc, d_err + 1, s, dsm, z_threads_for(N)));
+  NCK(launch_reduce_bins(d_part, d_partc, zpass_blocks(pr, z_threads_for(N), dsm), pb->nbins, d_bins, d_binc, s));
 
   const int nb = pb->nbins;
   std::vector<double> hb(BQ_N * nb);

@@ -33,7 +33,7 @@ template <int N_, int LMAX, bool PO = false>
 __global__ void __launch_bounds__(32 * ((nfields_of(LMAX) + 1) / 2), LMAX < 4 ? 1 : (N_ > 0 && N_ <= 256 ? 4 : 3))
     k_xpass2(
     const unsigned long long* __restrict__ gq, const float* __restrict__ gf, GeomDev g, FftPlan fp,
-    const float2* __restrict__ twg, float2* __restrict__ S1, MockBatch mb) {
+    const float2* __restrict__ twg, float2* __restrict__ S1, int nxt, MockBatch mb) {
   if (gq) gq += (long long)blockIdx.z * mb.in;
   if (gf) gf += (long long)blockIdx.z * mb.in;
   S1 += (long long)blockIdx.z * mb.out;
@@ -112,11 +112,11 @@ __global__ void __launch_bounds__(32 * ((nfields_of(LMAX) + 1) / 2), LMAX < 4 ? 
     }
     __syncthreads();
     const float2* R = fft_any<N_, NP, NTX, -1, SWZ>(A, B, fp, tw);
-    // unpack: consecutive threads take consecutive k_x of one field, so the
-    // stores into the tile-major layout are 64-byte contiguous runs
-    const int ncol = NXT * kT;
-    for (int t = tid; t < NP * ncol; t += NTX) {
-      const int p = t / ncol, k = t - p * ncol;
+    // unpack: warp p takes pencil p (the block has NP warps), consecutive lanes
+    // consecutive k_x, so the stores into the tile-major layout are 64-byte
+    // contiguous runs; only the k_x tiles that hold a wanted mode are stored
+    const int ncol = nxt * kT, p = tid >> 5;
+    for (int k = tid & 31; k < ncol; k += 32) {
       float2 o0 = make_float2(0.f, 0.f), o1 = o0;
       if (k < NH) {
         const float2 zk = R[ilv<NP, SWZ>(k, p)];
@@ -162,7 +162,7 @@ static size_t xsm(int N, int NP) { return sizeof(float2) * (N + N / 2 + 2 * (siz
 
 template <int N_, int LMAX, bool PO = false>
 static cudaError_t xrun(const unsigned long long* gq, const float* gf, const GeomDev& g, const FftPlan& fp,
-                        const float2* tw, float2* S1, int nsm, cudaStream_t s, int xm, const MockBatch& mb) {
+                        const float2* tw, float2* S1, int nsm, cudaStream_t s, int nxt, int xm, const MockBatch& mb) {
   constexpr int NP = (nfields_of(LMAX) + 1) / 2;
   const size_t sm = xsm(g.N, NP);
   raise_smem_limit((const void*)k_xpass2<N_, LMAX, PO>, sm);
@@ -170,37 +170,37 @@ static cudaError_t xrun(const unsigned long long* gq, const float* gf, const Geo
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_xpass2<N_, LMAX, PO>, 32 * NP, sm);
   int grid = nsm * (occ > 0 ? occ : 1) * (xm > 0 ? xm : 2);
   if (grid > g.N * g.N) grid = g.N * g.N;
-  k_xpass2<N_, LMAX, PO><<<dim3(grid, 1, mb.n), dim3(NP, 32), sm, s>>>(gq, gf, g, fp, tw, S1, mb);
+  k_xpass2<N_, LMAX, PO><<<dim3(grid, 1, mb.n), dim3(NP, 32), sm, s>>>(gq, gf, g, fp, tw, S1, nxt, mb);
   return cudaGetLastError();
 }
 
 template <int LMAX>
 static cudaError_t xdispatch(const unsigned long long* gq, const float* gf, const GeomDev& g, const FftPlan& fp,
-                             const float2* tw, float2* S1, int nsm, cudaStream_t s, int xm, const MockBatch& mb,
+                             const float2* tw, float2* S1, int nsm, cudaStream_t s, int nxt, int xm, const MockBatch& mb,
                              bool po) {
   // the per-object variant: the runtime-size kernel, whatever N
-  if (po) return xrun<0, LMAX, true>(gq, gf, g, fp, tw, S1, nsm, s, xm, mb);
+  if (po) return xrun<0, LMAX, true>(gq, gf, g, fp, tw, S1, nsm, s, nxt, xm, mb);
   if (LMAX == 4) {
     switch (g.N) {
-      case 512: return xrun<512, LMAX>(gq, gf, g, fp, tw, S1, nsm, s, xm, mb);
-      case 384: return xrun<384, LMAX>(gq, gf, g, fp, tw, S1, nsm, s, xm, mb);
-      case 360: return xrun<360, LMAX>(gq, gf, g, fp, tw, S1, nsm, s, xm, mb);
-      case 256: return xrun<256, LMAX>(gq, gf, g, fp, tw, S1, nsm, s, xm, mb);
-      case 128: return xrun<128, LMAX>(gq, gf, g, fp, tw, S1, nsm, s, xm, mb);
-      case 64: return xrun<64, LMAX>(gq, gf, g, fp, tw, S1, nsm, s, xm, mb);
+      case 512: return xrun<512, LMAX>(gq, gf, g, fp, tw, S1, nsm, s, nxt, xm, mb);
+      case 384: return xrun<384, LMAX>(gq, gf, g, fp, tw, S1, nsm, s, nxt, xm, mb);
+      case 360: return xrun<360, LMAX>(gq, gf, g, fp, tw, S1, nsm, s, nxt, xm, mb);
+      case 256: return xrun<256, LMAX>(gq, gf, g, fp, tw, S1, nsm, s, nxt, xm, mb);
+      case 128: return xrun<128, LMAX>(gq, gf, g, fp, tw, S1, nsm, s, nxt, xm, mb);
+      case 64: return xrun<64, LMAX>(gq, gf, g, fp, tw, S1, nsm, s, nxt, xm, mb);
       default: break;
     }
   }
-  return xrun<0, LMAX>(gq, gf, g, fp, tw, S1, nsm, s, xm, mb);
+  return xrun<0, LMAX>(gq, gf, g, fp, tw, S1, nsm, s, nxt, xm, mb);
 }
 
 cudaError_t launch_xpass(const unsigned long long* gq, const float* gf, const GeomDev& g, const MomentTable& mt,
-                         const FftPlan& fp, const float2* tw, float2* S1, int nsm, cudaStream_t s, int xm,
-                         MockBatch mb, bool per_object) {
+                         const FftPlan& fp, const float2* tw, float2* S1, int nsm, cudaStream_t s,
+                         const PassReach& pr, int xm, MockBatch mb, bool per_object) {
   if (per_object && (!gq || gf || mb.n != 1)) return cudaErrorInvalidValue;
-  if (mt.nfields == nfields_of(4)) return xdispatch<4>(gq, gf, g, fp, tw, S1, nsm, s, xm, mb, per_object);
-  if (mt.nfields == nfields_of(2)) return xdispatch<2>(gq, gf, g, fp, tw, S1, nsm, s, xm, mb, per_object);
-  return xdispatch<0>(gq, gf, g, fp, tw, S1, nsm, s, xm, mb, per_object);
+  if (mt.nfields == nfields_of(4)) return xdispatch<4>(gq, gf, g, fp, tw, S1, nsm, s, pr.nxt, xm, mb, per_object);
+  if (mt.nfields == nfields_of(2)) return xdispatch<2>(gq, gf, g, fp, tw, S1, nsm, s, pr.nxt, xm, mb, per_object);
+  return xdispatch<0>(gq, gf, g, fp, tw, S1, nsm, s, pr.nxt, xm, mb, per_object);
 }
 
 }  // namespace fkp

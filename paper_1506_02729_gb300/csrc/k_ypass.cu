@@ -19,7 +19,7 @@ __global__ void __launch_bounds__(NT, PassShape<NT>::kMinBlocks) k_ypass2(const 
                                                    const unsigned long long* __restrict__ gq,
                                                    const float* __restrict__ gf, GeomDev g, MomentTable mt,
                                                    FftPlan fp, const float2* __restrict__ twg,
-                                                   float2* __restrict__ S2, int* __restrict__ err, MockBatch mb) {
+                                                   float2* __restrict__ S2, int* __restrict__ err, int r2, MockBatch mb) {
   S1 += (long long)blockIdx.z * mb.in;
   if (gq) gq += (long long)blockIdx.z * mb.in2;
   if (gf) gf += (long long)blockIdx.z * mb.in2;
@@ -70,6 +70,7 @@ __global__ void __launch_bounds__(NT, PassShape<NT>::kMinBlocks) k_ypass2(const 
   const int c = threadIdx.x, run = threadIdx.y;
   const int rl = (N + PassShape<NT>::kRun - 1) / PassShape<NT>::kRun;
   const int kx = xt * kT + c;
+  const int ry2 = r2 - xt * kT * xt * kT;
   int it = 0;
   for (int sw = 0; sw < mt.nsweeps; ++sw) {
     const int nout = mt.s_nout[sw];
@@ -148,7 +149,9 @@ __global__ void __launch_bounds__(NT, PassShape<NT>::kMinBlocks) k_ypass2(const 
 #pragma unroll
       for (int i = 0; i < PassShape<NT>::kRL; ++i) {
         const int ky = i * PassShape<NT>::kRun + run;
-        if (i < rl && ky < N) dst[(size_t)ky * tile] = o ? acc1[i] : acc0[i];
+        // the pencils the z-pass reads: those whose first column meets the disc
+        const int ny = smode(ky, N);
+        if (i < rl && ky < N && ny * ny <= ry2) dst[(size_t)ky * tile] = o ? acc1[i] : acc0[i];
       }
     }
   }
@@ -161,36 +164,36 @@ __global__ void __launch_bounds__(NT, PassShape<NT>::kMinBlocks) k_ypass2(const 
 template <int N_, int NT>
 static cudaError_t yrun_nt(const float2* S1, const unsigned long long* gq, const float* gf, const GeomDev& g,
                            const MomentTable& mt, const FftPlan& fp, const float2* tw, float2* S2, int* err,
-                           cudaStream_t s, const MockBatch& mb) {
+                           cudaStream_t s, const PassReach& pr, const MockBatch& mb) {
   int total = 0;
   for (int q = 0; q < mt.nsweeps; ++q) total += mt.s_nmem[q];
   const size_t sm = ysm(g.N) + sizeof(float) * 10 * kT * (size_t)total;
   raise_smem_limit((const void*)k_ypass2<N_, NT>, sm);
-  k_ypass2<N_, NT><<<dim3(tiles_x(g.N), g.N, mb.n), dim3(kT, NT / kT), sm, s>>>(S1, gq, gf, g, mt, fp, tw, S2, err,
-                                                                                    mb);
+  k_ypass2<N_, NT><<<dim3(pr.nxt, g.N, mb.n), dim3(kT, NT / kT), sm, s>>>(S1, gq, gf, g, mt, fp, tw, S2, err, pr.r2,
+                                                                              mb);
   return cudaGetLastError();
 }
 
 template <int N_>
 static cudaError_t yrun(const float2* S1, const unsigned long long* gq, const float* gf, const GeomDev& g,
                         const MomentTable& mt, const FftPlan& fp, const float2* tw, float2* S2, int* err,
-                        cudaStream_t s, int nt, const MockBatch& mb) {
-  return nt == 512 ? yrun_nt<N_, 512>(S1, gq, gf, g, mt, fp, tw, S2, err, s, mb)
-                   : yrun_nt<N_, 256>(S1, gq, gf, g, mt, fp, tw, S2, err, s, mb);
+                        cudaStream_t s, const PassReach& pr, int nt, const MockBatch& mb) {
+  return nt == 512 ? yrun_nt<N_, 512>(S1, gq, gf, g, mt, fp, tw, S2, err, s, pr, mb)
+                   : yrun_nt<N_, 256>(S1, gq, gf, g, mt, fp, tw, S2, err, s, pr, mb);
 }
 
 // gq / gf: the grid the x-pass read (for the observer node's value).
 cudaError_t launch_ypass(const float2* S1, const unsigned long long* gq, const float* gf, const GeomDev& g,
                          const MomentTable& mt, const FftPlan& fp, const float2* tw, float2* S2, int* err,
-                         cudaStream_t s, int nt, MockBatch mb) {
+                         cudaStream_t s, const PassReach& pr, int nt, MockBatch mb) {
   switch (g.N) {
-    case 512: return yrun<512>(S1, gq, gf, g, mt, fp, tw, S2, err, s, nt, mb);
-    case 384: return yrun<384>(S1, gq, gf, g, mt, fp, tw, S2, err, s, nt, mb);
-    case 360: return yrun<360>(S1, gq, gf, g, mt, fp, tw, S2, err, s, nt, mb);
-    case 256: return yrun<256>(S1, gq, gf, g, mt, fp, tw, S2, err, s, nt, mb);
-    case 128: return yrun<128>(S1, gq, gf, g, mt, fp, tw, S2, err, s, nt, mb);
-    case 64: return yrun<64>(S1, gq, gf, g, mt, fp, tw, S2, err, s, nt, mb);
-    default: return yrun<0>(S1, gq, gf, g, mt, fp, tw, S2, err, s, nt, mb);
+    case 512: return yrun<512>(S1, gq, gf, g, mt, fp, tw, S2, err, s, pr, nt, mb);
+    case 384: return yrun<384>(S1, gq, gf, g, mt, fp, tw, S2, err, s, pr, nt, mb);
+    case 360: return yrun<360>(S1, gq, gf, g, mt, fp, tw, S2, err, s, pr, nt, mb);
+    case 256: return yrun<256>(S1, gq, gf, g, mt, fp, tw, S2, err, s, pr, nt, mb);
+    case 128: return yrun<128>(S1, gq, gf, g, mt, fp, tw, S2, err, s, pr, nt, mb);
+    case 64: return yrun<64>(S1, gq, gf, g, mt, fp, tw, S2, err, s, pr, nt, mb);
+    default: return yrun<0>(S1, gq, gf, g, mt, fp, tw, S2, err, s, pr, nt, mb);
   }
 }
 

@@ -1,6 +1,9 @@
 // k_zpass.cu - the z-pass of the power-spectrum path: FFT along z, Legendre
 // recombination (eqs. F2, delta4), window compensation and shell binning (eq. shell)
 // (shared helpers and layouts in k_fftpass.cuh).
+#include <algorithm>
+#include <vector>
+
 #include "k_fftpass.cuh"
 
 namespace fkp {
@@ -46,7 +49,7 @@ __device__ __forceinline__ void zgroup(const float2* R, int z0, int rl, int N, i
 // order, so the bins are bit-reproducible for a given launch shape.
 template <int N_, int MODE, int NT>
 __global__ void __launch_bounds__(NT, PassShape<NT>::kMinBlocks) k_zpass2(const float2* __restrict__ S2, GeomDev g, MomentTable mt,
-                                                   FftPlan fp, const float2* __restrict__ twg, ZParams zp,
+                                                   FftPlan fp, const float2* __restrict__ twg, ZParams zp, PassReach pr,
                                                    double* __restrict__ part, int* __restrict__ partc,
                                                    int* __restrict__ err, MockBatch mb) {
   S2 += (long long)blockIdx.z * mb.in;
@@ -73,7 +76,7 @@ __global__ void __launch_bounds__(NT, PassShape<NT>::kMinBlocks) k_zpass2(const 
   int* sc = reinterpret_cast<int*>(sbi + BQ_N * nkey);
   unsigned* tmax = reinterpret_cast<unsigned*>(sc + nkey);  // the tile's bound on |value| (FP32 bits)
   const int tid = threadIdx.y * kT + threadIdx.x;
-  const int ntiles = NXT * N;
+  const int ntiles = pr.nzt;
   const size_t gsz = (size_t)N * NXT * N * kT;
   const uint32_t bytes = (uint32_t)(tile * sizeof(float2));
   for (int i = tid; i < N; i += NT) {
@@ -100,13 +103,14 @@ __global__ void __launch_bounds__(NT, PassShape<NT>::kMinBlocks) k_zpass2(const 
     mbar_fence_init();
   }
   __syncthreads();
-  // tile t = (xt, ky) = (t % NXT, t / NXT); group gi of tile t
-  auto src_of = [&](int t, int gi) {
-    return S2 + (size_t)gi * gsz + ((size_t)(t % NXT) * N + t / NXT) * tile;
+  // group gi of tile id = 64 k_y + k_x tile
+  auto src_of = [&](int id, int gi) {
+    return S2 + (size_t)gi * gsz + ((size_t)(id & 63) * N + (id >> 6)) * tile;
   };
+  int id = (int)blockIdx.x < ntiles ? __ldg(pr.ztiles + blockIdx.x) : 0;
   if (tid == 0 && (int)blockIdx.x < ntiles) {
     mbar_expect_tx(&bar[0], bytes);
-    tma_load_1d(buf0, src_of(blockIdx.x, 0), bytes, &bar[0]);
+    tma_load_1d(buf0, src_of(id, 0), bytes, &bar[0]);
   }
   const int c = threadIdx.x, run = threadIdx.y;
   const int rl = (N + PassShape<NT>::kRun - 1) / PassShape<NT>::kRun;
@@ -116,7 +120,12 @@ __global__ void __launch_bounds__(NT, PassShape<NT>::kMinBlocks) k_zpass2(const 
   // it & 1, phase (it >> 1) & 1)
   int it = 0;
   for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-  const int xt = t % NXT, ky = t / NXT;
+  const int xt = id & 63, ky = id >> 6;
+  const int idn = t + (int)gridDim.x < ntiles ? __ldg(pr.ztiles + t + gridDim.x) : -1;
+  // whether the thread's run of k_z meets the ball of wanted modes
+  const int zn = min(z0, max(N - z0 - rl + 1, 0));  // the run's least |n_z|
+  const int rt2 = pr.r2 - xt * kT * xt * kT - smode(ky, N) * smode(ky, N);
+  const bool act = zn * zn <= rt2;
   float2 f0[PassShape<NT>::kRL], s2[PassShape<NT>::kRL], s4[PassShape<NT>::kRL];
 #pragma unroll
   for (int i = 0; i < PassShape<NT>::kRL; ++i) {
@@ -128,9 +137,9 @@ __global__ void __launch_bounds__(NT, PassShape<NT>::kMinBlocks) k_zpass2(const 
     const int cur = it & 1;
     float2* bc = cur ? buf1 : buf0;
     if (tid == 0) {
-      const int tn = gi + 1 < ngt ? t : t + (int)gridDim.x;
+      const int tn = gi + 1 < ngt ? id : idn;
       const int gn = gi + 1 < ngt ? gi + 1 : 0;
-      if (tn < ntiles) {
+      if (tn >= 0) {
         fence_proxy_async();
         mbar_expect_tx(&bar[cur ^ 1], bytes);
         tma_load_1d(cur ? buf0 : buf1, src_of(tn, gn), bytes, &bar[cur ^ 1]);
@@ -142,11 +151,12 @@ __global__ void __launch_bounds__(NT, PassShape<NT>::kMinBlocks) k_zpass2(const 
     // second grid of an interlaced pair: its half-cell phase
     // e^{-i pi (n_x + n_y + n_z)/N}, the n_x, n_y part fixed per thread
     const float2 phxy = gi < mt.ngroups ? make_float2(1.f, 0.f)
-                                        : cmul(zph[(t % NXT) * kT + c < N ? (t % NXT) * kT + c : 0], zph[t / NXT]);
+                                        : cmul(zph[xt * kT + c < N ? xt * kT + c : 0], zph[ky]);
     const int p2 = mt.g_p2[gg], p4 = mt.g_p4[gg];
     const float c2 = mt.g_c2[gg], c4 = mt.g_c4[gg];
     constexpr int RLc = PassShape<NT>::kRL;
-    if (gi < mt.ngroups) {
+    if (!act) {
+    } else if (gi < mt.ngroups) {
       if (mt.g_f0[gg]) zgroup<N_, RLc, true, true, false, false>(R, z0, rl, N, c, c2, p2, c4, p4, f0, s2, s4, zph, phxy);
       else if (c2 != 0.f && c4 != 0.f) zgroup<N_, RLc, false, true, true, false>(R, z0, rl, N, c, c2, p2, c4, p4, f0, s2, s4, zph, phxy);
       else if (c2 != 0.f) zgroup<N_, RLc, false, true, false, false>(R, z0, rl, N, c, c2, p2, c4, p4, f0, s2, s4, zph, phxy);
@@ -174,7 +184,7 @@ __global__ void __launch_bounds__(NT, PassShape<NT>::kMinBlocks) k_zpass2(const 
 #pragma unroll
   for (int i = 0; i < PassShape<NT>::kRL; ++i) {
     const int kz = z0 + i;
-    if (colok && rowok && i < rl && kz < N && kz != N / 2) {
+    if (act && colok && rowok && i < rl && kz < N && kz != N / 2) {
       const int nzv = smode(kz, N);
       const int n2 = kx * kx + nyv * nyv + nzv * nzv;
       if (n2 > 0) {
@@ -226,7 +236,7 @@ __global__ void __launch_bounds__(NT, PassShape<NT>::kMinBlocks) k_zpass2(const 
     float vals[BQ_N];
 #pragma unroll
     for (int q = 0; q < BQ_N; ++q) vals[q] = 0.f;
-    if (colok && rowok && i < rl && kz < N && kz != N / 2) {
+    if (act && colok && rowok && i < rl && kz < N && kz != N / 2) {
       const int nzv = smode(kz, N);
       const int n2 = kx * kx + nyv * nyv + nzv * nzv;
       const int sh = (MODE != 0 && n2 < zp.nsh2) ? (int)zp.slut[n2] : -1;
@@ -313,6 +323,7 @@ __global__ void __launch_bounds__(NT, PassShape<NT>::kMinBlocks) k_zpass2(const 
     sbh[q] = 0;
   }
   if (tid == 0) *tmax = 0u;
+  id = idn;
   __syncthreads();
   }
   const int blk = blockIdx.x, nblk = gridDim.x;
@@ -328,60 +339,75 @@ static size_t zsm(int N, int nkey) {
   return ysm(N) + sizeof(float2) * N + (sizeof(double) + sizeof(long long)) * BQ_N * nkey + sizeof(int) * nkey + 16;
 }
 
+std::vector<int> reach_tiles(int N, int r2, PassReach& pr) {
+  std::vector<int> t;
+  pr.r2 = std::max(r2, 1);
+  pr.nxt = 1;
+  for (int ky = 0; ky < N; ++ky) {
+    const int ny = ky <= N / 2 ? ky : ky - N;
+    if (ky == N / 2) continue;
+    for (int xt = 0; xt * kT < N / 2 && xt * kT * xt * kT + ny * ny <= pr.r2; ++xt) {
+      t.push_back(ky * 64 + xt);
+      pr.nxt = std::max(pr.nxt, xt + 1);
+    }
+  }
+  pr.nzt = (int)t.size();
+  return t;
+}
+
 // Persistent z-pass grid: one block per resident slot (two 256-thread or one
 // 512-thread block per SM), at most one per tile.
-int zpass_blocks(int N, int nt, int nsm) {
-  const int ntiles = tiles_x(N) * N;
+int zpass_blocks(const PassReach& pr, int nt, int nsm) {
   const int nb = nsm * (nt == 256 ? 2 : 1);
-  return nb < ntiles ? nb : ntiles;
+  return nb < pr.nzt ? nb : pr.nzt;
 }
 
 template <int N_, int MODE, int NT>
 static cudaError_t zrun_nt(const float2* S2, const GeomDev& g, const MomentTable& mt, const FftPlan& fp,
-                           const float2* tw, const ZParams& zp, double* part, int* partc, int* err, cudaStream_t s,
+                           const float2* tw, const ZParams& zp, const PassReach& pr, double* part, int* partc, int* err, cudaStream_t s,
                            int nsm, const MockBatch& mb) {
   const size_t sm = zsm(g.N, MODE == 2 ? zp.nshells : zp.nbins);
   raise_smem_limit((const void*)k_zpass2<N_, MODE, NT>, sm);
-  k_zpass2<N_, MODE, NT><<<dim3(zpass_blocks(g.N, NT, nsm), 1, mb.n), dim3(kT, NT / kT), sm, s>>>(
-      S2, g, mt, fp, tw, zp, part, partc, err, mb);
+  k_zpass2<N_, MODE, NT><<<dim3(zpass_blocks(pr, NT, nsm), 1, mb.n), dim3(kT, NT / kT), sm, s>>>(
+      S2, g, mt, fp, tw, zp, pr, part, partc, err, mb);
   return cudaGetLastError();
 }
 
 template <int N_, int MODE>
 static cudaError_t zrun(const float2* S2, const GeomDev& g, const MomentTable& mt, const FftPlan& fp,
-                        const float2* tw, const ZParams& zp, double* part, int* partc, int* err, cudaStream_t s,
+                        const float2* tw, const ZParams& zp, const PassReach& pr, double* part, int* partc, int* err, cudaStream_t s,
                         int nsm, int nt, const MockBatch& mb) {
-  return nt == 256 ? zrun_nt<N_, MODE, 256>(S2, g, mt, fp, tw, zp, part, partc, err, s, nsm, mb)
-                   : zrun_nt<N_, MODE, 512>(S2, g, mt, fp, tw, zp, part, partc, err, s, nsm, mb);
+  return nt == 256 ? zrun_nt<N_, MODE, 256>(S2, g, mt, fp, tw, zp, pr, part, partc, err, s, nsm, mb)
+                   : zrun_nt<N_, MODE, 512>(S2, g, mt, fp, tw, zp, pr, part, partc, err, s, nsm, mb);
 }
 
 template <int MODE>
 static cudaError_t zdispatch(const float2* S2, const GeomDev& g, const MomentTable& mt, const FftPlan& fp,
-                             const float2* tw, const ZParams& zp, double* part, int* partc, int* err,
+                             const float2* tw, const ZParams& zp, const PassReach& pr, double* part, int* partc, int* err,
                              cudaStream_t s, int nsm, int nt, const MockBatch& mb) {
   switch (g.N) {
-    case 512: return zrun<512, MODE>(S2, g, mt, fp, tw, zp, part, partc, err, s, nsm, nt, mb);
-    case 360: return zrun<360, MODE>(S2, g, mt, fp, tw, zp, part, partc, err, s, nsm, nt, mb);
-    case 256: return zrun<256, MODE>(S2, g, mt, fp, tw, zp, part, partc, err, s, nsm, nt, mb);
+    case 512: return zrun<512, MODE>(S2, g, mt, fp, tw, zp, pr, part, partc, err, s, nsm, nt, mb);
+    case 360: return zrun<360, MODE>(S2, g, mt, fp, tw, zp, pr, part, partc, err, s, nsm, nt, mb);
+    case 256: return zrun<256, MODE>(S2, g, mt, fp, tw, zp, pr, part, partc, err, s, nsm, nt, mb);
     default: break;
   }
   if (MODE == 0) {
     switch (g.N) {
-      case 384: return zrun<384, MODE>(S2, g, mt, fp, tw, zp, part, partc, err, s, nsm, nt, mb);
-      case 128: return zrun<128, MODE>(S2, g, mt, fp, tw, zp, part, partc, err, s, nsm, nt, mb);
-      case 64: return zrun<64, MODE>(S2, g, mt, fp, tw, zp, part, partc, err, s, nsm, nt, mb);
+      case 384: return zrun<384, MODE>(S2, g, mt, fp, tw, zp, pr, part, partc, err, s, nsm, nt, mb);
+      case 128: return zrun<128, MODE>(S2, g, mt, fp, tw, zp, pr, part, partc, err, s, nsm, nt, mb);
+      case 64: return zrun<64, MODE>(S2, g, mt, fp, tw, zp, pr, part, partc, err, s, nsm, nt, mb);
       default: break;
     }
   }
-  return zrun<0, MODE>(S2, g, mt, fp, tw, zp, part, partc, err, s, nsm, nt, mb);
+  return zrun<0, MODE>(S2, g, mt, fp, tw, zp, pr, part, partc, err, s, nsm, nt, mb);
 }
 
 cudaError_t launch_zpass(const float2* S2, const GeomDev& g, const MomentTable& mt, const FftPlan& fp,
-                         const float2* tw, const ZParams& zp, double* part, int* partc, int* err, cudaStream_t s,
+                         const float2* tw, const ZParams& zp, const PassReach& pr, double* part, int* partc, int* err, cudaStream_t s,
                          int nsm, int nt, MockBatch mb) {
-  if (zp.mode == 0) return zdispatch<0>(S2, g, mt, fp, tw, zp, part, partc, err, s, nsm, nt, mb);
-  if (zp.mode == 1) return zdispatch<1>(S2, g, mt, fp, tw, zp, part, partc, err, s, nsm, nt, mb);
-  return zdispatch<2>(S2, g, mt, fp, tw, zp, part, partc, err, s, nsm, nt, mb);
+  if (zp.mode == 0) return zdispatch<0>(S2, g, mt, fp, tw, zp, pr, part, partc, err, s, nsm, nt, mb);
+  if (zp.mode == 1) return zdispatch<1>(S2, g, mt, fp, tw, zp, pr, part, partc, err, s, nsm, nt, mb);
+  return zdispatch<2>(S2, g, mt, fp, tw, zp, pr, part, partc, err, s, nsm, nt, mb);
 }
 
 }  // namespace fkp
