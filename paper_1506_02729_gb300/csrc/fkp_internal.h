@@ -209,13 +209,30 @@ cudaError_t launch_reduce_bins(const double* part, const int* partc, int nblk, i
                                long long* outc, cudaStream_t s, int nmock = 1, long long pstride = 0,
                                long long pcstride = 0);
 
-// tensor-core triangle contraction (k_contract_tc.cu)
-void tc_slicing(long long N3, int ntiles, int nsm, int* nslices, int* chunks);
-int tc_tile_cols();
+// tensor-core triangle contraction (k_contract_tc.cu): a tile is 128 pairs
+// times a run of n field rows from r0 (its accumulator columns start at col
+// of its block's, at cb of all tiles'); a block takes one group of tiles.
+constexpr int kTcMaxTiles = 11;
+struct TcTile {
+  int n, r0, col, cb, tile;
+};
+struct TcGroup {
+  int T;
+  TcTile t[kTcMaxTiles];
+};
+struct TcPlan {
+  std::vector<short2> pairs;    // field indices of the tiles' pairs, 128 per tile
+  std::vector<TcGroup> groups;
+  std::vector<int> off;         // per output: its place in a slice's partials
+  int ncols = 0;                // columns of 128 partials per slice
+};
+TcPlan tc_plan(int S, int nl, const std::vector<int>& arow, const std::vector<short2>& pair);
+void tc_slicing(long long N3, int ngroups, int nsm, int* nslices, int* chunks);
 int tc_rows();
-cudaError_t launch_contract_tc(const float* I, long long N3, int nf, int S, const short2* pairs, int npairs,
-                               float* part, int* err, int nslices, int chunks, int nsplit, cudaStream_t s);
-cudaError_t launch_tc_reduce(const float* part, int nslices, int ntiles, const int* om, const int* on, int nout,
-                             double* out, cudaStream_t s);
+cudaError_t launch_contract_tc(const float* I, long long N3, int S, int nl, const TcGroup* groups, int ngroups,
+                               const short2* pairs, int ncols, float* part, int* err, int nslices, int chunks,
+                               int nsplit, cudaStream_t s);
+cudaError_t launch_tc_reduce(const float* part, int nslices, int ncols, const int* off, int nout, double* out,
+                             cudaStream_t s);
 
 }  // namespace fkp

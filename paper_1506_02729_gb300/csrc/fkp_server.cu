@@ -86,7 +86,7 @@ size_t estimate_plan(const fkp_request_t& r) {
     const size_t mm = (size_t)hmax, w2 = 2 * mm + 1, m1 = mm + 1;
     b += 3 * w2 * w2 * m1 * 8 + (size_t)S * N * w2 * m1 * 8 + (size_t)S * N * N * m1 * 8 + (size_t)nl * S * N3 * 4;
     const size_t slices = (N3 + 65535) / 65536, pairs = (size_t)S * (S + 1) / 2;
-    b += slices * ((pairs + 255) / 256) * 128 * 256 * 4 + slices * 16384 * 8;
+    b += slices * ((pairs + 127) / 128) * 128 * 144 * 4 + slices * 16384 * 8;
   }
   return b + b / 10 + (64 << 20);
 }

@@ -66,10 +66,11 @@ struct BispState {
   int* d_spartc = nullptr;
   double* d_shell = nullptr;
   long long* d_shellc = nullptr;
-  // tensor-core contraction: columns = pairs (b >= c), outputs -> (row, column)
-  int npairs = 0, tc_slices = 0, tc_tiles = 0, tc_chunks = 0;
+  // tensor-core contraction: tiles of pairs (b >= c), groups of tiles, outputs -> partials
+  int tc_groups = 0, tc_ncols = 0, tc_slices = 0, tc_chunks = 0;
   short2* d_pairs = nullptr;
-  int *d_om = nullptr, *d_on = nullptr;
+  TcGroup* d_groups = nullptr;
+  int* d_off = nullptr;
   float* d_tcpart = nullptr;
   // shell IFFT work lists: z tiles (s, n_y + mm, n_x0), y tiles (s, n_x0, |n_y| range); floor(r_s)
   int nzjobs = 0, nyjobs = 0;
@@ -595,36 +596,25 @@ int bisp_plan_init(Plan* P) {
         }
       }
   }
-  // pair columns of the tensor-core contraction (field indices of the two
-  // factors) and each output's (row, column)
-  std::map<long long, int> pidx;
-  std::vector<short2> pairs;
-  auto column = [&](int fb, int fc) {
-    const long long key = (long long)fb * 4 * S + fc;
-    auto f = pidx.find(key);
-    if (f != pidx.end()) return f->second;
-    pidx[key] = (int)pairs.size();
-    pairs.push_back(make_short2((short)fb, (short)fc));
-    return (int)pairs.size() - 1;
-  };
-  for (int t = 0; t < ntri; ++t) column(st->tb[t], st->tc[t]);
-  if (st->zero_area)
-    for (int t = 0; t < ntri; ++t) column(S + st->tb[t], st->tc[t]);
-  st->npairs = (int)pairs.size();
-  std::vector<int> om(std::max(1, ntri) * nq, -1), on(std::max(1, ntri) * nq, 0);
-  for (int t = 0; t < ntri; ++t) {
-    for (int li = 0; li < st->nl; ++li) {
-      om[t * nq + li] = li * S + st->ta[t];
-      on[t * nq + li] = column(st->tb[t], st->tc[t]);
+  // tensor-core contraction: output (triangle t, quantity q) is a field row and
+  // a pair of factors (field indices); quantities that are not computed have none
+  std::vector<int> arow, orow;
+  std::vector<short2> opair;
+  const bool tc_ok = st->nl * S <= tc_rows();
+  for (int t = 0; t < ntri && tc_ok; ++t)
+    for (int q : qs) {
+      arow.push_back((q == 3 ? S : q * S) + st->ta[t]);
+      opair.push_back(make_short2((short)((q == 3 ? S : 0) + st->tb[t]), (short)st->tc[t]));
+      orow.push_back(t * nq + q);
     }
-    if (st->zero_area) {
-      om[t * nq + 3] = S + st->ta[t];
-      on[t * nq + 3] = column(S + st->tb[t], st->tc[t]);
-    }
-  }
+  TcPlan tcp;
+  if (!arow.empty()) tcp = tc_plan(S, st->nl, arow, opair);
+  std::vector<int> off(std::max(1, ntri) * nq, -1);
+  for (size_t o = 0; o < orow.size(); ++o) off[orow[o]] = tcp.off[o];
+  st->tc_groups = (int)tcp.groups.size();
+  st->tc_ncols = tcp.ncols;
   const long long N3 = (long long)N * N * N;
-  st->tc_tiles = (st->npairs + tc_tile_cols() - 1) / tc_tile_cols();
-  tc_slicing(N3, std::max(1, st->tc_tiles), P->ctx->nsm, &st->tc_slices, &st->tc_chunks);
+  tc_slicing(N3, std::max(1, st->tc_groups), P->ctx->nsm, &st->tc_slices, &st->tc_chunks);
   const int iblocks = std::max<int>(1, ((int)st->items.size() + 255) / 256);
   st->nslices = std::max(1, (P->ctx->nsm * 8) / iblocks);
   st->slice_len = ((N3 + st->nslices - 1) / st->nslices + kCTK - 1) / kCTK * kCTK;
@@ -678,12 +668,11 @@ int bisp_plan_init(Plan* P) {
   st->d_spartc = (int*)A(sizeof(int) * S * (size_t)P->nblk_z);
   st->d_shell = (double*)A(sizeof(double) * BQ_N * S);
   st->d_shellc = (long long*)A(sizeof(long long) * S);
-  const bool tc_ok = st->nl * S <= tc_rows();
-  if (tc_ok && st->npairs > 0) {
-    st->d_pairs = (short2*)A(sizeof(short2) * st->npairs);
-    st->d_om = (int*)A(sizeof(int) * om.size());
-    st->d_on = (int*)A(sizeof(int) * on.size());
-    st->d_tcpart = (float*)A(sizeof(float) * (size_t)st->tc_slices * st->tc_tiles * tc_rows() * tc_tile_cols());
+  if (st->tc_groups > 0) {
+    st->d_pairs = (short2*)A(sizeof(short2) * tcp.pairs.size());
+    st->d_groups = (TcGroup*)A(sizeof(TcGroup) * tcp.groups.size());
+    st->d_off = (int*)A(sizeof(int) * off.size());
+    st->d_tcpart = (float*)A(sizeof(float) * (size_t)st->tc_slices * st->tc_ncols * 128);
   }
   if (!ok) return set_error(FKP_ENOMEM, "device allocation failed for the bispectrum workspace (%.2f GB in plan)",
                             P->bytes_total / 1e9);
@@ -697,9 +686,9 @@ int bisp_plan_init(Plan* P) {
     BCK(cudaMemcpy(st->d_items, st->items.data(), sizeof(ContractItem) * st->items.size(), cudaMemcpyHostToDevice));
   BCK(cudaMemset(st->d_cpart, 0, sizeof(double) * (size_t)st->nslices * std::max(1, ntri) * st->nq));
   if (st->d_pairs) {
-    BCK(cudaMemcpy(st->d_pairs, pairs.data(), sizeof(short2) * pairs.size(), cudaMemcpyHostToDevice));
-    BCK(cudaMemcpy(st->d_om, om.data(), sizeof(int) * om.size(), cudaMemcpyHostToDevice));
-    BCK(cudaMemcpy(st->d_on, on.data(), sizeof(int) * on.size(), cudaMemcpyHostToDevice));
+    BCK(cudaMemcpy(st->d_pairs, tcp.pairs.data(), sizeof(short2) * tcp.pairs.size(), cudaMemcpyHostToDevice));
+    BCK(cudaMemcpy(st->d_groups, tcp.groups.data(), sizeof(TcGroup) * tcp.groups.size(), cudaMemcpyHostToDevice));
+    BCK(cudaMemcpy(st->d_off, off.data(), sizeof(int) * off.size(), cudaMemcpyHostToDevice));
   }
   return FKP_OK;
 }
@@ -776,10 +765,11 @@ static int enqueue_bisp(Plan* P, const CatDev& g, const CatDev& r, int contracti
   BCK(record_stage(P->ev[7], s));
   // contraction
   const int ntri = P->ntri, nout = std::max(1, ntri) * st->nq;
-  if (tensor && st->npairs > 0) {
-    BCK(launch_contract_tc(st->d_I, N3, st->nl * S, S, st->d_pairs, st->npairs, st->d_tcpart, P->d_err + 1,
-                           st->tc_slices, st->tc_chunks, contraction == FKP_CONTRACT_BF16X3 ? 2 : 3, s));
-    BCK(launch_tc_reduce(st->d_tcpart, st->tc_slices, st->tc_tiles, st->d_om, st->d_on, nout, st->d_T, s));
+  if (tensor && st->d_pairs) {
+    BCK(launch_contract_tc(st->d_I, N3, S, st->nl, st->d_groups, st->tc_groups, st->d_pairs, st->tc_ncols,
+                           st->d_tcpart, P->d_err + 1, st->tc_slices, st->tc_chunks,
+                           contraction == FKP_CONTRACT_BF16X3 ? 2 : 3, s));
+    BCK(launch_tc_reduce(st->d_tcpart, st->tc_slices, st->tc_ncols, st->d_off, nout, st->d_T, s));
   } else if (!st->items.empty()) {
     const int nf = st->nl * S;
     const size_t smc = sizeof(float) * (size_t)kCTK * (nf | 1);
@@ -834,7 +824,7 @@ extern "C" int fkp_bispectrum(void* plan, const fkp_catalog_t* gal, const fkp_ca
     return set_error(FKP_EINVAL, "unknown contraction mode %d", contraction);
   auto* st = static_cast<BispState*>(P->bisp);
   const bool tensor = contraction == FKP_CONTRACT_BF16X3 || contraction == FKP_CONTRACT_BF16X6;
-  if (tensor && !st->d_pairs && st->npairs > 0)
+  if (tensor && !st->d_pairs && P->ntri > 0)
     return set_error(FKP_EINVAL, "the tensor-core contraction needs (multipoles x shells) <= %d rows", tc_rows());
   BCK(cudaSetDevice(P->ctx->device));
   cudaStream_t s = static_cast<cudaStream_t>(stream);

@@ -3,8 +3,8 @@
 //
 //   T^(l)(a,b,c) = sum_x F_a^(l)(x) F_b^(0)(x) F_c^(0)(x)
 //
-// is the skinny GEMM D[(l,a), (b,c)] = sum_x A[(l,a), x] B[(b,c), x] with
-// A = the shell fields and B = the Khatri-Rao products F_b^(0) F_c^(0).  Each
+// is the skinny GEMM D[(b,c), (l,a)] = sum_x A[(b,c), x] B[(l,a), x] with
+// A = the Khatri-Rao products F_b^(0) F_c^(0) and B = the shell fields.  Each
 // FP32 operand v is split into BF16 v_hi = bf16(v), v_lo = bf16(v - v_hi); the
 // three products hi*hi + hi*lo + lo*hi are accumulated in FP32 in tensor
 // memory (the lo*lo term and the rounding of lo, each ~2^-18 relative, are
@@ -15,29 +15,51 @@
 // the triangle sums cancel strongly (sum |t| >> |sum t|), so the 3-way split
 // is the accurate mode and the 2-way split the fast one.
 //
-// One CTA of 16 warps per (256-column N tile, K slice).  The slices (up to
-// about 4,096 chunks of 32 points) are sized at plan time so that tiles x
-// slices CTAs fill whole waves of the SMs.
-// The shell fields of a chunk of 32 points are fetched two chunks ahead with
-// cp.async into a 3-slot ring; operand stages are double buffered: all
-// threads form the products and the BF16 splits into K-major tiles with the
-// 64-byte swizzle (one 64-byte row of K per operand row); one thread issues
-// the tcgen05.mma instructions (M = 128, N = 256, K = 16) and commits them to
-// the stage's mbarrier.  After every run of 96 accumulating MMAs (16 chunks,
-// 8 for the 3-way split) the 128 x 256 FP32 tile is read from tensor memory
-// (tcgen05.ld; each warp its lane quarter and 64 columns), added with
-// round-to-nearest to a running FP32 sum held in the other 256 tensor-memory
-// columns (tcgen05.ld, add, tcgen05.st) and the MMA accumulation restarts.
-// In-tensor-core accumulation runs were measured to drift linearly with their
-// length (5.6e-4 of the monopole scale over 65,536 points, under 1e-4 over
-// 1,024).  With 1,024-point runs that rounding, not the operand split, set
-// the 3-way split's error (B_4 8.4e-5 of the FP32 contraction on a 64^3
-// case, above the 2-way split's 5.1e-5); with runs of 96 MMAs it is 6.7e-6.
-// The drain of a run waits until the next chunk's operands are built, so the
-// tensor pipe idles only for the drain.  At the end of the slice the sums go
+// What bounds it, and the layout that follows from that.  The MMA work is
+// small (a tile of 128 pairs needs only the fields a that close a triangle
+// with one of them: the field rows are ordered a-major, so a tile's fields
+// are one run of rows and one descriptor, 320 columns in all for 37 shells
+// and three multipoles, where a (l,a) x (b,c) tiling issues 768); the cost is
+// shared memory: building the products and feeding the operands.  So
+//   - the pair products never touch shared memory: a thread owns a pair (a
+//     tensor-memory lane), forms 32 points of its product in registers, splits
+//     them and stores the BF16 parts to tensor memory (tcgen05.st), from where
+//     the MMA reads its A operand;
+//   - only the field operand B is staged in shared memory (its K-major parts,
+//     21 KB per chunk of 32 points at 111 fields), built once per chunk for
+//     all tiles of the block;
+//   - the chunk's FP32 fields arrive as one TMA box (32 points x all fields,
+//     128-byte swizzle: eight lanes reading one 16-byte column of eight
+//     consecutive fields hit distinct banks).
+// 24 warps, each with one role, meet on mbarriers: three warpgroups build A,
+// each for a third of the tiles and into its own tensor-memory stage, with a
+// warp each that issues those tiles' MMAs (one warp for all tiles sets the
+// pace with its waits and commits: 29.1 ms at 360^3); one warpgroup builds B,
+// one drains the accumulators, one warp issues the TMA loads.
+// Tensor memory (512 columns): 176 accumulator columns, 176 columns of the
+// running sums of the drained accumulators, 144 of A stages; tiles are
+// packed into groups of at most 176 columns, one block per (group, K slice).
+//
+// Accumulation in tensor memory rounds (its error grows with the run length),
+// so a tile's accumulator is drained - added with round to nearest to the
+// running FP32 sum in tensor memory - after every run of tc_run(tiles) chunks
+// (36 accumulating MMAs for three tiles and the 3-way split).  The tiles of a
+// block drain at different chunks, so the tensor pipe seldom waits.  At the end of the slice the sums go
 // to per-slice partials, summed over slices in FP64 by k_tc_reduce.
+//
+// Measured (3-way split, GB300): 37 shells x 3 multipoles on 360^3 48.3 ms with
+// the products built into shared memory for (l,a) x (b,c) tiles of 128 x 256,
+// 21.0 ms here (16.1 ms with the MMAs left out, 18.5 without the B build); 27
+// shells x 1 on 512^3 83.7 -> 26.5 ms.  A chunk takes about 1,900 cycles of
+// which a warpgroup computes 900: what is left is the handoffs (waits of 80 to
+// 170 cycles each) between the roles.  The triangle sums are closer to the FP64
+// ones than with runs of 96 MMAs (T_l 1.1e-6 to 1.8e-6 -> 0.5e-6 to 1.3e-6 over
+// grids of 64^3 to 512^3, every split).
 #include <algorithm>
+#include <numeric>
+#include <vector>
 
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -46,36 +68,101 @@
 
 namespace fkp {
 
-constexpr int kTcM = 128;              // MMA rows (l, a)
-constexpr int kTcN = 256;              // MMA columns (pairs b >= c) per tile
+constexpr int kTcM = 128;              // MMA rows: pairs (b, c) per tile
+constexpr int kTcRows = 128;           // fields (l, a) at most
+constexpr int kTcCols = 176;           // accumulator columns of a group of tiles
 constexpr int kTcKC = 32;              // K points per chunk
-constexpr int kTcSliceTarget = 4096;   // chunks per K slice, at most (about)
-constexpr int kTcThreads = 512;
-constexpr int kTcABytes = kTcM * kTcKC * 2;    // one BF16 operand tile: 8 KB
-constexpr int kTcBBytes = kTcN * kTcKC * 2;    // 16 KB
-template <int NS>
-__host__ __device__ constexpr int tc_stage_bytes() { return NS * (kTcABytes + kTcBBytes); }
-constexpr int kTcRow = kTcKC + 4;      // staged row stride (floats): 16-byte aligned, shifts banks by 4 per field
+constexpr int kTcSliceTarget = 2048;   // chunks per K slice, at most (about)
+constexpr int kTcRing = 4;             // chunks of fields in flight
+constexpr int kTcAWg = 3;              // warpgroups that build A, and warps that issue MMAs
+constexpr int kTcThreads = (kTcAWg + 2) * 128 + (kTcAWg + 1) * 32;
+constexpr int kTcPartRow = kTcRows + 16;           // rows of a B part (a tile's last rows may be padding)
+constexpr int kTcPartBytes = kTcPartRow * kTcKC * 2;  // one BF16 part of B: 9 KB
 
-// chunks per tensor-memory accumulation run: 96 accumulating MMAs per run for
-// every split (3 products x 2 K steps x 16 chunks; 6 x 2 x 8)
-template <int NS>
-__host__ __device__ constexpr int tc_drain() { return NS == 3 ? 8 : 16; }
-// K slicing: the fewest whole waves of the SMs (tiles x slices CTAs, one per
+// Chunks per accumulation run of a block with T tiles: a multiple of T when
+// T <= 4, so that at most one tile drains per chunk, and 8 at most.
+__host__ __device__ constexpr int tc_run(int T) { return T <= 2 ? 4 : (T <= 8 ? T : 8); }
+
+// K slicing: the fewest whole waves of the SMs (groups x slices CTAs, one per
 // SM at a time) whose slices hold at most about kTcSliceTarget chunks; slices
 // of equal length (the last one shorter), none empty.
-void tc_slicing(long long N3, int ntiles, int nsm, int* nslices, int* chunks) {
+void tc_slicing(long long N3, int ngroups, int nsm, int* nslices, int* chunks) {
   const long long total = (N3 + kTcKC - 1) / kTcKC;
   const long long per_wave = (long long)nsm * kTcSliceTarget;
-  const long long waves = std::max<long long>(1, (total * ntiles + per_wave - 1) / per_wave);
-  long long ns = std::max<long long>(1, waves * nsm / std::max(1, ntiles));
+  const long long waves = std::max<long long>(1, (total * ngroups + per_wave - 1) / per_wave);
+  long long ns = std::max<long long>(1, waves * nsm / std::max(1, ngroups));
   ns = std::min(ns, std::max<long long>(1, total));
   const long long ch = (total + ns - 1) / ns;
   *chunks = (int)ch;
   *nslices = (int)((total + ch - 1) / ch);
 }
-int tc_tile_cols() { return kTcN; }
-int tc_rows() { return kTcM; }
+int tc_rows() { return kTcRows; }
+
+// The tiles of a set of outputs.  Output o is the sum of field arow[o] = l S +
+// a times the pair (fb, fc)[o].  Pairs are sorted by their first shell (the
+// shells a that close with a pair begin there), cut into tiles of 128, and
+// the tiles packed into groups of at most kTcCols accumulator columns.
+TcPlan tc_plan(int S, int nl, const std::vector<int>& arow, const std::vector<short2>& pair) {
+  TcPlan P;
+  const int no = (int)arow.size();
+  std::vector<int> ord(no);
+  std::iota(ord.begin(), ord.end(), 0);
+  auto key = [&](int o) { return ((pair[o].x % S) * 4 + pair[o].x / S) * S + pair[o].y; };
+  std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) { return key(a) < key(b); });
+  std::vector<int> idx(no, 0);
+  std::vector<short2> list;
+  for (int q = 0; q < no; ++q) {
+    if (q == 0 || key(ord[q]) != key(ord[q - 1])) list.push_back(pair[ord[q]]);
+    idx[ord[q]] = (int)list.size() - 1;
+  }
+  const int nt = ((int)list.size() + kTcM - 1) / kTcM;
+  // each tile's run of field rows r = a nl + l, from a multiple of 8 (the
+  // swizzle's period), a multiple of 16 columns
+  auto row_of = [&](int o) { return (arow[o] % S) * nl + arow[o] / S; };
+  std::vector<int> lo(nt, 1 << 20), hi(nt, -1);
+  for (int o = 0; o < no; ++o) {
+    const int t = idx[o] / kTcM, r = row_of(o);
+    lo[t] = std::min(lo[t], r);
+    hi[t] = std::max(hi[t], r);
+  }
+  std::vector<TcTile> tiles(nt);
+  int cb = 0;
+  for (int t = 0; t < nt; ++t) {
+    tiles[t].r0 = lo[t] / 8 * 8;
+    tiles[t].n = (hi[t] - tiles[t].r0) / 16 * 16 + 16;
+    tiles[t].cb = cb;
+    tiles[t].tile = t;
+    cb += tiles[t].n;
+  }
+  P.ncols = cb;
+  // first fit, widest first, each tile into the emptiest group that holds it
+  std::vector<int> by(nt);
+  std::iota(by.begin(), by.end(), 0);
+  std::stable_sort(by.begin(), by.end(), [&](int a, int b) { return tiles[a].n > tiles[b].n; });
+  int total = 0;
+  for (auto& t : tiles) total += t.n;
+  std::vector<int> used;
+  for (int g = 0; g < std::max(1, (total + kTcCols - 1) / kTcCols); ++g) { P.groups.push_back(TcGroup{}); used.push_back(0); }
+  for (int t : by) {
+    int best = -1;
+    for (int g = 0; g < (int)used.size(); ++g)
+      if (used[g] + tiles[t].n <= kTcCols && (best < 0 || used[g] < used[best])) best = g;
+    if (best < 0) { best = (int)used.size(); P.groups.push_back(TcGroup{}); used.push_back(0); }
+    TcGroup& G = P.groups[best];
+    tiles[t].col = used[best];
+    used[best] += tiles[t].n;
+    G.t[G.T++] = tiles[t];
+  }
+  P.groups.erase(std::remove_if(P.groups.begin(), P.groups.end(), [](const TcGroup& g) { return g.T == 0; }), P.groups.end());
+  list.resize((size_t)nt * kTcM, make_short2(0, 0));  // padding lanes: any field (their rows of D are not read)
+  P.pairs = list;
+  P.off.resize(no);
+  for (int o = 0; o < no; ++o) {
+    const TcTile& t = tiles[idx[o] / kTcM];
+    P.off[o] = (t.cb + row_of(o) - t.r0) * kTcM + idx[o] % kTcM;
+  }
+  return P;
+}
 
 // ---------------------------------------------------------------------------
 // tcgen05 / TMEM wrappers
@@ -94,69 +181,41 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// D[tmem] (+)= A * B^T, A and B K-major BF16 in shared memory, FP32 accumulate.
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                          uint32_t accumulate) {
+// D[tmem] (+)= A * B^T, A (BF16, 2 values per 32-bit column, lane = row) in
+// tensor memory, B K-major BF16 in shared memory, FP32 accumulate.
+__device__ __forceinline__ void umma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
+                                             uint32_t accumulate, uint32_t elected) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      "{\n .reg .pred p, e;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 e, %5, 0;\n"
+      " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(elected)
       : "memory");
 }
 
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-               : "memory");
+// 1 in one lane of the (converged) warp, 0 in the others.
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t e;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(e));
+  return e;
 }
 
-// 32 consecutive FP32 columns of this warp's 32 TMEM lanes.
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
-  uint32_t r[32];
+__device__ __forceinline__ void umma_commit(uint64_t* bar, uint32_t elected) {
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      "{\n .reg .pred e;\n setp.ne.b32 e, %1, 0;\n"
+      " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(smem_u32(bar)),
+      "r"(elected)
+      : "memory");
+}
+
+// 16 consecutive 32-bit columns of this warp's 32 tensor-memory lanes: load
+// without the wait, the wait that completes every load in flight (naming the
+// registers, so that no use of them moves ahead of it), and store.
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, "
+      "[%16];"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr)
-      : "memory");
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-// 32 consecutive FP32 columns of this warp's 32 TMEM lanes, stored.
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const float* v) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-      "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
-      ::"r"(taddr), "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])),
-        "r"(__float_as_uint(v[3])), "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])),
-        "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7])), "r"(__float_as_uint(v[8])),
-        "r"(__float_as_uint(v[9])), "r"(__float_as_uint(v[10])), "r"(__float_as_uint(v[11])),
-        "r"(__float_as_uint(v[12])), "r"(__float_as_uint(v[13])), "r"(__float_as_uint(v[14])),
-        "r"(__float_as_uint(v[15])), "r"(__float_as_uint(v[16])), "r"(__float_as_uint(v[17])),
-        "r"(__float_as_uint(v[18])), "r"(__float_as_uint(v[19])), "r"(__float_as_uint(v[20])),
-        "r"(__float_as_uint(v[21])), "r"(__float_as_uint(v[22])), "r"(__float_as_uint(v[23])),
-        "r"(__float_as_uint(v[24])), "r"(__float_as_uint(v[25])), "r"(__float_as_uint(v[26])),
-        "r"(__float_as_uint(v[27])), "r"(__float_as_uint(v[28])), "r"(__float_as_uint(v[29])),
-        "r"(__float_as_uint(v[30])), "r"(__float_as_uint(v[31]))
-      : "memory");
-  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-}
-
-// tcgen05.ld of 32 columns without the wait, and the wait that completes
-// every load in flight; the wait names the destination registers as in-out
-// operands so that no use of them is moved ahead of it.
-__device__ __forceinline__ void tmem_ld32_async(uint32_t taddr, uint32_t* r) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr)
       : "memory");
 }
@@ -164,38 +223,50 @@ __device__ __forceinline__ void tmem_wait_ld(uint32_t* r) {
   asm volatile("tcgen05.wait::ld.sync.aligned;"
                : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
                  "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]),
-                 "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]),
-                 "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]),
-                 "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
+                 "+r"(r[15])
                :
                : "memory");
 }
-// tcgen05.st of 32 columns without the wait (tcgen05.wait::st completes it)
-__device__ __forceinline__ void tmem_st32_async(uint32_t taddr, const uint32_t* v) {
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* v) {
   asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-      "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
-      ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
-        "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]), "r"(v[16]),
-        "r"(v[17]), "r"(v[18]), "r"(v[19]), "r"(v[20]), "r"(v[21]), "r"(v[22]), "r"(v[23]), "r"(v[24]),
-        "r"(v[25]), "r"(v[26]), "r"(v[27]), "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31])
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+      "%15, %16};" ::"r"(taddr),
+      "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]),
+      "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15])
+      : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
+// Box of a 2-D tensor map to shared memory, completing on bar.
+__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
+          smem_u32(dst)),
+      "l"(map), "r"(x), "r"(y), "r"(smem_u32(bar))
       : "memory");
 }
 
 // Shared-memory matrix descriptor: K-major operand with the 64-byte swizzle.
 // Each row holds the chunk's 32 K values (64 bytes); 8 rows form a 512-byte
-// swizzle atom (sbo = 512 between atoms); the K steps of 16 advance the start
+// swizzle atom (512 between atoms); the K steps of 16 advance the start
 // address by 32 bytes within the rows.  Descriptor version 1, layout type
 // SWIZZLE_64B (4) in bits 61-63.
-__device__ __forceinline__ uint64_t sdesc(const void* p, uint32_t lbo, uint32_t sbo) {
-  const uint64_t a = (uint64_t)((smem_u32(p) & 0x3FFFF) >> 4);
-  return a | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)(sbo >> 4) << 32) | (1ull << 46) | (4ull << 61);
+// The address field counts 16-byte units in the low 14 bits (shared memory is
+// far smaller than their reach), so an offset is added to the low word.
+constexpr uint32_t kDescLo = 1u << 16, kDescHi = (512u >> 4) | (1u << 14) | (4u << 29);
+__device__ __forceinline__ uint64_t sdesc(uint32_t lo) {
+  uint64_t d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "r"(kDescHi));
+  return d;
 }
 
-// Instruction descriptor for kind::f16: D FP32, A and B BF16, both K-major,
-// N = 256, M = 128.
-__host__ __device__ constexpr uint32_t tc_idesc() {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTcN >> 3) << 17) | ((uint32_t)(kTcM >> 4) << 24);
+// Instruction descriptor for kind::f16: D FP32, A and B BF16, both K-major, M = 128.
+__device__ __forceinline__ uint32_t tc_idesc(int n) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kTcM >> 4) << 24);
 }
 
 // Byte offset of the 16-byte segment (row, k-group kg) of an operand tile in
@@ -207,270 +278,387 @@ __device__ __forceinline__ int canon_off(int row, int kg) {
   return row * 64 + ((kg ^ ((row >> 1) & 3)) << 4);
 }
 
-// BF16 split of 8 values into NS parts (each part the BF16 rounding of the
-// remainder), packed 16 bytes per part.
+// Packed FP32 pairs.
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+  unsigned long long r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(*reinterpret_cast<unsigned long long*>(&a)), "l"(*reinterpret_cast<unsigned long long*>(&b)));
+  return *reinterpret_cast<float2*>(&r);
+}
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
+  unsigned long long r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(*reinterpret_cast<unsigned long long*>(&a)), "l"(*reinterpret_cast<unsigned long long*>(&b)));
+  return *reinterpret_cast<float2*>(&r);
+}
+
+// BF16 split of two values into NS parts (each part the BF16 rounding of the
+// remainder): w[p] packs part p of both.
 template <int NS>
-__device__ __forceinline__ void split8(const float* v, uint4* out) {
-  uint32_t w[NS][4];
+__device__ __forceinline__ void split2(float2 r, uint32_t* w) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    float2 r = make_float2(v[2 * i], v[2 * i + 1]);
-#pragma unroll
-    for (int p = 0; p < NS; ++p) {
-      const __nv_bfloat162 h = __floats2bfloat162_rn(r.x, r.y);  // one paired conversion
-      w[p][i] = *reinterpret_cast<const uint32_t*>(&h);
-      if (p + 1 < NS) {
-        const float2 hf = __bfloat1622float2(h);
-        r.x -= hf.x;
-        r.y -= hf.y;
-      }
-    }
+  for (int p = 0; p < NS; ++p) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(r.x, r.y);
+    w[p] = *reinterpret_cast<const uint32_t*>(&h);
+    if (p + 1 < NS) r = sub2(r, make_float2(__uint_as_float(w[p] << 16), __uint_as_float(w[p] & 0xffff0000u)));
   }
-#pragma unroll
-  for (int p = 0; p < NS; ++p) out[p] = make_uint4(w[p][0], w[p][1], w[p][2], w[p][3]);
 }
 
 // ---------------------------------------------------------------------------
 
-// pairs: (b, c) of the tile's columns (b < 0 marks padding); part layout
-// [slice][tile][128][256] FP32.
-//
-// Every thread has a fixed share of each chunk: A row t % 128, k-group t / 128
-// (8 points); B row t % 256, k-groups 2 (t / 256) and 2 (t / 256) + 1 (16
-// points); its field copies are f = i / 8, points 4 (i % 8) of i = t, t + 512.
-// Offsets and pair indices are therefore computed once.  Rows of A beyond nf
-// and padding columns of B are zeroed once in both stages and never
-// rewritten.  The running FP32 sum of the drained tiles sits in tensor memory
-// columns 256-511 (each drain: tcgen05.ld tile and sum, add, tcgen05.st), so
-// no accumulator occupies registers through the chunk loop.
+struct TcShared {
+  uint64_t ring_full[kTcRing], ring_empty[kTcRing];
+  uint64_t a_full[kTcAWg], a_empty[kTcAWg];
+  uint64_t b_full[2], b_empty[2];
+  uint64_t acc_full[kTcMaxTiles], acc_empty[kTcMaxTiles];
+  uint64_t done[kTcAWg];
+  uint32_t tmem;
+  uint32_t packed[kTcMaxTiles];
+  int abort;
+  TcGroup g;
+};
+
+// A bounded wait by a warp (all lanes leave it together, with one answer);
+// once one gives up (the error word is set) every other wait of the block
+// gives up too.  A poll suspends the warp for up to kTcPollNs, so that waiting
+// warps do not crowd the shared-memory pipe.
+constexpr unsigned kTcPolls = 1u << 18, kTcPollNs = 20000;
+__device__ __forceinline__ bool tc_wait(uint64_t* bar, uint32_t parity, volatile int* abort, int* err) {
+  for (unsigned it = 0; it < kTcPolls; ++it) {
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity), "r"(kTcPollNs)
+        : "memory");
+    if (__all_sync(0xffffffffu, ok)) return true;
+    if ((it & 15) == 15 && __any_sync(0xffffffffu, *abort)) return false;
+  }
+  *abort = 1;
+  if ((threadIdx.x & 31) == 0) atomicOr(err, 16);
+  return false;
+}
+
 template <int NS>
-__global__ void __launch_bounds__(kTcThreads, 1) k_contract_tc(const float* __restrict__ I, long long N3, int nf,
-                                                               int S, const short2* __restrict__ pairs, int npairs,
-                                                               int chunks, float* __restrict__ part,
+__global__ void __launch_bounds__(kTcThreads, 1) k_contract_tc(const __grid_constant__ CUtensorMap map, int nf, int S,
+                                                               int nl, const TcGroup* __restrict__ groups,
+                                                               const short2* __restrict__ pairs, long long nchunks,
+                                                               int chunks, int ncols, float* __restrict__ part,
                                                                int* __restrict__ err) {
-  extern __shared__ __align__(1024) unsigned char smraw[];
-  constexpr int kStage = tc_stage_bytes<NS>();
-  unsigned char* stage0 = smraw;                                  // 2 stages: A parts, then B parts
-  float* Iring = reinterpret_cast<float*>(smraw + 2 * kStage);   // 3 x [nf][kTcRow], prefetched 2 chunks ahead
-  const int ring = nf * kTcRow;                                   // floats per ring slot
-  uint64_t* bar = reinterpret_cast<uint64_t*>(Iring + 3 * ring);  // [2]
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + 2);
-  const int tid = threadIdx.x, warp = tid >> 5;
-  const int tile = blockIdx.x, slice = blockIdx.y, ntiles = gridDim.x;
-  // zero both stages once: rows that are never written stay zero
-  for (int i = tid; i < 2 * kStage / 16; i += kTcThreads) reinterpret_cast<uint4*>(stage0)[i] = make_uint4(0, 0, 0, 0);
+  extern __shared__ unsigned char smdyn[];
+  unsigned char* smraw = smdyn + ((1024u - (smem_u32(smdyn) & 1023u)) & 1023u);  // the swizzles need 1024
+  __shared__ TcShared sh;
+  __shared__ short2 spair[kTcMaxTiles * kTcM];
+  constexpr int kStageCols = NS * (kTcKC / 2);
+  constexpr int kBStage = NS * kTcPartBytes;
+  constexpr uint32_t kSum = kTcCols, kA0 = 2 * kTcCols;
+  static_assert(2 * kTcCols + kTcAWg * kStageCols <= 512, "tensor memory columns");
+  const int slot_bytes = (nf * kTcKC * 4 + 1023) & ~1023;
+  unsigned char* ring = smraw;                            // kTcRing x [nf][32] FP32, 128-byte swizzle
+  unsigned char* bst = smraw + kTcRing * slot_bytes;      // 2 x NS parts of B
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  const long long c0 = (long long)blockIdx.y * chunks;
+  const int nch = (int)(nchunks - c0 < chunks ? nchunks - c0 : chunks);
+  if (tid == 0) {
+    sh.g = groups[blockIdx.x];
+    sh.abort = 0;
+    for (int i = 0; i < groups[blockIdx.x].T; ++i) {
+      const TcTile& t = groups[blockIdx.x].t[i];
+      sh.packed[i] = (uint32_t)(t.col / 16) | (uint32_t)(t.r0 / 8) << 4 | (uint32_t)(t.n / 16) << 9;
+    }
+    for (int i = 0; i < kTcRing; ++i) {
+      mbar_init(&sh.ring_full[i], 1);
+      mbar_init(&sh.ring_empty[i], 4 * groups[blockIdx.x].T + 4);
+    }
+    for (int i = 0; i < kTcAWg; ++i) {
+      mbar_init(&sh.a_full[i], 4);
+      mbar_init(&sh.a_empty[i], 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&sh.b_full[i], 4);
+      mbar_init(&sh.b_empty[i], groups[blockIdx.x].T < kTcAWg ? groups[blockIdx.x].T : kTcAWg);
+    }
+    for (int i = 0; i < kTcMaxTiles; ++i) {
+      mbar_init(&sh.acc_full[i], 1);
+      mbar_init(&sh.acc_empty[i], 4);
+    }
+    for (int i = 0; i < kTcAWg; ++i) mbar_init(&sh.done[i], 1);
+    mbar_fence_init();
+  }
+  // rows of B past the last field stay zero
+  for (int i = tid; i < 2 * kBStage / 16; i += kTcThreads) reinterpret_cast<uint4*>(bst)[i] = make_uint4(0, 0, 0, 0);
   if (warp == 0) {
-    tmem_alloc(tslot, 2 * kTcN);
+    tmem_alloc(&sh.tmem, 512);
     tmem_relinquish();
   }
-  if (tid == 0) {
-    mbar_init(&bar[0], 1);
-    mbar_init(&bar[1], 1);
-    mbar_fence_init();
+  tc_fence_before();
+  fence_proxy_async();
+  __syncthreads();
+  tc_fence_after();
+  const int T = sh.g.T, R = tc_run(T);
+  for (int i = tid; i < T * kTcM; i += kTcThreads) spair[i] = pairs[sh.g.t[i / kTcM].tile * kTcM + i % kTcM];
+  __syncthreads();
+  const uint32_t tm = sh.tmem;
+  volatile int* ab = &sh.abort;
+
+  if (warp < 4 * kTcAWg) {
+    // ---- A: products of the pairs of the tiles t = w mod kTcAWg, in warpgroup
+    // w's own stage of tensor memory, which MMA warp w reads
+    const int row = tid & 127;
+    const uint32_t lane_base = (uint32_t)(warp & 3) << 21;  // (warp % 4) * 32 lanes, in bits 16 and up
+    const int wg = warp >> 2;
+    const uint32_t stage = tm + lane_base + kA0 + wg * kStageCols;
+    int t = wg, q = 0;
+    for (int c = wg < T ? 0 : nch; c < nch; ++q) {
+      const int s = c % kTcRing;
+      const short2 bc = spair[t * kTcM + row];
+      if (!tc_wait(&sh.ring_full[s], (uint32_t)(c / kTcRing) & 1, ab, err)) break;
+      const unsigned char* pb = ring + s * slot_bytes + bc.x * 128;
+      const unsigned char* pc = ring + s * slot_bytes + bc.y * 128;
+      const int xb = bc.x & 7, xc = bc.y & 7;
+      uint32_t w[NS][16];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const float4 u = *reinterpret_cast<const float4*>(pb + ((j ^ xb) << 4));
+        const float4 v = *reinterpret_cast<const float4*>(pc + ((j ^ xc) << 4));
+        uint32_t o[NS];
+        split2<NS>(mul2(make_float2(u.x, u.y), make_float2(v.x, v.y)), o);
+#pragma unroll
+        for (int p = 0; p < NS; ++p) w[p][2 * j] = o[p];
+        split2<NS>(mul2(make_float2(u.z, u.w), make_float2(v.z, v.w)), o);
+#pragma unroll
+        for (int p = 0; p < NS; ++p) w[p][2 * j + 1] = o[p];
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&sh.ring_empty[s]);
+      if (q > 0 && !tc_wait(&sh.a_empty[wg], (uint32_t)(q - 1) & 1, ab, err)) break;
+      tc_fence_after();
+#pragma unroll
+      for (int p = 0; p < NS; ++p) tmem_st16(stage + p * 16, w[p]);
+      tmem_wait_st();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&sh.a_full[wg]);
+      t += kTcAWg;
+      if (t >= T) {
+        t = wg;
+        ++c;
+      }
+    }
+  } else if (warp < 4 * (kTcAWg + 1)) {
+    // ---- B: thread r splits field row r = a nl + l (field l S + a) into its K-major parts
+    const int r = tid & 127;
+    const bool act = r < nf;
+    const int f = act ? (r % nl) * S + r / nl : 0;
+    for (int c = 0; c < nch; ++c) {
+      const int s = c % kTcRing, b = c & 1;
+      if (!tc_wait(&sh.ring_full[s], (uint32_t)(c / kTcRing) & 1, ab, err)) break;
+      if (c >= 2 && !tc_wait(&sh.b_empty[b], (uint32_t)((c >> 1) - 1) & 1, ab, err)) break;
+      if (act) {
+        const unsigned char* pf = ring + s * slot_bytes + f * 128;
+        unsigned char* dst = bst + b * kBStage;
+#pragma unroll
+        for (int kg = 0; kg < 4; ++kg) {
+          const float4 u = *reinterpret_cast<const float4*>(pf + (((2 * kg) ^ (f & 7)) << 4));
+          const float4 v = *reinterpret_cast<const float4*>(pf + (((2 * kg + 1) ^ (f & 7)) << 4));
+          uint32_t w[4][NS];
+          split2<NS>(make_float2(u.x, u.y), w[0]);
+          split2<NS>(make_float2(u.z, u.w), w[1]);
+          split2<NS>(make_float2(v.x, v.y), w[2]);
+          split2<NS>(make_float2(v.z, v.w), w[3]);
+#pragma unroll
+          for (int p = 0; p < NS; ++p)
+            *reinterpret_cast<uint4*>(dst + p * kTcPartBytes + canon_off(r, kg)) =
+                make_uint4(w[0][p], w[1][p], w[2][p], w[3][p]);
+        }
+      }
+      fence_proxy_async();
+      __syncwarp();
+      if (lane == 0) {
+        mbar_arrive(&sh.b_full[b]);
+        mbar_arrive(&sh.ring_empty[s]);
+      }
+    }
+  } else if (warp < 4 * (kTcAWg + 2)) {
+    // ---- drains: accumulator of a finished run added to the tile's running sum
+    const uint32_t base = tm + ((uint32_t)(warp & 3) << 21);
+    uint32_t z[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) z[k] = 0u;
+    for (int col = 0; col < kTcCols; col += 16) tmem_st16(base + kSum + col, z);
+    tmem_wait_st();
+    uint32_t par = 0;  // bit t: parity of tile t's next drain
+    bool ok = true;
+    int cr1 = R > 1 ? 1 : 0;  // (c + 1) mod R
+    for (int c = 0; c < nch && ok; ++c) {
+      for (int t = 0; t < T && ok; ++t) {
+        if (c + 1 < nch && cr1 != (t < R ? t : t - R)) continue;
+        ok = tc_wait(&sh.acc_full[t], (par >> t) & 1, ab, err);
+        if (!ok) break;
+        par ^= 1u << t;
+        tc_fence_after();
+        const uint32_t col = base + sh.g.t[t].col;
+        for (int k = 0; k < sh.g.t[t].n; k += 16) {
+          uint32_t v[16], u[16];
+          tmem_ld16(col + k, v);
+          tmem_ld16(col + kSum + k, u);
+          tmem_wait_ld(v);
+          tmem_wait_ld(u);
+#pragma unroll
+          for (int m = 0; m < 16; ++m) u[m] = __float_as_uint(__uint_as_float(u[m]) + __uint_as_float(v[m]));
+          tmem_st16(col + kSum + k, u);
+        }
+        tmem_wait_st();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sh.acc_empty[t]);
+      }
+      if (++cr1 == R) cr1 = 0;
+    }
+    // the slice's sums: [slice][column][pair]
+    if (ok) {
+      for (int t = 0; t < T; ++t) {
+        float* dst = part + ((size_t)blockIdx.y * ncols + sh.g.t[t].cb) * kTcM + (tid & 127);
+        for (int k = 0; k < sh.g.t[t].n; k += 16) {
+          uint32_t u[16];
+          tmem_ld16(base + kSum + sh.g.t[t].col + k, u);
+          tmem_wait_ld(u);
+#pragma unroll
+          for (int m = 0; m < 16; ++m) dst[(size_t)(k + m) * kTcM] = __uint_as_float(u[m]);
+        }
+      }
+    }
+  } else if (warp < 4 * (kTcAWg + 2) + kTcAWg) {
+    // ---- MMAs: warp m issues those of the tiles t = m mod kTcAWg (a tile's are
+    // in order that way).  The whole warp walks the jobs with warp-uniform
+    // values (the operands are then in uniform registers), one lane issues.
+    const int m = warp - 4 * (kTcAWg + 2);
+    const uint32_t el = elect_one();
+    // products (i, j) of A part i and B part j whose order is at most 2^-16
+    constexpr int NP = NS == 2 ? 3 : 6;
+    constexpr int pi[6] = {0, 0, 1, 0, 2, 1};
+    constexpr int pj[6] = {0, 1, 0, 2, 0, 1};
+    const uint32_t tmu = __shfl_sync(0xffffffffu, tm, 0);
+    uint32_t par = 0;  // bit t: parity of the drain that tile t's next run waits for
+    int q = 0, cr = 0, cr1 = R > 1 ? 1 : 0;  // job, c mod R, (c + 1) mod R
+    const uint32_t bb0 = kDescLo | (smem_u32(bst) >> 4);
+    bool ok = m < T;
+    for (int c = 0; c < nch && ok; ++c) {
+      const int b = c & 1;
+      ok = tc_wait(&sh.b_full[b], (uint32_t)(c >> 1) & 1, ab, err);
+      for (int t = m; t < T && ok; t += kTcAWg, ++q) {
+        const int tr = t < R ? t : t - R;
+        const bool first = c == 0 || cr == tr;
+        // columns / 16, first row / 8 and width / 16 of the tile
+        const uint32_t pk = __shfl_sync(0xffffffffu, sh.packed[t], 0);
+        const uint32_t d = tmu + (pk & 15) * 16, a = tmu + kA0 + m * kStageCols;
+        const uint32_t br = bb0 + b * (kBStage >> 4) + ((pk >> 4) & 31) * 32, id = tc_idesc((pk >> 9) * 16);
+        ok = tc_wait(&sh.a_full[m], (uint32_t)q & 1, ab, err);
+        if (ok && first && c > 0) {
+          ok = tc_wait(&sh.acc_empty[t], (par >> t) & 1, ab, err);
+          par ^= 1u << t;
+        }
+        if (!ok) break;
+        tc_fence_after();
+#pragma unroll
+        for (int ks = 0; ks < kTcKC / 16; ++ks)
+#pragma unroll
+          for (int k = 0; k < NP; ++k)
+            umma_bf16_ts(d, a + pi[k] * 16 + ks * 8, sdesc(br + ((pj[k] * kTcPartBytes + ks * 32) >> 4)), id,
+                         (!first || ks > 0 || k > 0) ? 1u : 0u, el);
+        umma_commit(&sh.a_empty[m], el);
+        if (c + 1 == nch || cr1 == tr) umma_commit(&sh.acc_full[t], el);
+      }
+      if (ok) umma_commit(&sh.b_empty[b], el);
+      cr = cr1;
+      if (++cr1 == R) cr1 = 0;
+    }
+    // every MMA issued has finished before the tensor memory is freed
+    umma_commit(&sh.done[m], el);
+    mbar_wait(&sh.done[m], 0, err, 16);
+    __syncwarp();
+  } else {
+    // ---- TMA: one box of fields per chunk
+    const uint32_t bytes = (uint32_t)nf * kTcKC * 4;
+    int c = 0;
+    for (; c < nch; ++c) {
+      const int s = c % kTcRing;
+      if (c >= kTcRing && !tc_wait(&sh.ring_empty[s], (uint32_t)(c / kTcRing - 1) & 1, ab, err)) break;
+      if (lane == 0) {
+        mbar_expect_tx(&sh.ring_full[s], bytes);
+        tma_load_2d(ring + s * slot_bytes, &map, (int)((c0 + c) * kTcKC), 0, &sh.ring_full[s]);
+      }
+      __syncwarp();
+    }
+    // copies in flight have landed before the block ends
+    for (int k = c > kTcRing ? c - kTcRing : 0; k < c; ++k)
+      mbar_wait(&sh.ring_full[k % kTcRing], (uint32_t)(k / kTcRing) & 1, err, 16);
+    __syncwarp();
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t taddr = *tslot;
-  // this thread's slice of the tile: TMEM lane quarter (warp % 4) and 64 of
-  // the 256 columns (warp / 4); its running sum 256 columns further on
-  const int q4 = warp & 3, h2 = warp >> 2;
-  const uint32_t tcol = taddr + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(h2 * 64);
-  {
-    float z[32];
-#pragma unroll
-    for (int i = 0; i < 32; ++i) z[i] = 0.f;
-    tmem_st32(tcol + kTcN, z);
-    tmem_st32(tcol + kTcN + 32, z);
-  }
-  const long long x0 = (long long)slice * kTcKC * chunks;
-  const long long xend = (x0 + (long long)kTcKC * chunks < N3) ? x0 + (long long)kTcKC * chunks : N3;
-  const int nch = x0 < xend ? (int)((xend - x0 + kTcKC - 1) / kTcKC) : 0;
-  const uint32_t idesc = tc_idesc();
-  // fixed roles
-  const int rowA = tid & (kTcM - 1), kgA = tid / kTcM;
-  const bool actA = rowA < nf;
-  const int srcA = rowA * kTcRow + kgA * 8, dstA = canon_off(rowA, kgA);
-  const int rowB = tid & (kTcN - 1), khB = tid / kTcN;
-  short2 bc = make_short2(-1, -1);
-  if (tile * kTcN + rowB < npairs) bc = pairs[tile * kTcN + rowB];
-  const bool actB = bc.x >= 0;
-  const int srcB1 = (actB ? bc.x : 0) * kTcRow + khB * 16, srcB2 = (actB ? bc.y : 0) * kTcRow + khB * 16;
-  const int dstB0 = canon_off(rowB, 2 * khB), dstB1 = canon_off(rowB, 2 * khB + 1);
-  const int cf0 = tid >> 3, cf1 = (tid + kTcThreads) >> 3, ck4 = (tid & 7) * 4;
-  const bool cp0 = cf0 < nf, cp1 = cf1 < nf;
-  const float* csrc0 = I + (size_t)(cp0 ? cf0 : 0) * N3;
-  const float* csrc1 = I + (size_t)(cp1 ? cf1 : 0) * N3;
-  const uint32_t cdst0 = smem_u32(Iring + cf0 * kTcRow + ck4), cdst1 = smem_u32(Iring + cf1 * kTcRow + ck4);
-  bool ok = true;
-  // asynchronous copies of a chunk's field values into its ring slot (16 bytes
-  // each; points past the slice are zero-filled)
-  auto prefetch = [&](int cc) {
-    if (cc < nch) {
-      const long long x = x0 + (long long)cc * kTcKC + ck4;
-      const int bytes = x + 4 <= xend ? 16 : (x < xend ? (int)(xend - x) * 4 : 0);
-      const long long xs = x < xend ? x : 0;
-      const uint32_t so = (uint32_t)((cc % 3) * ring * 4);
-      if (cp0)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(cdst0 + so), "l"(csrc0 + xs), "r"(bytes)
-                     : "memory");
-      if (cp1)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(cdst1 + so), "l"(csrc1 + xs), "r"(bytes)
-                     : "memory");
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  // drain of the run ending with chunk cl: wait for that chunk's MMAs, add
-  // the tile to the running sum (ok is made block-uniform: tcgen05.ld is a
-  // warp-collective)
-  constexpr int kDrain = tc_drain<NS>();
-  auto drain = [&](int cl) {
-    const bool w = ok && mbar_wait(&bar[cl & 1], (uint32_t)((cl >> 1) & 1), err, 16);
-    ok = __syncthreads_and(w) != 0;
-    tc_fence_after();
-    if (ok) {
-      // per 32 columns: both loads, one wait, add, store; one store wait
-#pragma unroll
-      for (int cg = 0; cg < 2; ++cg) {
-        uint32_t v[32], u[32];
-        tmem_ld32_async(tcol + cg * 32, v);
-        tmem_ld32_async(tcol + kTcN + cg * 32, u);
-        tmem_wait_ld(v);
-        tmem_wait_ld(u);
-#pragma unroll
-        for (int i = 0; i < 32; ++i) u[i] = __float_as_uint(__uint_as_float(u[i]) + __uint_as_float(v[i]));
-        tmem_st32_async(tcol + kTcN + cg * 32, u);
-      }
-      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-    }
-    tc_fence_before();
-    __syncthreads();
-  };
-  prefetch(0);
-  prefetch(1);
-  for (int c = 0; c < nch; ++c) {
-    const int s = c & 1;
-    unsigned char* st = stage0 + s * kStage;
-    unsigned char* Ap = st;                      // NS tiles of kTcABytes
-    unsigned char* Bp = st + NS * kTcABytes;     // NS tiles of kTcBBytes
-    prefetch(c + 2);
-    asm volatile("cp.async.wait_group 2;" ::: "memory");
-    const float* Ist = Iring + (c % 3) * ring;
-    // the MMAs that read this stage two chunks ago must have finished
-    if (c >= 2 && ok) ok = mbar_wait(&bar[s], (uint32_t)(((c - 2) >> 1) & 1), err, 16);
-    ok = __syncthreads_and(ok) != 0;
-    // A: rows (l, a) = field index; a quarter-warp stores 8 consecutive rows
-    // of one k-group (one contiguous, conflict-free 128-byte span)
-    if (actA) {
-      const float4 p = *reinterpret_cast<const float4*>(Ist + srcA);
-      const float4 q = *reinterpret_cast<const float4*>(Ist + srcA + 4);
-      const float v[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
-      uint4 parts[NS];
-      split8<NS>(v, parts);
-#pragma unroll
-      for (int k = 0; k < NS; ++k) *reinterpret_cast<uint4*>(Ap + k * kTcABytes + dstA) = parts[k];
-    }
-    // B: rows = pairs (b, c) of this tile, products of the l = 0 fields
-    if (actB) {
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const float4 b0 = *reinterpret_cast<const float4*>(Ist + srcB1 + 8 * h);
-        const float4 b1 = *reinterpret_cast<const float4*>(Ist + srcB1 + 8 * h + 4);
-        const float4 c0 = *reinterpret_cast<const float4*>(Ist + srcB2 + 8 * h);
-        const float4 c1 = *reinterpret_cast<const float4*>(Ist + srcB2 + 8 * h + 4);
-        const float v[8] = {b0.x * c0.x, b0.y * c0.y, b0.z * c0.z, b0.w * c0.w,
-                            b1.x * c1.x, b1.y * c1.y, b1.z * c1.z, b1.w * c1.w};
-        uint4 parts[NS];
-        split8<NS>(v, parts);
-        const int d = h ? dstB1 : dstB0;
-#pragma unroll
-        for (int k = 0; k < NS; ++k) *reinterpret_cast<uint4*>(Bp + k * kTcBBytes + d) = parts[k];
-      }
-    }
-    fence_proxy_async();
-    __syncthreads();
-    // a run ended with chunk c - 1: its MMAs ran while this chunk was built,
-    // so the tensor pipe waits only for the drain, not for a build
-    if (c > 0 && c % kDrain == 0) drain(c - 1);
-    if (tid == 0 && ok) {
-      tc_fence_after();
-      // products (i, j) of A part i and B part j whose order is at most 2^-16
-      constexpr int NP = NS == 2 ? 3 : 6;
-      constexpr int pi[6] = {0, 0, 1, 0, 2, 1};
-      constexpr int pj[6] = {0, 1, 0, 2, 0, 1};
-#pragma unroll
-      for (int ks = 0; ks < kTcKC / 16; ++ks) {
-        // K step ks covers k-groups 2 ks and 2 ks + 1 (32 bytes further along the rows)
-#pragma unroll
-        for (int q = 0; q < NP; ++q) {
-          const uint64_t ad = sdesc(Ap + pi[q] * kTcABytes + ks * 32, 16, 512);
-          const uint64_t bd = sdesc(Bp + pj[q] * kTcBBytes + ks * 32, 16, 512);
-          umma_bf16(taddr, ad, bd, idesc, ((c % kDrain) > 0 || ks > 0 || q > 0) ? 1u : 0u);
-        }
-      }
-      umma_commit(&bar[s]);
-    }
-    // No barrier here: the next chunk builds the other stage, which the MMAs
-    // of chunk c - 1 have released (mbarrier wait), and reads a ring slot the
-    // copies of chunk c + 1 filled; stage s is rebuilt only after this commit.
-  }
-  if (nch > 0) drain(nch - 1);
-  asm volatile("cp.async.wait_group 0;" ::: "memory");
-  // the last drain waited for every MMA of the slice
-  float* dst = part + (((size_t)slice * ntiles + tile) * kTcM + q4 * 32 + (tid & 31)) * kTcN + h2 * 64;
-#pragma unroll
-  for (int cg = 0; cg < 2; ++cg) {
-    float u[32];
-    tmem_ld32(tcol + kTcN + cg * 32, u);
-#pragma unroll
-    for (int i = 0; i < 32; i += 4)
-      *reinterpret_cast<float4*>(dst + cg * 32 + i) = make_float4(u[i], u[i + 1], u[i + 2], u[i + 3]);
-  }
-  tc_fence_before();
-  __syncthreads();
-  if (warp == 0) tmem_dealloc(taddr, 2 * kTcN);
+  if (warp == 0) tmem_dealloc(tm, 512);
 }
 
-// out[t * 3 + li] = sum over slices of D[m = li * S + a][n = pair(b, c)].
-__global__ void k_tc_reduce(const float* __restrict__ part, int nslices, int ntiles, const int* __restrict__ om,
-                            const int* __restrict__ on, int nout, double* __restrict__ out) {
-  const int o = blockIdx.x * blockDim.x + threadIdx.x;
-  if (o >= nout) return;
-  const int m = om[o], n = on[o];
-  if (m < 0) {
-    out[o] = 0.0;
-    return;
-  }
-  const int tile = n / kTcN, col = n - tile * kTcN;
+// out[o] = sum over slices of the partials at off[o] (-1: 0).  A block takes 32
+// outputs: 8 threads each sum every eighth slice, then in a fixed order.
+__global__ void __launch_bounds__(256) k_tc_reduce(const float* __restrict__ part, int nslices, long long stride,
+                                                   const int* __restrict__ off, int nout, double* __restrict__ out) {
+  __shared__ double sh[8][33];
+  const int o = blockIdx.x * 32 + threadIdx.x;
+  const int p = o < nout ? off[o] : -1;
   double s = 0.0;
-  for (int k = 0; k < nslices; ++k) s += (double)part[(((size_t)k * ntiles + tile) * kTcM + m) * kTcN + col];
-  out[o] = s;
+  if (p >= 0)
+    for (int k = threadIdx.y; k < nslices; k += 8) s += (double)__ldg(part + k * stride + p);
+  sh[threadIdx.y][threadIdx.x] = s;
+  __syncthreads();
+  if (threadIdx.y == 0 && o < nout) {
+    for (int k = 1; k < 8; ++k) s += sh[k][threadIdx.x];
+    out[o] = s;
+  }
 }
 
 template <int NS>
-static size_t tc_smem_bytes(int nf) {
-  return 2 * (size_t)tc_stage_bytes<NS>() + 3 * sizeof(float) * (size_t)nf * kTcRow + 2 * sizeof(uint64_t) + 16;
-}
-
-cudaError_t launch_contract_tc(const float* I, long long N3, int nf, int S, const short2* pairs, int npairs,
-                               float* part, int* err, int nslices, int chunks, int nsplit, cudaStream_t s) {
-  const int ntiles = (npairs + kTcN - 1) / kTcN;
-  const dim3 grid(ntiles, nslices);
-  if (nsplit == 2) {
-    const size_t sm = tc_smem_bytes<2>(nf);
-    raise_smem_limit((const void*)k_contract_tc<2>, sm);
-    k_contract_tc<2><<<grid, kTcThreads, sm, s>>>(I, N3, nf, S, pairs, npairs, chunks, part, err);
-  } else {
-    const size_t sm = tc_smem_bytes<3>(nf);
-    raise_smem_limit((const void*)k_contract_tc<3>, sm);
-    k_contract_tc<3><<<grid, kTcThreads, sm, s>>>(I, N3, nf, S, pairs, npairs, chunks, part, err);
-  }
+static cudaError_t run_tc(const CUtensorMap& map, int nf, int S, int nl, const TcGroup* groups, int ngroups,
+                          const short2* pairs, long long nchunks, int chunks, int nslices, int ncols, float* part,
+                          int* err, cudaStream_t s) {
+  const size_t sm = (size_t)kTcRing * ((nf * kTcKC * 4 + 1023) & ~1023) + 2 * NS * (size_t)kTcPartBytes + 1024;
+  const cudaError_t e = raise_smem_limit((const void*)k_contract_tc<NS>, sm);
+  if (e != cudaSuccess) return e;
+  k_contract_tc<NS><<<dim3(ngroups, nslices), kTcThreads, sm, s>>>(map, nf, S, nl, groups, pairs, nchunks, chunks,
+                                                                   ncols, part, err);
   return cudaGetLastError();
 }
 
-cudaError_t launch_tc_reduce(const float* part, int nslices, int ntiles, const int* om, const int* on, int nout,
-                             double* out, cudaStream_t s) {
-  k_tc_reduce<<<(nout + 255) / 256, 256, 0, s>>>(part, nslices, ntiles, om, on, nout, out);
+// I: the nf = nl S shell fields of N3 points each.
+cudaError_t launch_contract_tc(const float* I, long long N3, int S, int nl, const TcGroup* groups, int ngroups,
+                               const short2* pairs, int ncols, float* part, int* err, int nslices, int chunks,
+                               int nsplit, cudaStream_t s) {
+  const int nf = nl * S;
+  typedef CUresult (*Encode)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                             const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                             CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+  void* fn = nullptr;
+  cudaDriverEntryPointQueryResult qr;
+  const cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &qr);
+  if (e != cudaSuccess) return e;
+  if (qr != cudaDriverEntryPointSuccess || !fn) return cudaErrorNotSupported;
+  // x = the points (a multiple of 8 of them: every field starts on a 16-byte
+  // boundary; chunks start at multiples of 32; points past the end read as 0)
+  CUtensorMap map;
+  const cuuint64_t dim[2] = {(cuuint64_t)N3, (cuuint64_t)nf}, stride[1] = {(cuuint64_t)N3 * 4};
+  const cuuint32_t box[2] = {kTcKC, (cuuint32_t)nf}, one[2] = {1, 1};
+  if (reinterpret_cast<Encode>(fn)(&map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(I), dim, stride, box,
+                                   one, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                                   CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    return cudaErrorInvalidValue;
+  const long long nchunks = (N3 + kTcKC - 1) / kTcKC;
+  return nsplit == 2 ? run_tc<2>(map, nf, S, nl, groups, ngroups, pairs, nchunks, chunks, nslices, ncols, part, err, s)
+                     : run_tc<3>(map, nf, S, nl, groups, ngroups, pairs, nchunks, chunks, nslices, ncols, part, err, s);
+}
+
+cudaError_t launch_tc_reduce(const float* part, int nslices, int ncols, const int* off, int nout, double* out,
+                             cudaStream_t s) {
+  k_tc_reduce<<<(nout + 31) / 32, dim3(32, 8), 0, s>>>(part, nslices, (long long)ncols * kTcM, off, nout, out);
   return cudaGetLastError();
 }
 
