@@ -85,7 +85,7 @@ extern "C" void fkp_context_destroy(void* ctx) { delete static_cast<Context*>(ct
 // plan
 // ----------------------------------------------------------------------------
 
-static bool radix_plan(int n, FftPlan& p) {
+bool fkp::radix_plan(int n, FftPlan& p) {
   p.n = n;
   p.nst = 0;
   int m = n;

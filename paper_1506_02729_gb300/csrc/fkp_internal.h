@@ -135,6 +135,9 @@ int set_error(int code, const char* fmt, ...);
 // least `bytes`.  The limit is process-wide per kernel and is never lowered
 // here, so a launch with a smaller need on another thread stays valid.
 cudaError_t raise_smem_limit(const void* func, size_t bytes);
+bool radix_plan(int n, FftPlan& p);
+// Side of the grid of the triangle sums of a shell set with |n_a| <= mm on an N^3 plan.
+int sum_grid(int N, int mm);
 void build_moments(int lmax, MomentTable& mt);
 int z_threads_for(int N);
 bool moments_identities_hold(const MomentTable& mt, int lmax);

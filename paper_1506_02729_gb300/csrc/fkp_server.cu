@@ -84,8 +84,9 @@ size_t estimate_plan(const fkp_request_t& r) {
     const int nl = (r.want & FKP_B4) ? 3 : ((r.want & FKP_B2) ? 2 : 1);
     const double hmax = r.bshells.first + (S - 1.0) * r.bshells.step + 0.5 * r.bshells.width;
     const size_t mm = (size_t)hmax, w2 = 2 * mm + 1, m1 = mm + 1;
-    b += 3 * w2 * w2 * m1 * 8 + (size_t)S * N * w2 * m1 * 8 + (size_t)S * N * N * m1 * 8 + (size_t)nl * S * N3 * 4;
-    const size_t slices = (N3 + 65535) / 65536, pairs = (size_t)S * (S + 1) / 2;
+    const size_t M = (size_t)sum_grid(N, (int)mm), M3 = M * M * M;
+    b += 3 * w2 * w2 * m1 * 8 + (size_t)S * M * w2 * m1 * 8 + (size_t)S * M * M * m1 * 8 + (size_t)nl * S * M3 * 4;
+    const size_t slices = (M3 + 65535) / 65536, pairs = (size_t)S * (S + 1) / 2;
     b += slices * ((pairs + 127) / 128) * 128 * 144 * 4 + slices * 16384 * 8;
   }
   return b + b / 10 + (64 << 20);
