@@ -342,12 +342,12 @@ static int tune_schedule(Plan* P) {
     float bx = 1e30f, by = 1e30f, bz = 1e30f;
     for (int xm : {1, 2, 4, 8}) {
       const float t = timed([&] { return launch_xpass(P->d_grid, nullptr, P->g, P->mt, P->fp, P->d_tw, P->d_S1,
-                                                      P->ctx->nsm, s, P->reach, xm); }, "x-pass");
+                                                      P->ctx->nsm, s, P->reach, nullptr, xm); }, "x-pass");
       if (t < bx) { bx = t; best.x_mult = xm; }
     }
     for (int nt : {256, 512}) {
       const float t = timed([&] { return launch_ypass(P->d_S1, P->d_grid, nullptr, P->g, P->mt, P->fp, P->d_tw,
-                                                      P->d_S2, P->d_err + 1, s, P->reach, nt); }, "y-pass");
+                                                      P->d_S2, P->d_err + 1, s, P->reach, nullptr, nt); }, "y-pass");
       if (t < by) { by = t; best.y_threads = nt; }
     }
     // the z-pass block shape sets the partition of each k_z column into the
@@ -549,8 +549,10 @@ extern "C" int fkp_plan_create(void* vctx, const fkp_geometry_t* geom, const fkp
   auto A = [&](size_t bytes) { void* p = P->alloc(bytes); if (!p) ok = false; return p; };
   P->d_grid = (unsigned long long*)A(N3 * 8 * (P->per_object ? (size_t)P->mt.nfields : 1));
   if (wantB) P->d_gridw = (unsigned long long*)A(N3 * 8);
+  P->d_occ = (int*)A(sizeof(int) * occ_ints(N));
   if (P->interlace) {
     P->d_grid2 = (unsigned long long*)A(N3 * 8);
+    P->d_occ2 = (int*)A(sizeof(int) * occ_ints(N));
     if (wantB) P->d_gridw2 = (unsigned long long*)A(N3 * 8);
   }
   P->d_hph = (float2*)A(sizeof(float2) * N);
@@ -742,7 +744,8 @@ static int grid_pass(Plan* P, const CatDev& gal, const CatDev& ran, cudaStream_t
     CK(launch_bin_count(ran, 1, geo, P->d_scpart + (size_t)nbg * SC_NSUM, bh_ran, P->d_err, nbr, s));
   CK(launch_scalars_finalize(P->d_scpart, nbg, nbr, gal.n, nran, geo.alpha_mode, P->d_ds, s));
   CK(launch_tile_prefix(P->d_bhist, nbg + (cached ? 0 : nbr), P->ntiles, P->d_tcnt, s));
-  CK(launch_scan_tiles(P->d_tcnt, P->ntiles, P->d_toff, P->d_titem, s));
+  CK(launch_scan_tiles(P->d_tcnt, P->ntiles, P->d_toff, P->d_titem, s, geo,
+                       cached ? (which ? P->rc_tcnt2 : P->rc_tcnt) : nullptr, which ? P->d_occ2 : P->d_occ));
   CK(stage(1));
   CK(cudaStreamWaitEvent(s, P->ev_join, 0));
   const double* obs = P->geom.observer;
@@ -801,7 +804,9 @@ static int cache_randoms(Plan* P, const CatDev& ran, cudaStream_t s) {
     }
     P->rc_part = (double*)P->alloc(sizeof(double) * SC_NSUM * nb);
     P->rc_lab = (double*)P->alloc(sizeof(double) * LAB_NSUM);
-    if (!P->rc_grid || (P->d_gridw && !P->rc_gridw) || !P->rc_part || !P->rc_lab ||
+    P->rc_tcnt = (int*)P->alloc(sizeof(int) * P->ntiles);
+    P->rc_tcnt2 = P->interlace ? (int*)P->alloc(sizeof(int) * P->ntiles) : P->rc_tcnt;
+    if (!P->rc_grid || (P->d_gridw && !P->rc_gridw) || !P->rc_part || !P->rc_lab || !P->rc_tcnt || !P->rc_tcnt2 ||
         (P->interlace && (!P->rc_grid2 || (P->d_gridw && !P->rc_gridw2))))
       return set_error(FKP_ENOMEM, "cannot allocate the cached random grids");
   }
@@ -825,7 +830,8 @@ static int cache_randoms(Plan* P, const CatDev& ran, cudaStream_t s) {
     unsigned long long* rgw = which ? P->rc_gridw2 : P->rc_gridw;
     CK(launch_bin_count(ran, 1, geo, P->rc_part, P->d_bhist, P->d_err, nbr, s));
     CK(launch_tile_prefix(P->d_bhist, nbr, P->ntiles, P->d_tcnt, s));
-    CK(launch_scan_tiles(P->d_tcnt, P->ntiles, P->d_toff, P->d_titem, s));
+    CK(launch_scan_tiles(P->d_tcnt, P->ntiles, P->d_toff, P->d_titem, s, geo, nullptr, nullptr));
+    CK(cudaMemcpyAsync(which ? P->rc_tcnt2 : P->rc_tcnt, P->d_tcnt, sizeof(int) * P->ntiles, cudaMemcpyDeviceToDevice, s));
     CK(cudaMemsetAsync(rg, 0, N3 * 8, s));
     if (rgw) CK(cudaMemsetAsync(rgw, 0, N3 * 8, s));
     CK(launch_bin_scatter(ran, 1, geo, P->geom.observer, P->d_ds, P->d_toff, P->d_bhist, P->d_xyzv, vw2, P->d_labpart, nbr, s,
@@ -889,24 +895,28 @@ ZParams fkp::zparams(const Plan* P, int mode) {
   zp.interlace = P->interlace ? 1 : 0;
   zp.hph = P->d_hph;
   zp.scale = P->interlace ? 0.5f : 1.f;
+  zp.occ = P->d_occ;
+  zp.occ2 = P->d_occ2;
   zp.split68 = (P->want & (FKP_P6B | FKP_P8B)) && P->lmax >= 4 ? 1 : 0;
   return zp;
 }
 
 int fkp::enqueue_xy(Plan* P, const unsigned long long* gq, const unsigned long long* gq2, const float* gf,
                     cudaStream_t s, const PassReach& pr, bool events) {
-  CK(launch_xpass(gq, gf, P->g, P->mt, P->fp, P->d_tw, P->d_S1, P->ctx->nsm, s, pr, P->sched.x_mult, MockBatch(),
+  const int* occ = gq ? P->d_occ : nullptr;  // a given field: every row
+  CK(launch_xpass(gq, gf, P->g, P->mt, P->fp, P->d_tw, P->d_S1, P->ctx->nsm, s, pr, occ, P->sched.x_mult, MockBatch(),
                   P->per_object));
   if (events) CK(record_stage(P->ev[3], s));
-  CK(launch_ypass(P->d_S1, gq, gf, P->g, P->mt, P->fp, P->d_tw, P->d_S2, P->d_err + 1, s, pr,
+  CK(launch_ypass(P->d_S1, gq, gf, P->g, P->mt, P->fp, P->d_tw, P->d_S2, P->d_err + 1, s, pr, occ,
                   P->sched.y_threads));
   if (P->interlace) {
     // the second grid's groups follow the first's; the z-pass applies its
     // half-cell phase e^{-i pi (n_x + n_y + n_z)/N}
     float2* S2b = P->d_S2 + field_elems(P->g.N) * P->mt.ngroups;
-    CK(launch_xpass(gq2, nullptr, P->g2, P->mt, P->fp, P->d_tw, P->d_S1, P->ctx->nsm, s, pr, P->sched.x_mult));
+    CK(launch_xpass(gq2, nullptr, P->g2, P->mt, P->fp, P->d_tw, P->d_S1, P->ctx->nsm, s, pr, P->d_occ2,
+                    P->sched.x_mult));
     CK(launch_ypass(P->d_S1, gq2, nullptr, P->g2, P->mt, P->fp, P->d_tw, S2b, P->d_err + 1, s, pr,
-                    P->sched.y_threads));
+                    P->d_occ2, P->sched.y_threads));
   }
   if (events) CK(record_stage(P->ev[4], s));
   return FKP_OK;
@@ -917,7 +927,8 @@ int fkp::enqueue_xy(Plan* P, const unsigned long long* gq, const unsigned long l
 int fkp::enqueue_fft_bin(Plan* P, const unsigned long long* gq, const float* gf, cudaStream_t s) {
   const int rc = enqueue_xy(P, gq, P->d_grid2, gf, s, P->reach, true);
   if (rc) return rc;
-  const ZParams zp = zparams(P, 0);
+  ZParams zp = zparams(P, 0);
+  if (!gq) zp.occ = nullptr;
   CK(launch_zpass(P->d_S2, P->g, P->mt, P->fp, P->d_tw, zp, P->reach, P->d_zpart, P->d_zpartc, P->d_err + 1, s,
                   P->ctx->nsm, P->sched.z_threads));
   CK(launch_reduce_bins(P->d_zpart, P->d_zpartc, zpass_blocks(P->reach, P->sched.z_threads, P->ctx->nsm),
@@ -1117,7 +1128,7 @@ extern "C" int fkp_grid(void* plan, const fkp_catalog_t* gal, const fkp_catalog_
 // Per-mock element counts of the fused batch workspace.
 namespace {
 struct BatchSizes {
-  size_t grid, s1, s2, zpart, zpartc, bins, binc, ds, err;
+  size_t grid, s1, s2, zpart, zpartc, bins, binc, ds, err, occ;
 };
 BatchSizes batch_sizes(const fkp::Plan* P) {
   const size_t N = (size_t)P->g.N, half = fkp::field_elems(P->g.N);
@@ -1131,6 +1142,7 @@ BatchSizes batch_sizes(const fkp::Plan* P) {
   z.binc = (size_t)P->pb.nbins;
   z.ds = DS_COUNT + LAB_NSUM + 8;
   z.err = 4;
+  z.occ = occ_ints(P->g.N);
   return z;
 }
 size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
@@ -1142,9 +1154,10 @@ static int reserve_batch(fkp::Plan* P, int nmock) {
   if (P->batch_cap >= nmock) return FKP_OK;
   const BatchSizes z = batch_sizes(P);
   const size_t K = (size_t)nmock;
-  const size_t parts[9] = {align256(K * z.grid * 8),  align256(K * z.s1 * 8),     align256(K * z.s2 * 8),
+  const size_t parts[10] = {align256(K * z.grid * 8),  align256(K * z.s1 * 8),     align256(K * z.s2 * 8),
                            align256(K * z.zpart * 8), align256(K * z.zpartc * 4), align256(K * z.bins * 8),
-                           align256(K * z.binc * 8),  align256(K * z.ds * 8),     align256(K * z.err * 4)};
+                           align256(K * z.binc * 8),  align256(K * z.ds * 8),     align256(K * z.err * 4),
+                           align256(K * z.occ * 4)};
   size_t tot = 0;
   for (size_t b : parts) tot += b;
   if (P->ctx->budget && P->bytes_total + tot > P->ctx->budget)
@@ -1168,7 +1181,8 @@ static int reserve_batch(fkp::Plan* P, int nmock) {
   P->b_bins = reinterpret_cast<double*>(m);              m += parts[5];
   P->b_binc = reinterpret_cast<long long*>(m);           m += parts[6];
   P->b_ds = reinterpret_cast<double*>(m);                m += parts[7];
-  P->b_err = reinterpret_cast<int*>(m);
+  P->b_err = reinterpret_cast<int*>(m);                  m += parts[8];
+  P->b_occ = reinterpret_cast<int*>(m);
   P->batch_cap = nmock;
   P->batch_bytes = tot;
   return FKP_OK;
@@ -1193,6 +1207,7 @@ extern "C" int fkp_power_batch(void* plan, int nmock, const fkp_catalog_t* gals,
   unsigned long long* const grid0 = P->d_grid;
   double* const ds0 = P->d_ds;
   int* const err0 = P->d_err;
+  int* const occ0 = P->d_occ;
   CK(cudaEventRecord(P->ev[9], s));
   for (int k = 0; k < nmock; ++k) {
     CatDev g, r;
@@ -1202,7 +1217,9 @@ extern "C" int fkp_power_batch(void* plan, int nmock, const fkp_catalog_t* gals,
     P->d_grid = P->b_grid + k * z.grid;
     P->d_ds = P->b_ds + k * z.ds;
     P->d_err = P->b_err + k * z.err;
+    P->d_occ = P->b_occ + k * z.occ;
     rc = enqueue_grids(P, g, r, s);
+    P->d_occ = occ0;
     P->d_grid = grid0;
     P->d_ds = ds0;
     P->d_err = err0;
@@ -1212,18 +1229,19 @@ extern "C" int fkp_power_batch(void* plan, int nmock, const fkp_catalog_t* gals,
   // (blockIdx.z / blockIdx.y = mock); bounded-wait flags go to mock 0's word
   int* perr = P->b_err + 1;
   MockBatch mx;
-  mx.n = nmock; mx.in = (long long)z.grid; mx.out = (long long)z.s1;
-  CK(launch_xpass(P->b_grid, nullptr, P->g, P->mt, P->fp, P->d_tw, P->b_S1, P->ctx->nsm, s, P->reach, P->sched.x_mult,
+  mx.n = nmock; mx.in = (long long)z.grid; mx.out = (long long)z.s1; mx.occ = (int)z.occ;
+  CK(launch_xpass(P->b_grid, nullptr, P->g, P->mt, P->fp, P->d_tw, P->b_S1, P->ctx->nsm, s, P->reach, P->b_occ, P->sched.x_mult,
                   mx));
   CK(cudaEventRecord(P->ev[3], s));
   MockBatch my;
-  my.n = nmock; my.in = (long long)z.s1; my.in2 = (long long)z.grid; my.out = (long long)z.s2;
-  CK(launch_ypass(P->b_S1, P->b_grid, nullptr, P->g, P->mt, P->fp, P->d_tw, P->b_S2, perr, s, P->reach,
+  my.n = nmock; my.in = (long long)z.s1; my.in2 = (long long)z.grid; my.out = (long long)z.s2; my.occ = (int)z.occ;
+  CK(launch_ypass(P->b_S1, P->b_grid, nullptr, P->g, P->mt, P->fp, P->d_tw, P->b_S2, perr, s, P->reach, P->b_occ,
                   P->sched.y_threads, my));
   CK(cudaEventRecord(P->ev[4], s));
-  const ZParams zp = zparams(P, 0);
+  ZParams zp = zparams(P, 0);
+  zp.occ = P->b_occ;
   MockBatch mz;
-  mz.n = nmock; mz.in = (long long)z.s2; mz.out = (long long)z.zpart; mz.out2 = (long long)z.zpartc;
+  mz.n = nmock; mz.in = (long long)z.s2; mz.out = (long long)z.zpart; mz.out2 = (long long)z.zpartc; mz.occ = (int)z.occ;
   CK(launch_zpass(P->b_S2, P->g, P->mt, P->fp, P->d_tw, zp, P->reach, P->b_zpart, P->b_zpartc, perr, s, P->ctx->nsm,
                   P->sched.z_threads, mz));
   CK(launch_reduce_bins(P->b_zpart, P->b_zpartc, zpass_blocks(P->reach, P->sched.z_threads, P->ctx->nsm), P->pb.nbins,

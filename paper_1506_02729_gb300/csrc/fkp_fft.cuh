@@ -240,9 +240,11 @@ __device__ __forceinline__ int ilvx(int i, int p) {
 // The block is 2-D: threadIdx.x = pencil (blockDim.x == P), threadIdx.y
 // strides over the N/R butterflies of a stage (blockDim.y == NT / P).
 // RXI / RXO: the stage reads / writes the row-permuted layout.
-template <int N, int P, int NT, int DIR, int R, int NS, bool SWZ, bool RXI = false, bool RXO = false>
+// HULL (first stage): only the elements [lo, lo + len) of a pencil are in src,
+// the others are zero and not read.
+template <int N, int P, int NT, int DIR, int R, int NS, bool SWZ, bool RXI = false, bool RXO = false, bool HULL = false>
 __device__ __forceinline__ void fft_ct_stage(const float2* __restrict__ src, float2* __restrict__ dst,
-                                             const float2* __restrict__ tw) {
+                                             const float2* __restrict__ tw, int lo = 0, unsigned len = 0) {
   constexpr int NB = N / R;
   constexpr int JT = NT / P;
   constexpr int TWS = N / (NS * R);
@@ -254,7 +256,8 @@ __device__ __forceinline__ void fft_ct_stage(const float2* __restrict__ src, flo
       const int k = j % NS;
       float2 v[R];
 #pragma unroll
-      for (int r = 0; r < R; ++r) v[r] = src[ilvx<P, SWZ, RXI>(j + r * NB, p)];
+      for (int r = 0; r < R; ++r)
+        v[r] = !HULL || (unsigned)(j + r * NB - lo) < len ? src[ilvx<P, SWZ, RXI>(j + r * NB, p)] : make_float2(0.f, 0.f);
       if (NS > 1) {
 #pragma unroll
         for (int r = 1; r < R; ++r) {
@@ -271,13 +274,13 @@ __device__ __forceinline__ void fft_ct_stage(const float2* __restrict__ src, flo
   }
 }
 
-template <int N, int P, int NT, int DIR, int S, int NS, bool SWZ, bool RX = false>
-__device__ __forceinline__ float2* fft_ct_run(float2* a, float2* b, const float2* tw) {
+template <int N, int P, int NT, int DIR, int S, int NS, bool SWZ, bool RX = false, bool HULL = false>
+__device__ __forceinline__ float2* fft_ct_run(float2* a, float2* b, const float2* tw, int lo = 0, unsigned len = 0) {
   if constexpr (S == radix_count(N)) {
     return a;
   } else {
     constexpr int R = radix_at(N, S);
-    fft_ct_stage<N, P, NT, DIR, R, NS, SWZ, (RX && (S > 0)), RX>(a, b, tw);
+    fft_ct_stage<N, P, NT, DIR, R, NS, SWZ, (RX && (S > 0)), RX, (HULL && (S == 0))>(a, b, tw, lo, len);
     __syncthreads();
     return fft_ct_run<N, P, NT, DIR, S + 1, NS * R, SWZ, RX>(b, a, tw);
   }
@@ -288,22 +291,22 @@ __device__ __forceinline__ float2* fft_ct_run(float2* a, float2* b, const float2
 // block call it; it ends with a __syncthreads().  RX (P = 8, no swizzle):
 // the input is in the natural interleave and the result in the
 // row-permuted one (element i of pencil p at rowx(i) * 8 + p).
-template <int N, int P, int NT, int DIR, bool SWZ = false, bool RX = false>
-__device__ __forceinline__ float2* fft_ct(float2* a, float2* b, const float2* tw) {
+template <int N, int P, int NT, int DIR, bool SWZ = false, bool RX = false, bool HULL = false>
+__device__ __forceinline__ float2* fft_ct(float2* a, float2* b, const float2* tw, int lo = 0, unsigned len = 0) {
   static_assert(!RX || (P == 8 && !SWZ), "the row permutation is for 8 unswizzled pencils");
-  return fft_ct_run<N, P, NT, DIR, 0, 1, SWZ, RX>(a, b, tw);
+  return fft_ct_run<N, P, NT, DIR, 0, 1, SWZ, RX, HULL>(a, b, tw, lo, len);
 }
 
 // Stages S .. SEND-1 of fft_ct_run; returns the buffer holding their result.
-template <int N, int P, int NT, int DIR, int S, int NS, int SEND, bool SWZ, bool RX>
-__device__ __forceinline__ float2* fft_ct_upto(float2* a, float2* b, const float2* tw) {
+template <int N, int P, int NT, int DIR, int S, int NS, int SEND, bool SWZ, bool RX, bool HULL>
+__device__ __forceinline__ float2* fft_ct_upto(float2* a, float2* b, const float2* tw, int lo, unsigned len) {
   if constexpr (S == SEND) {
     return a;
   } else {
     constexpr int R = radix_at(N, S);
-    fft_ct_stage<N, P, NT, DIR, R, NS, SWZ, (RX && (S > 0)), RX>(a, b, tw);
+    fft_ct_stage<N, P, NT, DIR, R, NS, SWZ, (RX && (S > 0)), RX, (HULL && (S == 0))>(a, b, tw, lo, len);
     __syncthreads();
-    return fft_ct_upto<N, P, NT, DIR, S + 1, NS * R, SEND, SWZ, RX>(b, a, tw);
+    return fft_ct_upto<N, P, NT, DIR, S + 1, NS * R, SEND, SWZ, RX, HULL>(b, a, tw, lo, len);
   }
 }
 
@@ -324,20 +327,18 @@ __host__ __device__ constexpr bool fft_fusable() {
 // outputs to the caller instead of storing them: thread (p, y) receives
 // output index y + i NT/P of pencil p as f(i, value), for every i in
 // [0, N P / NT), each exactly once, in registers.  The earlier stages run as
-// in fft_ct and end with a __syncthreads(); the last one reads the buffer
-// returned in *last_src and stores nothing, so the other buffer is free and
-// the caller synchronises before either is reused.
-template <int N, int P, int NT, int DIR, bool SWZ, bool RX, class F>
-__device__ __forceinline__ void fft_ct_fused(float2* a, float2* b, const float2* tw, F&& f,
-                                             const float2** last_src = nullptr) {
+// in fft_ct and end with a __syncthreads(); the last one stores nothing, and
+// the caller synchronises before either buffer is reused.
+template <int N, int P, int NT, int DIR, bool SWZ, bool RX, bool HULL = false, class F>
+__device__ __forceinline__ void fft_ct_fused(float2* a, float2* b, const float2* tw, F&& f, int lo = 0,
+                                             unsigned len = 0) {
   static_assert(fft_fusable<N, P, NT>(), "the last stage's outputs do not map onto the threads' runs");
   constexpr int SL = radix_count(N) - 1;
   constexpr int R = radix_at(N, SL);
   constexpr int NS = radix_prod(N, SL);  // = N / R
   constexpr int NB = N / R;
   constexpr int JT = NT / P;
-  const float2* src = fft_ct_upto<N, P, NT, DIR, 0, 1, SL, SWZ, RX>(a, b, tw);
-  if (last_src) *last_src = src;
+  const float2* src = fft_ct_upto<N, P, NT, DIR, 0, 1, SL, SWZ, RX, HULL>(a, b, tw, lo, len);
   const int p = threadIdx.x;
 #pragma unroll
   for (int j0 = 0; j0 < NB; j0 += JT) {
@@ -360,9 +361,9 @@ __device__ __forceinline__ void fft_ct_fused(float2* a, float2* b, const float2*
 
 // Runtime-N version on the same interleaved layout (sizes without a
 // compiled specialisation).
-template <int R, int DIR, bool SWZ>
+template <int R, int DIR, bool SWZ, bool HULL>
 __device__ __forceinline__ void fft_rt_stage(const float2* __restrict__ src, float2* __restrict__ dst, int n, int P,
-                                             int ns, const float2* __restrict__ tw) {
+                                             int ns, const float2* __restrict__ tw, int lo, unsigned len) {
   const int nb = n / R;
   const int tot = nb * P;
   const int tws = n / (ns * R);
@@ -373,7 +374,11 @@ __device__ __forceinline__ void fft_rt_stage(const float2* __restrict__ src, flo
     const int k = j % ns;
     float2 v[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = src[SWZ ? (j + r * nb) * P + (p ^ (((j + r * nb) >> 1) & (P - 1))) : (j + r * nb) * P + p];
+    for (int r = 0; r < R; ++r) {
+      const int i = j + r * nb;
+      v[r] = make_float2(0.f, 0.f);
+      if (!HULL || ns > 1 || (unsigned)(i - lo) < len) v[r] = src[SWZ ? i * P + (p ^ ((i >> 1) & (P - 1))) : i * P + p];
+    }
     if (ns > 1) {
 #pragma unroll
       for (int r = 1; r < R; ++r) {
@@ -392,17 +397,18 @@ __device__ __forceinline__ void fft_rt_stage(const float2* __restrict__ src, flo
   }
 }
 
-template <int DIR, bool SWZ = false>
-__device__ float2* fft_rt(float2* a, float2* b, int P, const FftPlan& fp, const float2* tw) {
+template <int DIR, bool SWZ = false, bool HULL = false>
+__device__ float2* fft_rt(float2* a, float2* b, int P, const FftPlan& fp, const float2* tw, int lo = 0,
+                          unsigned len = 0) {
   int ns = 1;
   for (int s = 0; s < fp.nst; ++s) {
     const int R = fp.radix[s];
     switch (R) {
-      case 8: fft_rt_stage<8, DIR, SWZ>(a, b, fp.n, P, ns, tw); break;
-      case 4: fft_rt_stage<4, DIR, SWZ>(a, b, fp.n, P, ns, tw); break;
-      case 2: fft_rt_stage<2, DIR, SWZ>(a, b, fp.n, P, ns, tw); break;
-      case 5: fft_rt_stage<5, DIR, SWZ>(a, b, fp.n, P, ns, tw); break;
-      default: fft_rt_stage<3, DIR, SWZ>(a, b, fp.n, P, ns, tw); break;
+      case 8: fft_rt_stage<8, DIR, SWZ, HULL>(a, b, fp.n, P, ns, tw, lo, len); break;
+      case 4: fft_rt_stage<4, DIR, SWZ, HULL>(a, b, fp.n, P, ns, tw, lo, len); break;
+      case 2: fft_rt_stage<2, DIR, SWZ, HULL>(a, b, fp.n, P, ns, tw, lo, len); break;
+      case 5: fft_rt_stage<5, DIR, SWZ, HULL>(a, b, fp.n, P, ns, tw, lo, len); break;
+      default: fft_rt_stage<3, DIR, SWZ, HULL>(a, b, fp.n, P, ns, tw, lo, len); break;
     }
     __syncthreads();
     float2* t = a;
@@ -416,10 +422,11 @@ __device__ float2* fft_rt(float2* a, float2* b, int P, const FftPlan& fp, const 
 // N = 0 selects the runtime version.  SWZ: swizzled interleave (see ilv).
 // RX: the compile-time version leaves its result row-permuted (see fft_ct);
 // the runtime version ignores it, so read results through res_row<N, RX>.
-template <int N, int P, int NT, int DIR, bool SWZ = false, bool RX = false>
-__device__ __forceinline__ float2* fft_any(float2* a, float2* b, const FftPlan& fp, const float2* tw) {
-  if constexpr (N > 0) return fft_ct<N, P, NT, DIR, SWZ, RX>(a, b, tw);
-  else return fft_rt<DIR, SWZ>(a, b, P, fp, tw);
+template <int N, int P, int NT, int DIR, bool SWZ = false, bool RX = false, bool HULL = false>
+__device__ __forceinline__ float2* fft_any(float2* a, float2* b, const FftPlan& fp, const float2* tw, int lo = 0,
+                                           unsigned len = 0) {
+  if constexpr (N > 0) return fft_ct<N, P, NT, DIR, SWZ, RX, HULL>(a, b, tw, lo, len);
+  else return fft_rt<DIR, SWZ, HULL>(a, b, P, fp, tw, lo, len);
 }
 
 // Row of index i in the result of fft_any<N, ..., RX>.

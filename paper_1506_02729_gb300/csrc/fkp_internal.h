@@ -53,6 +53,7 @@ struct Plan {
 
   // power workspace
   unsigned long long *d_grid = nullptr, *d_gridw = nullptr;
+  int *d_occ = nullptr, *d_occ2 = nullptr;  // rows of the grids that hold objects (OccView)
   float2 *d_S1 = nullptr, *d_S2 = nullptr, *d_tw = nullptr;
   short* d_lut = nullptr;
   float* d_winv = nullptr;
@@ -89,6 +90,7 @@ struct Plan {
   bool rc_valid = false;
   unsigned long long *rc_grid = nullptr, *rc_gridw = nullptr;
   double *rc_part = nullptr, *rc_lab = nullptr;
+  int *rc_tcnt = nullptr, *rc_tcnt2 = nullptr;  // its tile counts
   int rc_nblk = 0;
   long long rc_n = 0;
 
@@ -121,7 +123,7 @@ struct Plan {
   unsigned long long* b_grid = nullptr;
   float2 *b_S1 = nullptr, *b_S2 = nullptr;
   double *b_zpart = nullptr, *b_bins = nullptr, *b_ds = nullptr;
-  int *b_zpartc = nullptr, *b_err = nullptr;
+  int *b_zpartc = nullptr, *b_err = nullptr, *b_occ = nullptr;
   long long* b_binc = nullptr;
 
   std::vector<void*> buffers;
@@ -172,7 +174,10 @@ int assign_tiles_per_axis(int N);
 cudaError_t launch_bin_count(const CatDev& c, int is_ran, const GeomDev& g, double* part, int* bh, int* err,
                              int nblk, cudaStream_t s);
 cudaError_t launch_tile_prefix(int* bh, int nrows, int ntiles, int* cnt, cudaStream_t s);
-cudaError_t launch_scan_tiles(const int* cnt, int ntiles, int* off, int* items, cudaStream_t s);
+// occ: NULL, or the plan's list of occupied rows; more: NULL, or the tile
+// counts of a cached random catalog.
+cudaError_t launch_scan_tiles(const int* cnt, int ntiles, int* off, int* items, cudaStream_t s, const GeomDev& g,
+                              const int* more, int* occ);
 cudaError_t launch_bin_scatter(const CatDev& c, int is_ran, const GeomDev& g, const double obs[3], const double* ds,
                                const int* off, const int* bpref, float4* xyzv, float* vw2, double* labpart, int nblk,
                                cudaStream_t s, int raw = 0);
@@ -194,11 +199,11 @@ cudaError_t launch_wait_selftest(unsigned polls, int* flag, cudaStream_t s);
 // the nodes.
 cudaError_t launch_xpass(const unsigned long long* gq, const float* gf, const GeomDev& g, const MomentTable& mt,
                          const FftPlan& fp, const float2* tw, float2* S1, int nsm, cudaStream_t s,
-                         const PassReach& pr, int xm = 2, MockBatch mb = MockBatch(), bool per_object = false);
+                         const PassReach& pr, const int* occ = nullptr, int xm = 2, MockBatch mb = MockBatch(), bool per_object = false);
 cudaError_t launch_ypass(const float2* S1, const unsigned long long* gq, const float* gf, const GeomDev& g,
                          const MomentTable& mt, const FftPlan& fp,
                          const float2* tw, float2* S2, int* err, cudaStream_t s,
-                         const PassReach& pr, int nt = 256, MockBatch mb = MockBatch());
+                         const PassReach& pr, const int* occ = nullptr, int nt = 256, MockBatch mb = MockBatch());
 // The z-pass is persistent: zpass_blocks(pr, nt, nsm) blocks, each writing
 // one column of the partial bins (part[key][block]); reduce over that count.
 cudaError_t launch_zpass(const float2* S2, const GeomDev& g, const MomentTable& mt, const FftPlan& fp,

@@ -77,6 +77,7 @@ struct MockBatch {
   long long in2 = 0;   // y: stride of the grid (observer-node value)
   long long out = 0;   // stride of the output (x: S1; y: S2; z: partial bin sums)
   long long out2 = 0;  // z: stride of the partial bin counts
+  int occ = 0;         // stride of the occupied-row lists
 };
 
 // The modes the passes have to carry: those with |n|^2 <= r2, r2 the largest
@@ -94,6 +95,47 @@ struct PassReach {
   int nxt = 1;
   int nzt = 0;
   const int* ztiles = nullptr;
+};
+
+// Where a gridded field can differ from zero: the rows (z, y) that some
+// occupied tile of the gridding reaches, as one range of y per plane z and one
+// range of planes.  A survey fills a part of its box (the BOSS-like cap: 69 %
+// of the planes, under half of the rows); a zero row has a zero transform, so
+// the x-pass walks only the listed rows, the y-pass copies the listed rows of
+// the listed planes and reads the others as zeros, and the z-pass reads the
+// planes outside the range as zeros.  512^3 mock 8.58 -> 6.51 ms, the same on
+// cached randoms 11.42 -> 6.16 ms (with the unbinned modes left out too); a
+// field whose rows are all occupied pays about 1 % (256^3, 1.22 -> 1.24 ms).
+// Device layout: rows in all, first plane,
+// end plane, 0, then per plane y0 | y1 << 16, then the rows before each plane.
+// A null pointer means every row.
+__host__ __device__ constexpr int occ_ints(int N) { return 4 + N + N; }
+struct OccView {
+  const int* p;
+  int N;
+  __device__ __forceinline__ int rows() const { return p ? __ldg(p) : N * N; }
+  __device__ __forceinline__ int z0() const { return p ? __ldg(p + 1) : 0; }
+  __device__ __forceinline__ int z1() const { return p ? __ldg(p + 2) : N; }
+  __device__ __forceinline__ int2 yrange(int z) const {
+    if (!p) return make_int2(0, N);
+    const int v = __ldg(p + 4 + z);
+    return make_int2(v & 0xffff, v >> 16);
+  }
+  // row r of the list as (z, y)
+  __device__ __forceinline__ int2 row(int r) const {
+    if (!p) {
+      const int z = r / N;
+      return make_int2(z, r - z * N);
+    }
+    const int* off = p + 4 + N;
+    int lo = z0(), hi = z1() - 1;  // the last plane that begins at or before r (empty planes begin where the next does)
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (__ldg(off + mid) <= r) lo = mid;
+      else hi = mid - 1;
+    }
+    return make_int2(lo, (__ldg(p + 4 + lo) & 0xffff) + r - __ldg(off + lo));
+  }
 };
 
 // z-pass parameters.
@@ -117,6 +159,8 @@ struct ZParams {
   int interlace = 0;
   const float2* hph = nullptr;
   float scale = 1.f;
+  const int* occ = nullptr;   // the occupied planes of the grid, and of the second of an interlaced pair
+  const int* occ2 = nullptr;
   int split68 = 0;   // accumulate Re F_4 F_2* and |F_4|^2 (P_6b, P_8b)
 };
 

@@ -169,9 +169,25 @@ __global__ void __launch_bounds__(256) k_tile_prefix(int* __restrict__ bh, int n
 // number of items).  One block of 1024 threads walks the tiles in rounds of
 // 1024 (coalesced loads, the next round's counts loaded during this round's
 // warp-shuffle scan).
+// occ (if not null) receives the rows that the occupied tiles reach (OccView),
+// a tile counting as occupied when cnt or more (the cached random catalog's
+// counts, or null) says so: a tile's objects reach its cells, one cell below
+// and reach - kTile + 1 above, wrapped around a periodic box.
 __global__ void __launch_bounds__(1024) k_scan_tiles(const int* __restrict__ cnt, int ntiles, int* __restrict__ off,
-                                                     int* __restrict__ items) {
+                                                     int* __restrict__ items, const int* __restrict__ more, int ntx,
+                                                     int N, int reach, int periodic, int* __restrict__ occ) {
   __shared__ int wsum[32], wsumi[32];
+  __shared__ int ty0[32], ty1[32];  // per plane of tiles: first and last occupied tile row
+  __shared__ int zfirst, zlast;
+  if (threadIdx.x < 32) {
+    ty0[threadIdx.x] = 64;
+    ty1[threadIdx.x] = -1;
+  }
+  if (threadIdx.x == 0) {
+    zfirst = N;
+    zlast = -1;
+  }
+  __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int carry = 0, carryi = 0;  // totals of the earlier rounds (the same in every thread)
   int c = (int)threadIdx.x < ntiles ? cnt[threadIdx.x] : 0;
@@ -179,6 +195,11 @@ __global__ void __launch_bounds__(1024) k_scan_tiles(const int* __restrict__ cnt
     const int i = base + (int)threadIdx.x;
     const int cn = i + 1024 < ntiles ? cnt[i + 1024] : 0;
     const int ci = (c + kAccumChunk - 1) / kAccumChunk;
+    if (occ && i < ntiles && (c > 0 || (more && more[i] > 0))) {
+      const int q = i / ntx, tz = q / ntx, ty = q - tz * ntx;
+      if (ty < *(volatile int*)&ty0[tz]) atomicMin(&ty0[tz], ty);
+      if (ty > *(volatile int*)&ty1[tz]) atomicMax(&ty1[tz], ty);
+    }
     int s = c, si = ci;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -220,6 +241,50 @@ __global__ void __launch_bounds__(1024) k_scan_tiles(const int* __restrict__ cnt
   if (threadIdx.x == 0) {
     off[ntiles] = carry;
     items[ntiles] = carryi;
+  }
+  if (!occ) return;
+  // plane z = threadIdx.x (N <= 512): the hull of the rows of the tile planes that reach it
+  const int z = threadIdx.x;
+  int y0 = N, y1 = 0;
+  if (z < N) {
+    for (int tz = 0; tz < ntx; ++tz) {
+      if (ty1[tz] < 0) continue;
+      const int a = tz * kTile - 1, b = tz * kTile + reach;
+      if (!((z >= a && z <= b) || (periodic && ((z - N >= a && z - N <= b) || (z + N >= a && z + N <= b))))) continue;
+      const int ya = ty0[tz] * kTile - 1, yb = ty1[tz] * kTile + reach;
+      if (periodic && (ya < 0 || yb >= N)) {
+        y0 = 0;
+        y1 = N;
+      } else {
+        y0 = min(y0, max(ya, 0));
+        y1 = max(y1, min(yb + 1, N));
+      }
+    }
+    if (y1 > y0) {
+      atomicMin(&zfirst, z);
+      atomicMax(&zlast, z);
+    } else {
+      y0 = y1 = 0;
+    }
+    occ[4 + z] = y0 | (y1 << 16);
+  }
+  const int len = z < N ? y1 - y0 : 0;
+  int sum = len;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, sum, o);
+    if (lane >= o) sum += v;
+  }
+  if (lane == 31) wsum[warp] = sum;
+  __syncthreads();
+  int before = 0;
+  for (int w = 0; w < warp; ++w) before += wsum[w];
+  if (z < N) occ[4 + N + z] = before + sum - len;
+  if (z == N - 1) {
+    occ[0] = before + sum;
+    occ[1] = zlast < 0 ? 0 : zfirst;  // without objects: one plane of zeros
+    occ[2] = zlast < 0 ? 1 : zlast + 1;
+    occ[3] = 0;
   }
 }
 
@@ -574,8 +639,10 @@ cudaError_t launch_tile_prefix(int* bh, int nrows, int ntiles, int* cnt, cudaStr
   return cudaGetLastError();
 }
 
-cudaError_t launch_scan_tiles(const int* cnt, int ntiles, int* off, int* items, cudaStream_t s) {
-  k_scan_tiles<<<1, 1024, 0, s>>>(cnt, ntiles, off, items);
+cudaError_t launch_scan_tiles(const int* cnt, int ntiles, int* off, int* items, cudaStream_t s, const GeomDev& g,
+                              const int* more, int* occ) {
+  k_scan_tiles<<<1, 1024, 0, s>>>(cnt, ntiles, off, items, more, assign_tiles_per_axis(g.N), g.N,
+                                  g.assign == 4 ? kTile + 1 : kTile, g.periodic, occ);
   return cudaGetLastError();
 }
 

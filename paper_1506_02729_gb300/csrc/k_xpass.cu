@@ -33,10 +33,11 @@ template <int N_, int LMAX, bool PO = false>
 __global__ void __launch_bounds__(32 * ((nfields_of(LMAX) + 1) / 2), LMAX < 4 ? 1 : (N_ > 0 && N_ <= 256 ? 4 : 3))
     k_xpass2(
     const unsigned long long* __restrict__ gq, const float* __restrict__ gf, GeomDev g, FftPlan fp,
-    const float2* __restrict__ twg, float2* __restrict__ S1, int nxt, MockBatch mb) {
+    const float2* __restrict__ twg, float2* __restrict__ S1, int nxt, const int* __restrict__ occp, MockBatch mb) {
   if (gq) gq += (long long)blockIdx.z * mb.in;
   if (gf) gf += (long long)blockIdx.z * mb.in;
   S1 += (long long)blockIdx.z * mb.out;
+  if (occp) occp += blockIdx.z * mb.occ;
   constexpr int NF = nfields_of(LMAX);
   constexpr int NP = (NF + 1) / 2;
   constexpr int NTX = 32 * NP;
@@ -58,13 +59,21 @@ __global__ void __launch_bounds__(32 * ((nfields_of(LMAX) + 1) / 2), LMAX < 4 ? 
   // transformed (N <= 512)
   constexpr int NPRE = (512 + NTX - 1) / NTX;
   float pre[NPRE];
-  auto load_row = [&](int row) {
+  // the block's rows of the list of rows that hold objects, as (z, y); the next
+  // one is located while this one is transformed
+  const OccView occ{occp, N};
+  const int nrow = occ.rows();
+  int2 next = make_int2(0, 0);
+  auto load_row = [&](int r) {
+    if (r >= nrow) return;
+    next = occ.row(r);
+    const int row = next.x * N + next.y;
     if constexpr (PO) return;
 #pragma unroll
     for (int j = 0; j < NPRE; ++j) {
       const int x = tid + j * NTX;
       float v = 0.f;
-      if (row < N * N && x < N) {
+      if (x < N) {
         const size_t gi = (size_t)row * N + x;
         v = gq ? (float)(long long)__ldg(gq + gi) * kFixInvF : __ldg(gf + gi);
       }
@@ -72,18 +81,18 @@ __global__ void __launch_bounds__(32 * ((nfields_of(LMAX) + 1) / 2), LMAX < 4 ? 
     }
   };
   load_row(blockIdx.x);
-  for (int row = blockIdx.x; row < N * N; row += gridDim.x) {
-    const int z = row / N, y = row - z * N;
+  for (int r = blockIdx.x; r < nrow; r += gridDim.x) {
+    const int z = next.x, y = next.y;
 #pragma unroll
     for (int j = 0; j < NPRE; ++j) {
       const int x = tid + j * NTX;
       if (x < N) rowF[x] = pre[j];
     }
-    load_row(row + gridDim.x);
+    load_row(r + gridDim.x);
     __syncthreads();
     const float Y = fmaf((float)y, g.H, g.ry), Z = fmaf((float)z, g.H, g.rz);
     if constexpr (PO) {
-      const size_t N3 = (size_t)N * N * N, r0 = (size_t)row * N;
+      const size_t N3 = (size_t)N * N * N, r0 = ((size_t)z * N + y) * N;
       for (int x = tid; x < N; x += NTX) {
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
@@ -162,45 +171,47 @@ static size_t xsm(int N, int NP) { return sizeof(float2) * (N + N / 2 + 2 * (siz
 
 template <int N_, int LMAX, bool PO = false>
 static cudaError_t xrun(const unsigned long long* gq, const float* gf, const GeomDev& g, const FftPlan& fp,
-                        const float2* tw, float2* S1, int nsm, cudaStream_t s, int nxt, int xm, const MockBatch& mb) {
+                        const float2* tw, float2* S1, int nsm, cudaStream_t s, const PassReach& pr, const int* occ, int xm,
+                        const MockBatch& mb) {
   constexpr int NP = (nfields_of(LMAX) + 1) / 2;
   const size_t sm = xsm(g.N, NP);
   raise_smem_limit((const void*)k_xpass2<N_, LMAX, PO>, sm);
-  int occ = 1;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_xpass2<N_, LMAX, PO>, 32 * NP, sm);
-  int grid = nsm * (occ > 0 ? occ : 1) * (xm > 0 ? xm : 2);
+  int resident = 1;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, k_xpass2<N_, LMAX, PO>, 32 * NP, sm);
+  int grid = nsm * (resident > 0 ? resident : 1) * (xm > 0 ? xm : 2);
   if (grid > g.N * g.N) grid = g.N * g.N;
-  k_xpass2<N_, LMAX, PO><<<dim3(grid, 1, mb.n), dim3(NP, 32), sm, s>>>(gq, gf, g, fp, tw, S1, nxt, mb);
+  k_xpass2<N_, LMAX, PO><<<dim3(grid, 1, mb.n), dim3(NP, 32), sm, s>>>(gq, gf, g, fp, tw, S1, pr.nxt, occ, mb);
   return cudaGetLastError();
 }
 
 template <int LMAX>
 static cudaError_t xdispatch(const unsigned long long* gq, const float* gf, const GeomDev& g, const FftPlan& fp,
-                             const float2* tw, float2* S1, int nsm, cudaStream_t s, int nxt, int xm, const MockBatch& mb,
+                             const float2* tw, float2* S1, int nsm, cudaStream_t s, const PassReach& pr, const int* occ, int xm,
+                             const MockBatch& mb,
                              bool po) {
   // the per-object variant: the runtime-size kernel, whatever N
-  if (po) return xrun<0, LMAX, true>(gq, gf, g, fp, tw, S1, nsm, s, nxt, xm, mb);
+  if (po) return xrun<0, LMAX, true>(gq, gf, g, fp, tw, S1, nsm, s, pr, occ, xm, mb);
   if (LMAX == 4) {
     switch (g.N) {
-      case 512: return xrun<512, LMAX>(gq, gf, g, fp, tw, S1, nsm, s, nxt, xm, mb);
-      case 384: return xrun<384, LMAX>(gq, gf, g, fp, tw, S1, nsm, s, nxt, xm, mb);
-      case 360: return xrun<360, LMAX>(gq, gf, g, fp, tw, S1, nsm, s, nxt, xm, mb);
-      case 256: return xrun<256, LMAX>(gq, gf, g, fp, tw, S1, nsm, s, nxt, xm, mb);
-      case 128: return xrun<128, LMAX>(gq, gf, g, fp, tw, S1, nsm, s, nxt, xm, mb);
-      case 64: return xrun<64, LMAX>(gq, gf, g, fp, tw, S1, nsm, s, nxt, xm, mb);
+      case 512: return xrun<512, LMAX>(gq, gf, g, fp, tw, S1, nsm, s, pr, occ, xm, mb);
+      case 384: return xrun<384, LMAX>(gq, gf, g, fp, tw, S1, nsm, s, pr, occ, xm, mb);
+      case 360: return xrun<360, LMAX>(gq, gf, g, fp, tw, S1, nsm, s, pr, occ, xm, mb);
+      case 256: return xrun<256, LMAX>(gq, gf, g, fp, tw, S1, nsm, s, pr, occ, xm, mb);
+      case 128: return xrun<128, LMAX>(gq, gf, g, fp, tw, S1, nsm, s, pr, occ, xm, mb);
+      case 64: return xrun<64, LMAX>(gq, gf, g, fp, tw, S1, nsm, s, pr, occ, xm, mb);
       default: break;
     }
   }
-  return xrun<0, LMAX>(gq, gf, g, fp, tw, S1, nsm, s, nxt, xm, mb);
+  return xrun<0, LMAX>(gq, gf, g, fp, tw, S1, nsm, s, pr, occ, xm, mb);
 }
 
 cudaError_t launch_xpass(const unsigned long long* gq, const float* gf, const GeomDev& g, const MomentTable& mt,
                          const FftPlan& fp, const float2* tw, float2* S1, int nsm, cudaStream_t s,
-                         const PassReach& pr, int xm, MockBatch mb, bool per_object) {
+                         const PassReach& pr, const int* occ, int xm, MockBatch mb, bool per_object) {
   if (per_object && (!gq || gf || mb.n != 1)) return cudaErrorInvalidValue;
-  if (mt.nfields == nfields_of(4)) return xdispatch<4>(gq, gf, g, fp, tw, S1, nsm, s, pr.nxt, xm, mb, per_object);
-  if (mt.nfields == nfields_of(2)) return xdispatch<2>(gq, gf, g, fp, tw, S1, nsm, s, pr.nxt, xm, mb, per_object);
-  return xdispatch<0>(gq, gf, g, fp, tw, S1, nsm, s, pr.nxt, xm, mb, per_object);
+  if (mt.nfields == nfields_of(4)) return xdispatch<4>(gq, gf, g, fp, tw, S1, nsm, s, pr, occ, xm, mb, per_object);
+  if (mt.nfields == nfields_of(2)) return xdispatch<2>(gq, gf, g, fp, tw, S1, nsm, s, pr, occ, xm, mb, per_object);
+  return xdispatch<0>(gq, gf, g, fp, tw, S1, nsm, s, pr, occ, xm, mb, per_object);
 }
 
 }  // namespace fkp

@@ -19,11 +19,12 @@ __global__ void __launch_bounds__(NT, PassShape<NT>::kMinBlocks) k_ypass2(const 
                                                    const unsigned long long* __restrict__ gq,
                                                    const float* __restrict__ gf, GeomDev g, MomentTable mt,
                                                    FftPlan fp, const float2* __restrict__ twg,
-                                                   float2* __restrict__ S2, int* __restrict__ err, int r2, MockBatch mb) {
+                                                   float2* __restrict__ S2, int* __restrict__ err, int r2, const int* __restrict__ occp, MockBatch mb) {
   S1 += (long long)blockIdx.z * mb.in;
   if (gq) gq += (long long)blockIdx.z * mb.in2;
   if (gf) gf += (long long)blockIdx.z * mb.in2;
   S2 += (long long)blockIdx.z * mb.out;
+  if (occp) occp += blockIdx.z * mb.occ;
   extern __shared__ __align__(128) unsigned char smraw[];
   const int N = N_ ? N_ : g.N;
   const int NH = N / 2 + 1, NXT = (NH + kT - 1) / kT;
@@ -38,9 +39,15 @@ __global__ void __launch_bounds__(NT, PassShape<NT>::kMinBlocks) k_ypass2(const 
   // of once per member and thread
   float* coef = reinterpret_cast<float*>(tw + N);
   const int xt = blockIdx.x, z = blockIdx.y;
+  // the plane's rows that hold objects: the others were not written by the
+  // x-pass and are zero; planes outside the occupied range are not read later
+  const OccView occ{occp, N};
+  if (z < occ.z0() || z >= occ.z1()) return;
+  const int2 yr = occ.yrange(z);
+  const unsigned ylen = (unsigned)(yr.y - yr.x);
   const size_t fsz = (size_t)N * NXT * N * kT;
   const size_t gsz = fsz;
-  const uint32_t bytes = (uint32_t)(tile * sizeof(float2));
+  const uint32_t bytes = ylen * (uint32_t)(kT * sizeof(float2));
   const int tid = threadIdx.y * kT + threadIdx.x;
   for (int i = tid; i < N; i += NT) tw[i] = twg[i];
   if (tid == 0) {
@@ -62,10 +69,10 @@ __global__ void __launch_bounds__(NT, PassShape<NT>::kMinBlocks) k_ypass2(const 
     coef[e] = v;
   }
   __syncthreads();
-  auto src_of = [&](int q) { return S1 + (size_t)q * fsz + ((size_t)z * NXT + xt) * tile; };
-  if (tid == 0) {
+  auto src_of = [&](int q) { return S1 + (size_t)q * fsz + ((size_t)z * NXT + xt) * tile + yr.x * kT; };
+  if (tid == 0 && ylen) {
     mbar_expect_tx(&bar[0], bytes);
-    tma_load_1d(buf0, src_of(mt.s_field[0][0]), bytes, &bar[0]);
+    tma_load_1d(buf0 + yr.x * kT, src_of(mt.s_field[0][0]), bytes, &bar[0]);
   }
   const int c = threadIdx.x, run = threadIdx.y;
   const int rl = (N + PassShape<NT>::kRun - 1) / PassShape<NT>::kRun;
@@ -83,12 +90,12 @@ __global__ void __launch_bounds__(NT, PassShape<NT>::kMinBlocks) k_ypass2(const 
     for (int m = 0; m < mt.s_nmem[sw]; ++m, ++it) {
       const int cur = it & 1;
       float2* bc = cur ? buf1 : buf0;
-      if (tid == 0 && it + 1 < total) {
+      if (tid == 0 && ylen && it + 1 < total) {
         int s2 = sw, m2 = m + 1;
         if (m2 == mt.s_nmem[sw]) { s2 = sw + 1; m2 = 0; }
         fence_proxy_async();
         mbar_expect_tx(&bar[cur ^ 1], bytes);
-        tma_load_1d(cur ? buf0 : buf1, src_of(mt.s_field[s2][m2]), bytes, &bar[cur ^ 1]);
+        tma_load_1d((cur ? buf0 : buf1) + yr.x * kT, src_of(mt.s_field[s2][m2]), bytes, &bar[cur ^ 1]);
       }
       // coefficients a[o][j] of n_y^j for this member and column
       float a[2][5];
@@ -110,13 +117,14 @@ __global__ void __launch_bounds__(NT, PassShape<NT>::kMinBlocks) k_ypass2(const 
           acc1[i].y = fmaf(s1, v.y, acc1[i].y);
         }
       };
+      if (ylen == 0) continue;  // a plane without objects inside the range: zeros
       mbar_wait(&bar[cur], (uint32_t)((it >> 1) & 1), err, 4);
       if constexpr (fft_fusable<N_, kT, NT>()) {
         // the last FFT stage's butterflies produce exactly this thread's k_y
         // (y + i kRun): they are summed from registers, never stored
-        fft_ct_fused<N_, kT, NT, -1, false, false>(bc, work, tw, accumulate);
+        fft_ct_fused<N_, kT, NT, -1, false, false, true>(bc, work, tw, accumulate, yr.x, ylen);
       } else {
-        const float2* R = fft_any<N_, kT, NT, -1>(bc, work, fp, tw);
+        const float2* R = fft_any<N_, kT, NT, -1, false, false, true>(bc, work, fp, tw, yr.x, ylen);
 #pragma unroll
         for (int i = 0; i < PassShape<NT>::kRL; ++i) {
           const int ky = i * PassShape<NT>::kRun + run;
@@ -164,36 +172,36 @@ __global__ void __launch_bounds__(NT, PassShape<NT>::kMinBlocks) k_ypass2(const 
 template <int N_, int NT>
 static cudaError_t yrun_nt(const float2* S1, const unsigned long long* gq, const float* gf, const GeomDev& g,
                            const MomentTable& mt, const FftPlan& fp, const float2* tw, float2* S2, int* err,
-                           cudaStream_t s, const PassReach& pr, const MockBatch& mb) {
+                           cudaStream_t s, const PassReach& pr, const int* occ, const MockBatch& mb) {
   int total = 0;
   for (int q = 0; q < mt.nsweeps; ++q) total += mt.s_nmem[q];
   const size_t sm = ysm(g.N) + sizeof(float) * 10 * kT * (size_t)total;
   raise_smem_limit((const void*)k_ypass2<N_, NT>, sm);
   k_ypass2<N_, NT><<<dim3(pr.nxt, g.N, mb.n), dim3(kT, NT / kT), sm, s>>>(S1, gq, gf, g, mt, fp, tw, S2, err, pr.r2,
-                                                                              mb);
+                                                                              occ, mb);
   return cudaGetLastError();
 }
 
 template <int N_>
 static cudaError_t yrun(const float2* S1, const unsigned long long* gq, const float* gf, const GeomDev& g,
                         const MomentTable& mt, const FftPlan& fp, const float2* tw, float2* S2, int* err,
-                        cudaStream_t s, const PassReach& pr, int nt, const MockBatch& mb) {
-  return nt == 512 ? yrun_nt<N_, 512>(S1, gq, gf, g, mt, fp, tw, S2, err, s, pr, mb)
-                   : yrun_nt<N_, 256>(S1, gq, gf, g, mt, fp, tw, S2, err, s, pr, mb);
+                        cudaStream_t s, const PassReach& pr, const int* occ, int nt, const MockBatch& mb) {
+  return nt == 512 ? yrun_nt<N_, 512>(S1, gq, gf, g, mt, fp, tw, S2, err, s, pr, occ, mb)
+                   : yrun_nt<N_, 256>(S1, gq, gf, g, mt, fp, tw, S2, err, s, pr, occ, mb);
 }
 
 // gq / gf: the grid the x-pass read (for the observer node's value).
 cudaError_t launch_ypass(const float2* S1, const unsigned long long* gq, const float* gf, const GeomDev& g,
                          const MomentTable& mt, const FftPlan& fp, const float2* tw, float2* S2, int* err,
-                         cudaStream_t s, const PassReach& pr, int nt, MockBatch mb) {
+                         cudaStream_t s, const PassReach& pr, const int* occ, int nt, MockBatch mb) {
   switch (g.N) {
-    case 512: return yrun<512>(S1, gq, gf, g, mt, fp, tw, S2, err, s, pr, nt, mb);
-    case 384: return yrun<384>(S1, gq, gf, g, mt, fp, tw, S2, err, s, pr, nt, mb);
-    case 360: return yrun<360>(S1, gq, gf, g, mt, fp, tw, S2, err, s, pr, nt, mb);
-    case 256: return yrun<256>(S1, gq, gf, g, mt, fp, tw, S2, err, s, pr, nt, mb);
-    case 128: return yrun<128>(S1, gq, gf, g, mt, fp, tw, S2, err, s, pr, nt, mb);
-    case 64: return yrun<64>(S1, gq, gf, g, mt, fp, tw, S2, err, s, pr, nt, mb);
-    default: return yrun<0>(S1, gq, gf, g, mt, fp, tw, S2, err, s, pr, nt, mb);
+    case 512: return yrun<512>(S1, gq, gf, g, mt, fp, tw, S2, err, s, pr, occ, nt, mb);
+    case 384: return yrun<384>(S1, gq, gf, g, mt, fp, tw, S2, err, s, pr, occ, nt, mb);
+    case 360: return yrun<360>(S1, gq, gf, g, mt, fp, tw, S2, err, s, pr, occ, nt, mb);
+    case 256: return yrun<256>(S1, gq, gf, g, mt, fp, tw, S2, err, s, pr, occ, nt, mb);
+    case 128: return yrun<128>(S1, gq, gf, g, mt, fp, tw, S2, err, s, pr, occ, nt, mb);
+    case 64: return yrun<64>(S1, gq, gf, g, mt, fp, tw, S2, err, s, pr, occ, nt, mb);
+    default: return yrun<0>(S1, gq, gf, g, mt, fp, tw, S2, err, s, pr, occ, nt, mb);
   }
 }
 

@@ -78,7 +78,12 @@ __global__ void __launch_bounds__(NT, PassShape<NT>::kMinBlocks) k_zpass2(const 
   const int tid = threadIdx.y * kT + threadIdx.x;
   const int ntiles = pr.nzt;
   const size_t gsz = (size_t)N * NXT * N * kT;
-  const uint32_t bytes = (uint32_t)(tile * sizeof(float2));
+  // the occupied planes [zs, zs + zl) of the grid (and of the second of an
+  // interlaced pair): the y-pass wrote those, the others are zero
+  const OccView oc1{zp.occ ? zp.occ + blockIdx.z * mb.occ : nullptr, N};
+  const OccView oc2{zp.interlace ? zp.occ2 : nullptr, N};
+  const int zs1 = oc1.z0(), zs2 = oc2.z0();
+  const unsigned zl1 = (unsigned)(oc1.z1() - zs1), zl2 = (unsigned)(oc2.z1() - zs2);
   for (int i = tid; i < N; i += NT) {
     tw[i] = twg[i];
     zph[i] = zp.interlace ? zp.hph[i] : make_float2(1.f, 0.f);
@@ -107,10 +112,16 @@ __global__ void __launch_bounds__(NT, PassShape<NT>::kMinBlocks) k_zpass2(const 
   auto src_of = [&](int id, int gi) {
     return S2 + (size_t)gi * gsz + ((size_t)(id & 63) * N + (id >> 6)) * tile;
   };
+  auto fetch = [&](int id, int gi, float2* dst, uint64_t* b) {
+    const bool second = gi >= mt.ngroups;
+    const int zs = (second ? zs2 : zs1) * kT;
+    const uint32_t bytes = (second ? zl2 : zl1) * (uint32_t)(kT * sizeof(float2));
+    mbar_expect_tx(b, bytes);
+    tma_load_1d(dst + zs, src_of(id, gi) + zs, bytes, b);
+  };
   int id = (int)blockIdx.x < ntiles ? __ldg(pr.ztiles + blockIdx.x) : 0;
   if (tid == 0 && (int)blockIdx.x < ntiles) {
-    mbar_expect_tx(&bar[0], bytes);
-    tma_load_1d(buf0, src_of(id, 0), bytes, &bar[0]);
+    fetch(id, 0, buf0, &bar[0]);
   }
   const int c = threadIdx.x, run = threadIdx.y;
   const int rl = (N + PassShape<NT>::kRun - 1) / PassShape<NT>::kRun;
@@ -141,12 +152,12 @@ __global__ void __launch_bounds__(NT, PassShape<NT>::kMinBlocks) k_zpass2(const 
       const int gn = gi + 1 < ngt ? gi + 1 : 0;
       if (tn >= 0) {
         fence_proxy_async();
-        mbar_expect_tx(&bar[cur ^ 1], bytes);
-        tma_load_1d(cur ? buf0 : buf1, src_of(tn, gn), bytes, &bar[cur ^ 1]);
+        fetch(tn, gn, cur ? buf0 : buf1, &bar[cur ^ 1]);
       }
     }
     mbar_wait(&bar[cur], (uint32_t)((it >> 1) & 1), err, 8);
-    const float2* R = fft_any<N_, kT, NT, -1, false, true>(bc, work, fp, tw);
+    const float2* R = fft_any<N_, kT, NT, -1, false, true, true>(bc, work, fp, tw, gi < mt.ngroups ? zs1 : zs2,
+                                                                gi < mt.ngroups ? zl1 : zl2);
     const int gg = gi < mt.ngroups ? gi : gi - mt.ngroups;  // the group's coefficients
     // second grid of an interlaced pair: its half-cell phase
     // e^{-i pi (n_x + n_y + n_z)/N}, the n_x, n_y part fixed per thread

@@ -1,0 +1,107 @@
+"""GPU: the FFT passes walk only the rows and planes that hold objects.  Small
+clouds of objects at chosen places of the box give the P_l of the FP64 oracle,
+whatever rows they leave empty."""
+import math
+
+import numpy as np
+import pytest
+
+import mockgen
+from oracle import power as op
+from tests.helpers import P_TOL, p_errors, to_device
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+L = 960.0
+
+
+def _cloud(boxes, n, seed):
+    g = np.random.default_rng(seed)
+    pos = np.concatenate([lo + (hi - lo) * g.random((n, 3)) for lo, hi in
+                          ((np.array(a, float), np.array(b, float)) for a, b in boxes)])
+    nb = np.full(len(pos), 1e-4)
+    return {k: pos[:, i].astype(np.float32) for i, k in enumerate("xyz")} | {"nbar": nb.astype(np.float32)}
+
+
+def _cell(*ijk, N):
+    return [np.array(v, float) * (L / N) for v in ijk]
+
+
+# boxes in cells: [lo, hi) per axis (x, y, z)
+PLACES = {
+    "one_tile": [((20, 20, 20), (28, 28, 28))],
+    "tile_edges": [((15.4, 31.5, 31.5), (16.6, 32.6, 32.6))],       # taps reach into the next tiles and planes
+    "two_planes_a_gap_between": [((10, 10, 6), (14, 14, 9)), ((30, 40, 50), (34, 44, 53))],
+    "low_corner": [((2.6, 2.6, 2.6), (5, 5, 5))],
+    "high_corner": [((51, 51, 51), (55, 55, 55))],
+}
+
+
+@pytest.mark.parametrize("place", sorted(PLACES))
+@pytest.mark.parametrize("N,assign,interlace", [(64, 2, False), (60, 3, False), (64, 4, False), (64, 4, True)],
+                         ids=["cic", "tsc_runtime", "pcs", "pcs_interlaced"])
+def test_empty_rows(place, N, assign, interlace):
+    import paper_1506_02729_gb300 as fkp
+    boxes = [_cell(a, b, N=64) for a, b in PLACES[place]]
+    gal, ran = _cloud(boxes, 200, 1), _cloud(boxes, 1500, 2)
+    geom = dict(L=L, N=N, assign=assign, origin=(0.0, 0.0, 0.0), observer=(480.0, 480.0, 480.0), P_fkp=1e4,
+                interlace=interlace)
+    kf = 2 * math.pi / L
+    bins = (0.5 * kf, kf, 24)
+    ref = op.power(gal, ran, geom, bins)
+    plan = fkp.Plan(geom, bins)
+    g, r = to_device(gal), to_device(ran)
+    got = plan.power(g, r)
+    assert np.array_equal(got["nmodes"], ref["nmodes"])
+    assert max(p_errors(got, ref).values()) < P_TOL, p_errors(got, ref)
+    # galaxies and the cached randoms in different places: both occupy rows
+    other = _cloud([_cell((34, 8, 40), (40, 12, 44), N=64)], 300, 3)
+    ref = op.power(other, ran, geom, bins)
+    plan.cache_randoms(r)
+    got = plan.power(to_device(other), None)
+    assert max(p_errors(got, ref).values()) < P_TOL, p_errors(got, ref)
+    # the next mock on the same buffers: nothing of the last one's rows is left
+    ref = op.power(gal, ran, geom, bins)
+    got = plan.power(g, None)
+    assert max(p_errors(got, ref).values()) < P_TOL, p_errors(got, ref)
+
+
+@pytest.mark.parametrize("lo", [(0.0, 0.0, 0.0), (-3.0, 61.0, 30.0), (62.5, 30.0, -1.0)])
+@pytest.mark.parametrize("N,assign", [(64, 3), (60, 4), (90, 2)])
+def test_periodic_wrap(lo, N, assign):
+    """Taps that wrap around the box reach the rows and planes of the far side."""
+    import paper_1506_02729_gb300 as fkp
+    box = [_cell(lo, tuple(v + 3.0 for v in lo), N=64)]
+    gal, ran = _cloud(box, 200, 4), _cloud(box, 1500, 5)
+    geom = dict(L=L, N=N, assign=assign, origin=(0.0, 0.0, 0.0), observer=(480.0, 480.0, 480.0), P_fkp=1e4,
+                periodic=True)
+    kf = 2 * math.pi / L
+    plan = fkp.Plan(geom, (0.5 * kf, kf, 24))
+    g, r = to_device(gal), to_device(ran)
+    got = plan.power(g, r)
+    # the same field handed in whole, where the passes take every row: the
+    # same arithmetic on the same values, so the same bits
+    F = torch.from_numpy(plan.grid(g, r).astype(np.float32) * np.float32(2.0 ** -40)).cuda()
+    ref = plan.power_from_grid(F, got["I22"], got["N0"])
+    for k in ("P0", "P2", "P4", "P4b", "nmodes"):
+        assert np.array_equal(got[k], ref[k], equal_nan=True), k
+
+
+def test_batch_of_mocks_in_different_places():
+    """Each mock of a fused batch has its own rows: the batch equals single calls."""
+    import paper_1506_02729_gb300 as fkp
+    N = 64
+    geom = dict(L=L, N=N, assign=3, origin=(0.0, 0.0, 0.0), observer=(480.0, 480.0, 480.0), P_fkp=1e4)
+    kf = 2 * math.pi / L
+    plan = fkp.Plan(geom, (0.5 * kf, kf, 24))
+    ms = []
+    for i, p in enumerate(sorted(PLACES)):
+        boxes = [_cell(a, b, N=64) for a, b in PLACES[p]]
+        ms.append((to_device(_cloud(boxes, 100, 10 + i)), to_device(_cloud(boxes, 900, 20 + i))))
+    got = plan.power_batch([g for g, _ in ms], [r for _, r in ms])
+    for (g, r), b in zip(ms, got):
+        one = plan.power(g, r)
+        for k in ("P0", "P2", "P4", "P4b"):
+            assert np.array_equal(b[k], one[k], equal_nan=True), k
