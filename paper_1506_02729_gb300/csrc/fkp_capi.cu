@@ -721,10 +721,13 @@ static int grid_pass(Plan* P, const CatDev& gal, const CatDev& ran, cudaStream_t
     P->sort_cap = cap;
   }
   // one 1024-thread block per SM for the binning kernels (their shared
-  // histogram spans every tile)
+  // histogram spans every tile), shared out between the catalogs by size
   const int nb = P->ctx->nsm;
-  auto nblocks = [&](long long n) { return (int)std::max<long long>(1, std::min<long long>(nb, (n + 4095) / 4096)); };
-  const int nbg = nblocks(gal.n), nbr = cached ? P->rc_nblk : nblocks(ran.n);
+  auto nblocks = [&](long long n, long long most) {
+    return (int)std::max<long long>(1, std::min<long long>(most, (n + 2047) / 2048));
+  };
+  const long long share = cached ? nb : std::max<long long>(1, std::min<long long>(nb - 1, nb * gal.n / std::max<long long>(1, ntot)));
+  const int nbg = nblocks(gal.n, share), nbr = cached ? P->rc_nblk : nblocks(ran.n, nb - share);
   const long long nran = cached ? P->rc_n : ran.n;
   if (!which) CK(cudaMemsetAsync(P->d_err, 0, sizeof(int) * 4, s));
   CK(stage(0));
@@ -735,33 +738,26 @@ static int grid_pass(Plan* P, const CatDev& gal, const CatDev& ran, cudaStream_t
   CK(cudaMemsetAsync(grid, 0, N3 * 8 * ngrid, P->side));
   if (gridw) CK(cudaMemsetAsync(gridw, 0, N3 * 8, P->side));
   CK(cudaEventRecord(P->ev_join, P->side));
-  int* bh_ran = P->d_bhist + (size_t)nbg * P->ntiles;
-  CK(launch_bin_count(gal, 0, geo, P->d_scpart, P->d_bhist, P->d_err, nbg, s));
+  const int nbx = cached ? 0 : nbr;  // blocks that read randoms
+  CK(launch_bin_count(gal, ran, nbg, nbx, geo, P->d_scpart, P->d_bhist, P->d_err, s));
   if (cached)
     CK(cudaMemcpyAsync(P->d_scpart + (size_t)nbg * SC_NSUM, P->rc_part, sizeof(double) * SC_NSUM * nbr,
                        cudaMemcpyDeviceToDevice, s));
-  else
-    CK(launch_bin_count(ran, 1, geo, P->d_scpart + (size_t)nbg * SC_NSUM, bh_ran, P->d_err, nbr, s));
-  CK(launch_scalars_finalize(P->d_scpart, nbg, nbr, gal.n, nran, geo.alpha_mode, P->d_ds, s));
-  CK(launch_tile_prefix(P->d_bhist, nbg + (cached ? 0 : nbr), P->ntiles, P->d_tcnt, s));
-  CK(launch_scan_tiles(P->d_tcnt, P->ntiles, P->d_toff, P->d_titem, s, geo,
+  CK(launch_tile_prefix(P->d_bhist, nbg + nbx, P->ntiles, P->d_tcnt, P->d_scpart, nbg, nbr, gal.n, nran,
+                        geo.alpha_mode, P->d_ds, s));
+  const int chunk = accum_chunk(ntot * ngrid, nb);
+  CK(launch_scan_tiles(P->d_tcnt, P->ntiles, P->d_toff, P->d_titem, chunk, s, geo,
                        cached ? (which ? P->rc_tcnt2 : P->rc_tcnt) : nullptr, which ? P->d_occ2 : P->d_occ));
   CK(stage(1));
   CK(cudaStreamWaitEvent(s, P->ev_join, 0));
-  const double* obs = P->geom.observer;
   float* vw2 = gridw ? P->d_vw2 : nullptr;
-  CK(launch_bin_scatter(gal, 0, geo, obs, P->d_ds, P->d_toff, P->d_bhist, P->d_xyzv, vw2, nullptr, nbg, s));
-  if (cached) {
+  CK(launch_bin_scatter(gal, ran, nbg, nbx, geo, P->geom.observer, P->d_ds, P->d_toff, P->d_bhist, P->d_xyzv, vw2,
+                        P->d_labpart, s));
+  if (cached)
     CK(cudaMemcpyAsync(P->d_ds + DS_COUNT, P->rc_lab, sizeof(double) * LAB_NSUM, cudaMemcpyDeviceToDevice, s));
-  } else {
-    CK(launch_bin_scatter(ran, 1, geo, obs, P->d_ds, P->d_toff, bh_ran, P->d_xyzv, vw2, P->d_labpart, nbr, s));
-    CK(launch_lab_finalize(P->d_labpart, ran.n > 0 ? nbr : 0, P->d_ds + DS_COUNT, s));
-  }
-  CK(launch_tile_accum(geo, P->d_toff, P->d_titem, gal.n + (cached ? 0 : ran.n), P->d_xyzv, vw2, grid, gridw, s));
   // per-object line of sight: moment field q grids w x^^e[q] with each object's x^
-  for (int q = 1; q < ngrid; ++q)
-    CK(launch_tile_accum(geo, P->d_toff, P->d_titem, gal.n + ran.n, P->d_xyzv, nullptr, grid + (size_t)q * N3,
-                         nullptr, s, P->mt.e[q]));
+  CK(launch_tile_accum(geo, P->d_toff, P->d_titem, ntot, chunk, P->d_xyzv, vw2, grid, gridw, s,
+                       P->per_object ? &P->mt : nullptr, P->d_labpart, nbr, cached ? nullptr : P->d_ds + DS_COUNT));
   if (cached)
     CK(launch_combine_randoms(grid, rgrid, gridw, rgridw, P->d_ds, (long long)N3, P->ctx->nsm, s));
   return FKP_OK;
@@ -794,7 +790,7 @@ static int cache_randoms(Plan* P, const CatDev& ran, cudaStream_t s) {
   if (ran.n == 0) return FKP_OK;
   if (ran.n >= (1ll << 31)) return set_error(FKP_EINVAL, "at most 2^31-1 randoms");
   const int nb = P->ctx->nsm;
-  const int nbr = (int)std::max<long long>(1, std::min<long long>(nb, (ran.n + 4095) / 4096));
+  const int nbr = (int)std::max<long long>(1, std::min<long long>(nb, (ran.n + 2047) / 2048));
   if (!P->rc_grid) {
     P->rc_grid = (unsigned long long*)P->alloc(N3 * 8);
     if (P->d_gridw) P->rc_gridw = (unsigned long long*)P->alloc(N3 * 8);
@@ -828,16 +824,17 @@ static int cache_randoms(Plan* P, const CatDev& ran, cudaStream_t s) {
     const GeomDev& geo = which ? P->g2 : P->g;
     unsigned long long* rg = which ? P->rc_grid2 : P->rc_grid;
     unsigned long long* rgw = which ? P->rc_gridw2 : P->rc_gridw;
-    CK(launch_bin_count(ran, 1, geo, P->rc_part, P->d_bhist, P->d_err, nbr, s));
-    CK(launch_tile_prefix(P->d_bhist, nbr, P->ntiles, P->d_tcnt, s));
-    CK(launch_scan_tiles(P->d_tcnt, P->ntiles, P->d_toff, P->d_titem, s, geo, nullptr, nullptr));
+    CK(launch_bin_count(ran, ran, 0, nbr, geo, P->rc_part, P->d_bhist, P->d_err, s));
+    CK(launch_tile_prefix(P->d_bhist, nbr, P->ntiles, P->d_tcnt, nullptr, 0, 0, 0, 0, 0, nullptr, s));
+    const int chunk = accum_chunk(ran.n, nb);
+    CK(launch_scan_tiles(P->d_tcnt, P->ntiles, P->d_toff, P->d_titem, chunk, s, geo, nullptr, nullptr));
     CK(cudaMemcpyAsync(which ? P->rc_tcnt2 : P->rc_tcnt, P->d_tcnt, sizeof(int) * P->ntiles, cudaMemcpyDeviceToDevice, s));
     CK(cudaMemsetAsync(rg, 0, N3 * 8, s));
     if (rgw) CK(cudaMemsetAsync(rgw, 0, N3 * 8, s));
-    CK(launch_bin_scatter(ran, 1, geo, P->geom.observer, P->d_ds, P->d_toff, P->d_bhist, P->d_xyzv, vw2, P->d_labpart, nbr, s,
-                          1));
-    CK(launch_lab_finalize(P->d_labpart, nbr, P->rc_lab, s));
-    CK(launch_tile_accum(geo, P->d_toff, P->d_titem, ran.n, P->d_xyzv, vw2, rg, rgw, s));
+    CK(launch_bin_scatter(ran, ran, 0, nbr, geo, P->geom.observer, P->d_ds, P->d_toff, P->d_bhist, P->d_xyzv, vw2,
+                          P->d_labpart, s, 1));
+    CK(launch_tile_accum(geo, P->d_toff, P->d_titem, ran.n, chunk, P->d_xyzv, vw2, rg, rgw, s, nullptr, P->d_labpart,
+                         nbr, P->rc_lab));
   }
   int herr = 0;
   CK(cudaMemcpyAsync(&herr, P->d_err, sizeof(int), cudaMemcpyDeviceToHost, s));

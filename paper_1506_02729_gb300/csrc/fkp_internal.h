@@ -168,28 +168,26 @@ int yz_tiles(int N);
 int tiles_x(int N);
 bool moments_match(const MomentTable& mt);
 size_t field_elems(int N);
-cudaError_t launch_scalars_finalize(const double* part, int nbg, int nbr, long long ng, long long nr, int amode,
-                                    double* ds, cudaStream_t s);
 int assign_tiles_per_axis(int N);
-cudaError_t launch_bin_count(const CatDev& c, int is_ran, const GeomDev& g, double* part, int* bh, int* err,
-                             int nblk, cudaStream_t s);
-cudaError_t launch_tile_prefix(int* bh, int nrows, int ntiles, int* cnt, cudaStream_t s);
+cudaError_t launch_bin_count(const CatDev& gal, const CatDev& ran, int nbg, int nbr, const GeomDev& g, double* part,
+                             int* bh, int* err, cudaStream_t s);
+cudaError_t launch_tile_prefix(int* bh, int nrows, int ntiles, int* cnt, const double* part, int nbg, int nbr,
+                               long long ng, long long nr, int alpha_mode, double* ds, cudaStream_t s);
+int accum_chunk(long long nobj, int nsm);
 // occ: NULL, or the plan's list of occupied rows; more: NULL, or the tile
 // counts of a cached random catalog.
-cudaError_t launch_scan_tiles(const int* cnt, int ntiles, int* off, int* items, cudaStream_t s, const GeomDev& g,
-                              const int* more, int* occ);
-cudaError_t launch_bin_scatter(const CatDev& c, int is_ran, const GeomDev& g, const double obs[3], const double* ds,
-                               const int* off, const int* bpref, float4* xyzv, float* vw2, double* labpart, int nblk,
-                               cudaStream_t s, int raw = 0);
+cudaError_t launch_scan_tiles(const int* cnt, int ntiles, int* off, int* items, int chunk, cudaStream_t s,
+                              const GeomDev& g, const int* more, int* occ);
+cudaError_t launch_bin_scatter(const CatDev& gal, const CatDev& ran, int nbg, int nbr, const GeomDev& g,
+                               const double obs[3], const double* ds, const int* off, const int* bpref, float4* xyzv,
+                               float* vw2, double* labpart, cudaStream_t s, int raw = 0);
 cudaError_t launch_combine_randoms(unsigned long long* grid, const unsigned long long* rgrid,
                                    unsigned long long* gridw, const unsigned long long* rgridw, const double* ds,
                                    long long n, int nsm, cudaStream_t s);
-// xe: NULL, or the exponents (a, b, c) of a moment field: each object's value
-// is then multiplied by x^_x^a x^_y^b x^_z^c of its own line of sight.
-cudaError_t launch_tile_accum(const GeomDev& g, const int* off, const int* items, long long nobj, const float4* xyzv,
-                              const float* vw2, unsigned long long* grid, unsigned long long* gridw, cudaStream_t s,
-                              const unsigned char* xe = nullptr);
-cudaError_t launch_lab_finalize(const double* labpart, int nblk, double* out, cudaStream_t s);
+cudaError_t launch_tile_accum(const GeomDev& g, const int* off, const int* items, long long nobj, int chunk,
+                              const float4* xyzv, const float* vw2, unsigned long long* grid,
+                              unsigned long long* gridw, cudaStream_t s, const MomentTable* mt,
+                              const double* labpart, int nlab, double* lab);
 cudaError_t launch_wait_selftest(unsigned polls, int* flag, cudaStream_t s);
 // xm: x-pass blocks = SMs x resident blocks x xm; nt: threads per y- or
 // z-pass block (256 or 512).  The defaults are the 512^3 choices.  mb: the

@@ -84,23 +84,29 @@ __device__ __forceinline__ int tile_of(int cx, int cy, int cz, int N, int ntx) {
 
 // ---------------------------------------------------------------------------
 
-// Each block owns a contiguous chunk of objects (the same chunks as the
-// scatter launch on the same catalog): its counts go to a shared-memory
-// histogram over all tiles, written out whole as the block's row of bh.
+// One launch for both catalogs: the first nbg blocks take the galaxies, the
+// others the randoms (a launch for the galaxies alone leaves most SMs idle:
+// 2e4 galaxies and 2e5 randoms took 19 + 26 us one after the other).  Each
+// block owns a contiguous chunk of objects (the same chunks as the scatter
+// launch on the same catalogs): its counts go to a shared-memory histogram
+// over all tiles, written out whole as the block's row of bh.
 constexpr int kBinThreads = 1024;
 
 template <int P>
-__global__ void __launch_bounds__(kBinThreads) k_bin_count(CatDev c, int is_ran, GeomDev g, int ntx, int ntiles,
-                                                           double* __restrict__ part, int* __restrict__ bh,
-                                                           int* __restrict__ err) {
+__global__ void __launch_bounds__(kBinThreads) k_bin_count(CatDev cg, CatDev cr, int nbg, GeomDev g, int ntx,
+                                                           int ntiles, double* __restrict__ part,
+                                                           int* __restrict__ bh, int* __restrict__ err) {
+  const int is_ran = (int)blockIdx.x >= nbg;
+  const CatDev& c = is_ran ? cr : cg;
   extern __shared__ int hist[];
   __shared__ double sh[32];
   for (int t = threadIdx.x; t < ntiles; t += blockDim.x) hist[t] = 0;
   __syncthreads();
   FFSum s_w, s_w2, s_w3, s_nw2, s_n2w3;
   bool bad = false;
-  const long long chunk = (c.n + gridDim.x - 1) / gridDim.x;
-  const long long i0 = blockIdx.x * chunk;
+  const int nblk = is_ran ? (int)gridDim.x - nbg : nbg, blk = is_ran ? (int)blockIdx.x - nbg : (int)blockIdx.x;
+  const long long chunk = (c.n + nblk - 1) / nblk;
+  const long long i0 = blk * chunk;
   const long long i1 = i0 + chunk < c.n ? i0 + chunk : c.n;
   // unrolled: the loads of several objects in flight at once
 #pragma unroll 4
@@ -141,31 +147,72 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_count(CatDev c, int is_ran,
   }
 }
 
-// Per tile t, over the rows of bh (one per block of the count launches,
+// Per tile t, over the rows of bh (one per block of the count launch,
 // galaxies' blocks first): each row's entry becomes the exclusive prefix of
-// the rows above it, and cnt[t] the tile's total.  Rows are read in batches
-// of 16 independent loads.
+// the rows above it, and cnt[t] the tile's total.  A block takes 32 tiles (one
+// 128-byte line per row) and cuts the rows among its 8 warps: 512^3, 304 rows
+// of 32,768 tiles, 37 us with one thread per tile.
+// The last block forms the scalars instead (ds not null): alpha, I_22, I_33,
+// N_0, S_3 from the count blocks' FP64 partial sums, warp q the sum of
+// quantity q in a fixed order (galaxy blocks [0, nbg), random blocks [nbg,
+// nbg + nbr)); one thread per sum took 17 us.
 __global__ void __launch_bounds__(256) k_tile_prefix(int* __restrict__ bh, int nrows, int ntiles,
-                                                     int* __restrict__ cnt) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+                                                     int* __restrict__ cnt, const double* __restrict__ part, int nbg,
+                                                     int nbr, long long ng, long long nr, int alpha_mode,
+                                                     double* __restrict__ ds) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (ds && blockIdx.x == gridDim.x - 1) {
+    __shared__ double tot[SC_NSUM];
+    static_assert(SC_NSUM == 8, "one warp per sum");
+    const bool gal = w <= SC_G_W3;
+    const int b0 = gal ? 0 : nbg, nb = gal ? nbg : nbr;
+    double v = 0.0;
+    for (int b = lane; b < nb; b += 32) v += part[(size_t)(b0 + b) * SC_NSUM + w];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (lane == 0) tot[w] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      const double Wg = tot[SC_G_W], Wr = tot[SC_R_W];
+      const double a = alpha_mode == 0 ? Wg / Wr : (double)ng / (double)nr;
+      ds[DS_ALPHA] = a;
+      ds[DS_I22] = a * tot[SC_R_NW2];
+      ds[DS_I33] = a * tot[SC_R_N2W3];
+      ds[DS_N0] = tot[SC_G_W2] + a * a * tot[SC_R_W2];
+      ds[DS_N0FKP] = a * (1.0 + a) * tot[SC_R_W2];
+      ds[DS_S3] = tot[SC_G_W3] - a * a * a * tot[SC_R_W3];
+      ds[DS_WG] = Wg;
+      ds[DS_WR] = Wr;
+      ds[DS_NG] = (double)ng;
+      ds[DS_NR] = (double)nr;
+    }
+    return;
+  }
+  __shared__ int sum[8][32];
+  const int t = blockIdx.x * 32 + lane;
+  const int per = (nrows + 7) / 8, r0 = w * per, r1 = min(nrows, r0 + per);
+  int s = 0;
+  if (t < ntiles) {
+#pragma unroll 8
+    for (int q = r0; q < r1; ++q) s += bh[(size_t)q * ntiles + t];
+  }
+  sum[w][lane] = s;
+  __syncthreads();
   if (t >= ntiles) return;
   int run = 0;
-  for (int r0 = 0; r0 < nrows; r0 += 16) {
-    int v[16];
-#pragma unroll
-    for (int q = 0; q < 16; ++q) v[q] = r0 + q < nrows ? bh[(size_t)(r0 + q) * ntiles + t] : 0;
-#pragma unroll
-    for (int q = 0; q < 16; ++q) {
-      if (r0 + q < nrows) bh[(size_t)(r0 + q) * ntiles + t] = run;
-      run += v[q];
-    }
+  for (int k = 0; k < w; ++k) run += sum[k][lane];
+  if (w == 7) cnt[t] = run + s;
+#pragma unroll 8
+  for (int q = r0; q < r1; ++q) {
+    const int v = bh[(size_t)q * ntiles + t];
+    bh[(size_t)q * ntiles + t] = run;
+    run += v;
   }
-  cnt[t] = run;
 }
 
 // Exclusive scan of the tile counts into offsets (off[ntiles] = total), and
 // of the tiles' work items (one per
-// kAccumChunk objects or part of it) into item offsets (items[ntiles] = the
+// chunk objects or part of it) into item offsets (items[ntiles] = the
 // number of items).  One block of 1024 threads walks the tiles in rounds of
 // 1024 (coalesced loads, the next round's counts loaded during this round's
 // warp-shuffle scan).
@@ -174,7 +221,7 @@ __global__ void __launch_bounds__(256) k_tile_prefix(int* __restrict__ bh, int n
 // counts, or null) says so: a tile's objects reach its cells, one cell below
 // and reach - kTile + 1 above, wrapped around a periodic box.
 __global__ void __launch_bounds__(1024) k_scan_tiles(const int* __restrict__ cnt, int ntiles, int* __restrict__ off,
-                                                     int* __restrict__ items, const int* __restrict__ more, int ntx,
+                                                     int* __restrict__ items, int chunk, const int* __restrict__ more, int ntx,
                                                      int N, int reach, int periodic, int* __restrict__ occ) {
   __shared__ int wsum[32], wsumi[32];
   __shared__ int ty0[32], ty1[32];  // per plane of tiles: first and last occupied tile row
@@ -194,7 +241,7 @@ __global__ void __launch_bounds__(1024) k_scan_tiles(const int* __restrict__ cnt
   for (int base = 0; base < ntiles; base += 1024) {
     const int i = base + (int)threadIdx.x;
     const int cn = i + 1024 < ntiles ? cnt[i + 1024] : 0;
-    const int ci = (c + kAccumChunk - 1) / kAccumChunk;
+    const int ci = (c + chunk - 1) / chunk;
     if (occ && i < ntiles && (c > 0 || (more && more[i] > 0))) {
       const int q = i / ntx, tz = q / ntx, ty = q - tz * ntx;
       if (ty < *(volatile int*)&ty0[tz]) atomicMin(&ty0[tz], ty);
@@ -295,13 +342,15 @@ __global__ void __launch_bounds__(1024) k_scan_tiles(const int* __restrict__ cnt
 // raw = 1 (randoms only): values w and w^2 without alpha, for the cached
 // random grids that later mocks combine with their own alpha.
 template <int P>
-__global__ void __launch_bounds__(kBinThreads) k_bin_scatter(CatDev c, int is_ran, int raw, GeomDev g, int ntx,
-                                                             int ntiles, float obx, float oby, float obz,
+__global__ void __launch_bounds__(kBinThreads) k_bin_scatter(CatDev cg, CatDev cr, int nbg, int raw, GeomDev g,
+                                                             int ntx, int ntiles, float obx, float oby, float obz,
                                                              const double* __restrict__ ds,
                                                              const int* __restrict__ off,
                                                              const int* __restrict__ bpref,
                                                              float4* __restrict__ xyzv, float* __restrict__ vw2,
                                                              double* __restrict__ labpart) {
+  const int is_ran = (int)blockIdx.x >= nbg;
+  const CatDev& c = is_ran ? cr : cg;
   extern __shared__ int hist[];
   __shared__ double sh[32];
   // alpha and alpha^2 as float pairs (hi + lo): each random's value is then
@@ -310,8 +359,9 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_scatter(CatDev c, int is_ra
   const double ad = raw ? 0.0 : ds[DS_ALPHA];
   const float alpha = (float)ad, alo = (float)(ad - (double)alpha);
   const float a2 = (float)(ad * ad), a2lo = (float)(ad * ad - (double)a2);
-  const long long chunk = (c.n + gridDim.x - 1) / gridDim.x;
-  const long long i0 = blockIdx.x * chunk;
+  const int nblk = is_ran ? (int)gridDim.x - nbg : nbg, blk = is_ran ? (int)blockIdx.x - nbg : (int)blockIdx.x;
+  const long long chunk = (c.n + nblk - 1) / nblk;
+  const long long i0 = blk * chunk;
   const long long i1 = i0 + chunk < c.n ? i0 + chunk : c.n;
   const int* brow = bpref + (size_t)blockIdx.x * ntiles;
   for (int t = threadIdx.x; t < ntiles; t += blockDim.x) hist[t] = off[t] + brow[t];
@@ -353,7 +403,7 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_scatter(CatDev c, int is_ra
 #pragma unroll
     for (int q = 0; q < LAB_NSUM; ++q) {
       const double v = block_sum_f64(lab[q].value(), sh);
-      if (threadIdx.x == 0) labpart[(size_t)blockIdx.x * LAB_NSUM + q] = v;
+      if (threadIdx.x == 0) labpart[(size_t)blk * LAB_NSUM + q] = v;
     }
   }
 }
@@ -425,7 +475,16 @@ __device__ __forceinline__ float object_moment(const GeomDev& g, const float4& o
   return ipow(hx, ea) * ipow(hy, eb) * ipow(hz, ec);
 }
 
-// One block per work item: up to kAccumChunk objects of one tile (items in
+// Exponents (a, b, c) of the moment fields of a per-object plan (n = 0:
+// only F): blockIdx.y picks the field, gridded N^3 cells after the one before
+// (one launch for all 16: on a small survey a launch per field leaves most
+// SMs idle, 128^3 and 2.2e5 objects 16 x 21 us).
+struct MomentExp {
+  int n = 0;
+  unsigned char e[kMaxFields][3];
+};
+
+// One block per work item: up to chunk (<= kAccumChunk) objects of one tile (items in
 // tile order; items[t] is tile t's first).  The tile's region, from one cell
 // below the tile to the end of its reach (reg_side cells a side), covers the
 // taps of every object whose centre cell lies in the tile.  Blocks past the
@@ -451,7 +510,25 @@ __global__ void __launch_bounds__(kAccumThreads, W2 ? 2 : 4) k_tile_accum(GeomDe
                                                                         const float* __restrict__ vw2,
                                                                         unsigned long long* __restrict__ grid,
                                                                         unsigned long long* __restrict__ gridw,
-                                                                        int ea, int eb, int ec) {
+                                                                        int chunk, MomentExp xe,
+                                                                        const double* __restrict__ labpart, int nlab,
+                                                                        double* __restrict__ lab) {
+  // the last block (one more than the items can be) sums L^ab instead, warp q
+  // quantity q over the random blocks in a fixed order
+  if (lab && blockIdx.x == gridDim.x - 1 && blockIdx.y == 0) {
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (w >= LAB_NSUM) return;
+    double v = 0.0;
+    for (int b = lane; b < nlab; b += 32) v += labpart[(size_t)b * LAB_NSUM + w];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (lane == 0) lab[w] = v;
+    return;
+  }
+  // moment field of a per-object plan (0: F)
+  const int fld = blockIdx.y;
+  const int ea = xe.n ? xe.e[fld][0] : 0, eb = xe.n ? xe.e[fld][1] : 0, ec = xe.n ? xe.e[fld][2] : 0;
+  grid += (size_t)fld * g.N * g.N * g.N;
   constexpr int kReg = reg_side<P>(), kReg3 = reg_cells<P>();
   static_assert(kAccumChunk * 262144ll < 2147483648ll, "the low words would wrap");
   extern __shared__ unsigned long long reg[];
@@ -484,8 +561,8 @@ __global__ void __launch_bounds__(kAccumThreads, W2 ? 2 : 4) k_tile_accum(GeomDe
   }
   __syncthreads();
   const int t = s_tile;
-  const int a = off[t] + (item - items[t]) * kAccumChunk;
-  const int b = min(off[t + 1], a + kAccumChunk);
+  const int a = off[t] + (item - items[t]) * chunk;
+  const int b = min(off[t + 1], a + chunk);
   const int tx = t % ntx, ty = (t / ntx) % ntx, tz = t / (ntx * ntx);
   const int lx0 = tx * kTile - 1, ly0 = ty * kTile - 1, lz0 = tz * kTile - 1;
   // the item's objects are read twice: for the bounds, then for the taps
@@ -510,7 +587,7 @@ __global__ void __launch_bounds__(kAccumThreads, W2 ? 2 : 4) k_tile_accum(GeomDe
   for (int i = a + threadIdx.x; i < b; i += kAccumThreads) {
     float4 o = xyzv[i];
     const float wv = W2 ? vw2[i] : 0.f;
-    if (ea >= 0) o.w *= object_moment(g, o, ea, eb, ec);  // |x^ products| <= 1: the bounds hold
+    if (fld > 0) o.w *= object_moment(g, o, ea, eb, ec);  // |x^ products| <= 1: the bounds hold
     const float ux = (o.x - g.ox) * g.invH, uy = (o.y - g.oy) * g.invH, uz = (o.z - g.oz) * g.invH;
     int ix, iy, iz;
     float wx[P], wy[P], wz[P];
@@ -610,87 +687,100 @@ cudaError_t launch_combine_randoms(unsigned long long* grid, const unsigned long
   return cudaGetLastError();
 }
 
-// bh: the nblk rows (ntiles ints each) this launch fills.
-cudaError_t launch_bin_count(const CatDev& c, int is_ran, const GeomDev& g, double* part, int* bh, int* err,
-                             int nblk, cudaStream_t s) {
+// Both catalogs in one launch, nbg + nbr blocks (nbg = 0: no galaxies, nbr = 0:
+// the randoms are cached); part and bh: their nbg + nbr rows.
+cudaError_t launch_bin_count(const CatDev& gal, const CatDev& ran, int nbg, int nbr, const GeomDev& g, double* part,
+                             int* bh, int* err, cudaStream_t s) {
   const int ntx = assign_tiles_per_axis(g.N);
   const int ntiles = ntx * ntx * ntx;
-  if (c.n == 0) {
-    cudaMemsetAsync(part, 0, sizeof(double) * SC_NSUM * nblk, s);
-    cudaMemsetAsync(bh, 0, sizeof(int) * (size_t)ntiles * nblk, s);
-    return cudaGetLastError();
-  }
   const size_t sm = sizeof(int) * ntiles;
+  const int nblk = nbg + nbr;
   if (g.assign == 2) {
     raise_smem_limit((const void*)k_bin_count<2>, sm);
-    k_bin_count<2><<<nblk, kBinThreads, sm, s>>>(c, is_ran, g, ntx, ntiles, part, bh, err);
+    k_bin_count<2><<<nblk, kBinThreads, sm, s>>>(gal, ran, nbg, g, ntx, ntiles, part, bh, err);
   } else if (g.assign == 3) {
     raise_smem_limit((const void*)k_bin_count<3>, sm);
-    k_bin_count<3><<<nblk, kBinThreads, sm, s>>>(c, is_ran, g, ntx, ntiles, part, bh, err);
+    k_bin_count<3><<<nblk, kBinThreads, sm, s>>>(gal, ran, nbg, g, ntx, ntiles, part, bh, err);
   } else {
     raise_smem_limit((const void*)k_bin_count<4>, sm);
-    k_bin_count<4><<<nblk, kBinThreads, sm, s>>>(c, is_ran, g, ntx, ntiles, part, bh, err);
+    k_bin_count<4><<<nblk, kBinThreads, sm, s>>>(gal, ran, nbg, g, ntx, ntiles, part, bh, err);
   }
   return cudaGetLastError();
 }
 
-cudaError_t launch_tile_prefix(int* bh, int nrows, int ntiles, int* cnt, cudaStream_t s) {
-  k_tile_prefix<<<(ntiles + 255) / 256, 256, 0, s>>>(bh, nrows, ntiles, cnt);
+// ds: NULL, or where the scalars go (formed from the nbg + nbr rows of part).
+cudaError_t launch_tile_prefix(int* bh, int nrows, int ntiles, int* cnt, const double* part, int nbg, int nbr,
+                               long long ng, long long nr, int alpha_mode, double* ds, cudaStream_t s) {
+  k_tile_prefix<<<(ntiles + 31) / 32 + (ds ? 1 : 0), 256, 0, s>>>(bh, nrows, ntiles, cnt, part, nbg, nbr, ng, nr,
+                                                                  alpha_mode, ds);
   return cudaGetLastError();
 }
 
-cudaError_t launch_scan_tiles(const int* cnt, int ntiles, int* off, int* items, cudaStream_t s, const GeomDev& g,
-                              const int* more, int* occ) {
-  k_scan_tiles<<<1, 1024, 0, s>>>(cnt, ntiles, off, items, more, assign_tiles_per_axis(g.N), g.N,
+// Objects per work item of the tile accumulation: kAccumChunk for large
+// catalogs (an item pays for clearing its region and adding it to the grid),
+// less where that would leave SMs without an item: about eight items per SM,
+// at least 512 objects (64^3, 2.2e5 objects: 33 us with one item per tile; with the
+// other launches merged, the whole 64^3 mock 294 -> 237 us).
+int accum_chunk(long long nobj, int nsm) {
+  const long long c = nobj / (8ll * nsm);
+  return (int)std::max<long long>(512, std::min<long long>(kAccumChunk, c));
+}
+
+cudaError_t launch_scan_tiles(const int* cnt, int ntiles, int* off, int* items, int chunk, cudaStream_t s,
+                              const GeomDev& g, const int* more, int* occ) {
+  k_scan_tiles<<<1, 1024, 0, s>>>(cnt, ntiles, off, items, chunk, more, assign_tiles_per_axis(g.N), g.N,
                                   g.assign == 4 ? kTile + 1 : kTile, g.periodic, occ);
   return cudaGetLastError();
 }
 
-// off: the tile offsets; bpref: the nblk prefixed count rows of this catalog.
-cudaError_t launch_bin_scatter(const CatDev& c, int is_ran, const GeomDev& g, const double obs[3], const double* ds,
-                               const int* off, const int* bpref, float4* xyzv, float* vw2, double* labpart, int nblk,
-                               cudaStream_t s, int raw) {
-  if (c.n == 0) {
-    if (is_ran) cudaMemsetAsync(labpart, 0, sizeof(double) * LAB_NSUM * nblk, s);
-    return cudaGetLastError();
-  }
+// off: the tile offsets; bpref: the nbg + nbr prefixed count rows.
+cudaError_t launch_bin_scatter(const CatDev& gal, const CatDev& ran, int nbg, int nbr, const GeomDev& g,
+                               const double obs[3], const double* ds, const int* off, const int* bpref, float4* xyzv,
+                               float* vw2, double* labpart, cudaStream_t s, int raw) {
   const int ntx = assign_tiles_per_axis(g.N);
   const int ntiles = ntx * ntx * ntx;
   const size_t sm = sizeof(int) * ntiles;
-  if (g.assign == 2) {
-    raise_smem_limit((const void*)k_bin_scatter<2>, sm);
-    k_bin_scatter<2><<<nblk, kBinThreads, sm, s>>>(c, is_ran, raw, g, ntx, ntiles, (float)obs[0], (float)obs[1],
-                                                   (float)obs[2], ds, off, bpref, xyzv, vw2, labpart);
-  } else if (g.assign == 3) {
-    raise_smem_limit((const void*)k_bin_scatter<3>, sm);
-    k_bin_scatter<3><<<nblk, kBinThreads, sm, s>>>(c, is_ran, raw, g, ntx, ntiles, (float)obs[0], (float)obs[1],
-                                                   (float)obs[2], ds, off, bpref, xyzv, vw2, labpart);
-  } else {
-    raise_smem_limit((const void*)k_bin_scatter<4>, sm);
-    k_bin_scatter<4><<<nblk, kBinThreads, sm, s>>>(c, is_ran, raw, g, ntx, ntiles, (float)obs[0], (float)obs[1],
-                                                   (float)obs[2], ds, off, bpref, xyzv, vw2, labpart);
-  }
+  const int nblk = nbg + nbr;
+#define FKP_SC(PP)                                                                                                 \
+  do {                                                                                                             \
+    raise_smem_limit((const void*)k_bin_scatter<PP>, sm);                                                          \
+    k_bin_scatter<PP><<<nblk, kBinThreads, sm, s>>>(gal, ran, nbg, raw, g, ntx, ntiles, (float)obs[0],             \
+                                                    (float)obs[1], (float)obs[2], ds, off, bpref, xyzv, vw2, labpart); \
+  } while (0)
+  if (g.assign == 2) FKP_SC(2);
+  else if (g.assign == 3) FKP_SC(3);
+  else FKP_SC(4);
+#undef FKP_SC
   return cudaGetLastError();
 }
 
-// nobj: the objects scattered into tile order (bounds the number of items).
-cudaError_t launch_tile_accum(const GeomDev& g, const int* off, const int* items, long long nobj, const float4* xyzv,
-                              const float* vw2, unsigned long long* grid, unsigned long long* gridw, cudaStream_t s,
-                              const unsigned char* xe) {
-  const int ea = xe ? xe[0] : -1, eb = xe ? xe[1] : 0, ec = xe ? xe[2] : 0;
+// nobj: the objects scattered into tile order (bounds the number of items);
+// mt: the moment table of a per-object plan, or NULL; lab: NULL, or where the
+// L^ab sums of the nlab rows of labpart go.
+cudaError_t launch_tile_accum(const GeomDev& g, const int* off, const int* items, long long nobj, int chunk,
+                              const float4* xyzv, const float* vw2, unsigned long long* grid,
+                              unsigned long long* gridw, cudaStream_t s, const MomentTable* mt,
+                              const double* labpart, int nlab, double* lab) {
+  MomentExp xe;
+  if (mt) {
+    xe.n = mt->nfields;
+    for (int q = 0; q < mt->nfields; ++q)
+      for (int a = 0; a < 3; ++a) xe.e[q][a] = mt->e[q][a];
+  }
   const int ntx = assign_tiles_per_axis(g.N);
   const int ntiles = ntx * ntx * ntx;
   // every non-empty tile has one item that may be partial, the rest are full
-  const long long nitems = std::min<long long>((long long)ntiles, nobj) + nobj / kAccumChunk;
+  const long long nitems = std::min<long long>((long long)ntiles, nobj) + nobj / chunk + (lab ? 1 : 0);
   if (nitems <= 0) return cudaSuccess;
   if (nitems > INT32_MAX) return cudaErrorInvalidValue;
   const bool w2 = gridw != nullptr;
+  const dim3 blocks((unsigned)nitems, mt ? mt->nfields : 1);
 #define FKP_TA(PP, WW)                                                                                 \
   do {                                                                                                 \
     const size_t sm = sizeof(unsigned long long) * reg_cells<PP>() * (WW ? 2 : 1);                     \
     raise_smem_limit((const void*)k_tile_accum<PP, WW>, sm);                                           \
-    k_tile_accum<PP, WW><<<(int)nitems, kAccumThreads, sm, s>>>(g, ntx, ntiles, off, items, xyzv, vw2, grid, \
-                                                                gridw, ea, eb, ec);                    \
+    k_tile_accum<PP, WW><<<blocks, kAccumThreads, sm, s>>>(g, ntx, ntiles, off, items, xyzv, vw2, grid, \
+                                                           gridw, chunk, xe, labpart, nlab, lab);      \
   } while (0)
   if (g.assign == 2) {
     if (w2) FKP_TA(2, true); else FKP_TA(2, false);

@@ -1,60 +1,13 @@
-// k_power.cu - scalar finalize and bin reduction of the power-spectrum
-// path (Sec. III.A of the paper):
-//   the FP64 finalize of the scalars (alpha, I_22, I_33, N_0, S_3; eqs.
-//   I22def, N0true, Noise0) and of L^ab (eq. Lab), and the fixed-order FP64
-//   reduction of the z-pass's per-block bin sums.  Gridding is in
-//   k_assign.cu, the three FFT passes in k_xpass.cu, k_ypass.cu and
-//   k_zpass.cu.
+// k_power.cu - the fixed-order FP64 reduction of the z-pass's per-block bin
+//   sums (Sec. III.A of the paper) and the bounded-wait diagnostic.  Gridding
+//   and the scalars are in k_assign.cu, the three FFT passes in k_xpass.cu,
+//   k_ypass.cu and k_zpass.cu.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
 #include "fkp_internal.h"
 
 namespace fkp {
-
-// ----------------------------------------------------------------------------
-// helpers
-// ----------------------------------------------------------------------------
-
-// One block of 32 threads: fixed-order sums over the per-block partials and
-// the derived scalars, all FP64.  Galaxy blocks are [0, nbg), random blocks
-// [nbg, nbg + nbr).
-__global__ void k_scalars_finalize(const double* __restrict__ part, int nbg, int nbr, long long ng, long long nr,
-                                   int alpha_mode, double* __restrict__ ds) {
-  __shared__ double tot[SC_NSUM];
-  const int q = threadIdx.x;
-  if (q < SC_NSUM) {
-    const bool gal = q <= SC_G_W3;
-    const int b0 = gal ? 0 : nbg, b1 = gal ? nbg : nbg + nbr;
-    double s = 0.0;
-    for (int b = b0; b < b1; ++b) s += part[(size_t)b * SC_NSUM + q];
-    tot[q] = s;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const double Wg = tot[SC_G_W], Wr = tot[SC_R_W];
-    const double a = alpha_mode == 0 ? Wg / Wr : (double)ng / (double)nr;
-    ds[DS_ALPHA] = a;
-    ds[DS_I22] = a * tot[SC_R_NW2];
-    ds[DS_I33] = a * tot[SC_R_N2W3];
-    ds[DS_N0] = tot[SC_G_W2] + a * a * tot[SC_R_W2];
-    ds[DS_N0FKP] = a * (1.0 + a) * tot[SC_R_W2];
-    ds[DS_S3] = tot[SC_G_W3] - a * a * a * tot[SC_R_W3];
-    ds[DS_WG] = Wg;
-    ds[DS_WR] = Wr;
-    ds[DS_NG] = (double)ng;
-    ds[DS_NR] = (double)nr;
-  }
-}
-
-__global__ void k_lab_finalize(const double* __restrict__ labpart, int nblk, double* __restrict__ out) {
-  const int q = threadIdx.x;
-  if (q < LAB_NSUM) {
-    double s = 0.0;
-    for (int b = 0; b < nblk; ++b) s += labpart[(size_t)b * LAB_NSUM + q];
-    out[q] = s;
-  }
-}
 
 // One block per (quantity, bin): fixed-order FP64 tree sum over the blocks.
 // blockIdx.y picks the mock of a fused launch (partials at pstride / pcstride,
@@ -101,19 +54,8 @@ __global__ void k_wait_selftest(unsigned polls, int* __restrict__ flag) {
 // host-side launch wrappers (called by the C ABI)
 // ----------------------------------------------------------------------------
 
-cudaError_t launch_scalars_finalize(const double* part, int nbg, int nbr, long long ng, long long nr, int amode,
-                                    double* ds, cudaStream_t s) {
-  k_scalars_finalize<<<1, 32, 0, s>>>(part, nbg, nbr, ng, nr, amode, ds);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_wait_selftest(unsigned polls, int* flag, cudaStream_t s) {
   k_wait_selftest<<<1, 32, 0, s>>>(polls, flag);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_lab_finalize(const double* labpart, int nblk, double* out, cudaStream_t s) {
-  k_lab_finalize<<<1, 32, 0, s>>>(labpart, nblk, out);
   return cudaGetLastError();
 }
 

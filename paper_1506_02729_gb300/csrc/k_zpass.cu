@@ -400,15 +400,10 @@ static cudaError_t zdispatch(const float2* S2, const GeomDev& g, const MomentTab
     case 512: return zrun<512, MODE>(S2, g, mt, fp, tw, zp, pr, part, partc, err, s, nsm, nt, mb);
     case 360: return zrun<360, MODE>(S2, g, mt, fp, tw, zp, pr, part, partc, err, s, nsm, nt, mb);
     case 256: return zrun<256, MODE>(S2, g, mt, fp, tw, zp, pr, part, partc, err, s, nsm, nt, mb);
+    case 384: return zrun<384, MODE>(S2, g, mt, fp, tw, zp, pr, part, partc, err, s, nsm, nt, mb);
+    case 128: return zrun<128, MODE>(S2, g, mt, fp, tw, zp, pr, part, partc, err, s, nsm, nt, mb);
+    case 64: return zrun<64, MODE>(S2, g, mt, fp, tw, zp, pr, part, partc, err, s, nsm, nt, mb);
     default: break;
-  }
-  if (MODE == 0) {
-    switch (g.N) {
-      case 384: return zrun<384, MODE>(S2, g, mt, fp, tw, zp, pr, part, partc, err, s, nsm, nt, mb);
-      case 128: return zrun<128, MODE>(S2, g, mt, fp, tw, zp, pr, part, partc, err, s, nsm, nt, mb);
-      case 64: return zrun<64, MODE>(S2, g, mt, fp, tw, zp, pr, part, partc, err, s, nsm, nt, mb);
-      default: break;
-    }
   }
   return zrun<0, MODE>(S2, g, mt, fp, tw, zp, pr, part, partc, err, s, nsm, nt, mb);
 }
