@@ -688,15 +688,11 @@ cudaError_t fkp::record_stage(cudaEvent_t ev, cudaStream_t s) {
 // Enqueues scalars and gridding of both catalogs into d_grid (and d_gridw):
 // tile counts with the scalar sums, offsets, scatter into tile order, and
 // shared-memory accumulation per tile.
-// One grid of the pair (which = 1: the interlaced second grid, nodes half a
-// cell further; no stage events).
-static int grid_pass(Plan* P, const CatDev& gal, const CatDev& ran, cudaStream_t s, int which) {
-  const GeomDev& geo = which ? P->g2 : P->g;
-  unsigned long long* grid = which ? P->d_grid2 : P->d_grid;
-  unsigned long long* gridw = which ? P->d_gridw2 : P->d_gridw;
-  const unsigned long long* rgrid = which ? P->rc_grid2 : P->rc_grid;
-  const unsigned long long* rgridw = which ? P->rc_gridw2 : P->rc_gridw;
-  auto stage = [&](int e) { return which ? cudaSuccess : record_stage(P->ev[e], s); };
+// The second grid of an interlaced pair (nodes half a cell further) is filled
+// from the same tile-sorted objects.
+static int grid_pass(Plan* P, const CatDev& gal, const CatDev& ran, cudaStream_t s) {
+  const GeomDev& geo = P->g;
+  unsigned long long *grid = P->d_grid, *gridw = P->d_gridw;
   const int N = P->g.N;
   const size_t N3 = (size_t)N * N * N;
   const bool cached = ran.n < 0;  // the plan's cached random grids (fkp_plan_cache_randoms)
@@ -729,17 +725,20 @@ static int grid_pass(Plan* P, const CatDev& gal, const CatDev& ran, cudaStream_t
   const long long share = cached ? nb : std::max<long long>(1, std::min<long long>(nb - 1, nb * gal.n / std::max<long long>(1, ntot)));
   const int nbg = nblocks(gal.n, share), nbr = cached ? P->rc_nblk : nblocks(ran.n, nb - share);
   const long long nran = cached ? P->rc_n : ran.n;
-  if (!which) CK(cudaMemsetAsync(P->d_err, 0, sizeof(int) * 4, s));
-  CK(stage(0));
+  CK(cudaMemsetAsync(P->d_err, 0, sizeof(int) * 4, s));
+  CK(record_stage(P->ev[0], s));
   // zero the grids on the side stream while the counts run
   CK(cudaEventRecord(P->ev_fork, s));
   CK(cudaStreamWaitEvent(P->side, P->ev_fork, 0));
   const int ngrid = P->per_object ? P->mt.nfields : 1;  // per object: the moment fields follow F
   CK(cudaMemsetAsync(grid, 0, N3 * 8 * ngrid, P->side));
   if (gridw) CK(cudaMemsetAsync(gridw, 0, N3 * 8, P->side));
+  if (P->interlace) CK(cudaMemsetAsync(P->d_grid2, 0, N3 * 8, P->side));
+  if (P->interlace && gridw) CK(cudaMemsetAsync(P->d_gridw2, 0, N3 * 8, P->side));
   CK(cudaEventRecord(P->ev_join, P->side));
   const int nbx = cached ? 0 : nbr;  // blocks that read randoms
-  CK(launch_bin_count(gal, ran, nbg, nbx, geo, P->d_scpart, P->d_bhist, P->d_err, s));
+  const GeomDev* geo2 = P->interlace ? &P->g2 : nullptr;
+  CK(launch_bin_count(gal, ran, nbg, nbx, geo, geo2, P->d_scpart, P->d_bhist, P->d_err, s));
   if (cached)
     CK(cudaMemcpyAsync(P->d_scpart + (size_t)nbg * SC_NSUM, P->rc_part, sizeof(double) * SC_NSUM * nbr,
                        cudaMemcpyDeviceToDevice, s));
@@ -747,8 +746,8 @@ static int grid_pass(Plan* P, const CatDev& gal, const CatDev& ran, cudaStream_t
                         geo.alpha_mode, P->d_ds, s));
   const int chunk = accum_chunk(ntot * ngrid, nb);
   CK(launch_scan_tiles(P->d_tcnt, P->ntiles, P->d_toff, P->d_titem, chunk, s, geo,
-                       cached ? (which ? P->rc_tcnt2 : P->rc_tcnt) : nullptr, which ? P->d_occ2 : P->d_occ));
-  CK(stage(1));
+                       cached ? P->rc_tcnt : nullptr, P->d_occ, P->d_occ2));
+  CK(record_stage(P->ev[1], s));
   CK(cudaStreamWaitEvent(s, P->ev_join, 0));
   float* vw2 = gridw ? P->d_vw2 : nullptr;
   CK(launch_bin_scatter(gal, ran, nbg, nbx, geo, P->geom.observer, P->d_ds, P->d_toff, P->d_bhist, P->d_xyzv, vw2,
@@ -756,10 +755,17 @@ static int grid_pass(Plan* P, const CatDev& gal, const CatDev& ran, cudaStream_t
   if (cached)
     CK(cudaMemcpyAsync(P->d_ds + DS_COUNT, P->rc_lab, sizeof(double) * LAB_NSUM, cudaMemcpyDeviceToDevice, s));
   // per-object line of sight: moment field q grids w x^^e[q] with each object's x^
-  CK(launch_tile_accum(geo, P->d_toff, P->d_titem, ntot, chunk, P->d_xyzv, vw2, grid, gridw, s,
+  CK(launch_tile_accum(geo, P->d_toff, P->d_titem, ntot, chunk, P->d_xyzv, vw2, grid, gridw, s, nullptr,
                        P->per_object ? &P->mt : nullptr, P->d_labpart, nbr, cached ? nullptr : P->d_ds + DS_COUNT));
   if (cached)
-    CK(launch_combine_randoms(grid, rgrid, gridw, rgridw, P->d_ds, (long long)N3, P->ctx->nsm, s));
+    CK(launch_combine_randoms(grid, P->rc_grid, gridw, P->rc_gridw, P->d_ds, (long long)N3, P->ctx->nsm, s));
+  if (P->interlace) {
+    CK(launch_tile_accum(P->g2, P->d_toff, P->d_titem, ntot, chunk, P->d_xyzv, vw2, P->d_grid2, P->d_gridw2, s, &geo,
+                         nullptr, nullptr, 0, nullptr));
+    if (cached)
+      CK(launch_combine_randoms(P->d_grid2, P->rc_grid2, P->d_gridw2, P->rc_gridw2, P->d_ds, (long long)N3,
+                                P->ctx->nsm, s));
+  }
   return FKP_OK;
 }
 
@@ -768,8 +774,7 @@ static int grid_pass(Plan* P, const CatDev& gal, const CatDev& ran, cudaStream_t
 // scalar sums, offsets, scatter into tile order, and shared-memory
 // accumulation per tile.
 int fkp::enqueue_grids(Plan* P, const CatDev& gal, const CatDev& ran, cudaStream_t s) {
-  int rc = grid_pass(P, gal, ran, s, 0);
-  if (!rc && P->interlace) rc = grid_pass(P, gal, ran, s, 1);
+  const int rc = grid_pass(P, gal, ran, s);
   if (rc) return rc;
   CK(record_stage(P->ev[2], s));
   return FKP_OK;
@@ -801,8 +806,7 @@ static int cache_randoms(Plan* P, const CatDev& ran, cudaStream_t s) {
     P->rc_part = (double*)P->alloc(sizeof(double) * SC_NSUM * nb);
     P->rc_lab = (double*)P->alloc(sizeof(double) * LAB_NSUM);
     P->rc_tcnt = (int*)P->alloc(sizeof(int) * P->ntiles);
-    P->rc_tcnt2 = P->interlace ? (int*)P->alloc(sizeof(int) * P->ntiles) : P->rc_tcnt;
-    if (!P->rc_grid || (P->d_gridw && !P->rc_gridw) || !P->rc_part || !P->rc_lab || !P->rc_tcnt || !P->rc_tcnt2 ||
+    if (!P->rc_grid || (P->d_gridw && !P->rc_gridw) || !P->rc_part || !P->rc_lab || !P->rc_tcnt ||
         (P->interlace && (!P->rc_grid2 || (P->d_gridw && !P->rc_gridw2))))
       return set_error(FKP_ENOMEM, "cannot allocate the cached random grids");
   }
@@ -820,21 +824,20 @@ static int cache_randoms(Plan* P, const CatDev& ran, cudaStream_t s) {
   }
   float* vw2 = P->d_gridw ? P->d_vw2 : nullptr;
   CK(cudaMemsetAsync(P->d_err, 0, sizeof(int) * 4, s));
+  CK(launch_bin_count(ran, ran, 0, nbr, P->g, P->interlace ? &P->g2 : nullptr, P->rc_part, P->d_bhist, P->d_err, s));
+  CK(launch_tile_prefix(P->d_bhist, nbr, P->ntiles, P->d_tcnt, nullptr, 0, 0, 0, 0, 0, nullptr, s));
+  const int chunk = accum_chunk(ran.n, nb);
+  CK(launch_scan_tiles(P->d_tcnt, P->ntiles, P->d_toff, P->d_titem, chunk, s, P->g, nullptr, nullptr, nullptr));
+  CK(cudaMemcpyAsync(P->rc_tcnt, P->d_tcnt, sizeof(int) * P->ntiles, cudaMemcpyDeviceToDevice, s));
+  CK(launch_bin_scatter(ran, ran, 0, nbr, P->g, P->geom.observer, P->d_ds, P->d_toff, P->d_bhist, P->d_xyzv, vw2,
+                        P->d_labpart, s, 1));
   for (int which = 0; which < (P->interlace ? 2 : 1); ++which) {
-    const GeomDev& geo = which ? P->g2 : P->g;
     unsigned long long* rg = which ? P->rc_grid2 : P->rc_grid;
     unsigned long long* rgw = which ? P->rc_gridw2 : P->rc_gridw;
-    CK(launch_bin_count(ran, ran, 0, nbr, geo, P->rc_part, P->d_bhist, P->d_err, s));
-    CK(launch_tile_prefix(P->d_bhist, nbr, P->ntiles, P->d_tcnt, nullptr, 0, 0, 0, 0, 0, nullptr, s));
-    const int chunk = accum_chunk(ran.n, nb);
-    CK(launch_scan_tiles(P->d_tcnt, P->ntiles, P->d_toff, P->d_titem, chunk, s, geo, nullptr, nullptr));
-    CK(cudaMemcpyAsync(which ? P->rc_tcnt2 : P->rc_tcnt, P->d_tcnt, sizeof(int) * P->ntiles, cudaMemcpyDeviceToDevice, s));
     CK(cudaMemsetAsync(rg, 0, N3 * 8, s));
     if (rgw) CK(cudaMemsetAsync(rgw, 0, N3 * 8, s));
-    CK(launch_bin_scatter(ran, ran, 0, nbr, geo, P->geom.observer, P->d_ds, P->d_toff, P->d_bhist, P->d_xyzv, vw2,
-                          P->d_labpart, s, 1));
-    CK(launch_tile_accum(geo, P->d_toff, P->d_titem, ran.n, chunk, P->d_xyzv, vw2, rg, rgw, s, nullptr, P->d_labpart,
-                         nbr, P->rc_lab));
+    CK(launch_tile_accum(which ? P->g2 : P->g, P->d_toff, P->d_titem, ran.n, chunk, P->d_xyzv, vw2, rg, rgw, s,
+                         which ? &P->g : nullptr, nullptr, P->d_labpart, nbr, which ? nullptr : P->rc_lab));
   }
   int herr = 0;
   CK(cudaMemcpyAsync(&herr, P->d_err, sizeof(int), cudaMemcpyDeviceToHost, s));

@@ -90,7 +90,7 @@ struct Plan {
   bool rc_valid = false;
   unsigned long long *rc_grid = nullptr, *rc_gridw = nullptr;
   double *rc_part = nullptr, *rc_lab = nullptr;
-  int *rc_tcnt = nullptr, *rc_tcnt2 = nullptr;  // its tile counts
+  int* rc_tcnt = nullptr;  // its tile counts
   int rc_nblk = 0;
   long long rc_n = 0;
 
@@ -169,15 +169,15 @@ int tiles_x(int N);
 bool moments_match(const MomentTable& mt);
 size_t field_elems(int N);
 int assign_tiles_per_axis(int N);
-cudaError_t launch_bin_count(const CatDev& gal, const CatDev& ran, int nbg, int nbr, const GeomDev& g, double* part,
-                             int* bh, int* err, cudaStream_t s);
+cudaError_t launch_bin_count(const CatDev& gal, const CatDev& ran, int nbg, int nbr, const GeomDev& g,
+                             const GeomDev* g2, double* part, int* bh, int* err, cudaStream_t s);
 cudaError_t launch_tile_prefix(int* bh, int nrows, int ntiles, int* cnt, const double* part, int nbg, int nbr,
                                long long ng, long long nr, int alpha_mode, double* ds, cudaStream_t s);
 int accum_chunk(long long nobj, int nsm);
 // occ: NULL, or the plan's list of occupied rows; more: NULL, or the tile
 // counts of a cached random catalog.
 cudaError_t launch_scan_tiles(const int* cnt, int ntiles, int* off, int* items, int chunk, cudaStream_t s,
-                              const GeomDev& g, const int* more, int* occ);
+                              const GeomDev& g, const int* more, int* occ, int* occ2);
 cudaError_t launch_bin_scatter(const CatDev& gal, const CatDev& ran, int nbg, int nbr, const GeomDev& g,
                                const double obs[3], const double* ds, const int* off, const int* bpref, float4* xyzv,
                                float* vw2, double* labpart, cudaStream_t s, int raw = 0);
@@ -186,7 +186,7 @@ cudaError_t launch_combine_randoms(unsigned long long* grid, const unsigned long
                                    long long n, int nsm, cudaStream_t s);
 cudaError_t launch_tile_accum(const GeomDev& g, const int* off, const int* items, long long nobj, int chunk,
                               const float4* xyzv, const float* vw2, unsigned long long* grid,
-                              unsigned long long* gridw, cudaStream_t s, const MomentTable* mt,
+                              unsigned long long* gridw, cudaStream_t s, const GeomDev* first, const MomentTable* mt,
                               const double* labpart, int nlab, double* lab);
 cudaError_t launch_wait_selftest(unsigned polls, int* flag, cudaStream_t s);
 // xm: x-pass blocks = SMs x resident blocks x xm; nt: threads per y- or

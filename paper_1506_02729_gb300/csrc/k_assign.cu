@@ -35,11 +35,12 @@ constexpr int kAccumChunk = 8160;
 constexpr int kAccumThreads = 512;
 // Region a tile's objects reach, from one cell below the tile: the tile
 // plus one halo cell on each side for CIC and TSC, and one more above for
-// PCS (taps c-1 .. c+2 of the centre cell c).
+// PCS (taps c-1 .. c+2 of the centre cell c)
+// (the second grid of an interlaced pair reaches one cell further down).
 template <int P>
-__host__ __device__ constexpr int reg_side() { return P == 4 ? kTile + 3 : kTile + 2; }
+__host__ __device__ constexpr int reg_side(bool second) { return (P == 4 ? kTile + 3 : kTile + 2) + (second ? 1 : 0); }
 template <int P>
-__host__ __device__ constexpr int reg_cells() { return reg_side<P>() * reg_side<P>() * reg_side<P>(); }
+__host__ __device__ constexpr int reg_cells(bool second) { return reg_side<P>(second) * reg_side<P>(second) * reg_side<P>(second); }
 
 int assign_tiles_per_axis(int N) { return (N + kTile - 1) / kTile; }
 
@@ -93,8 +94,8 @@ __device__ __forceinline__ int tile_of(int cx, int cy, int cz, int N, int ntx) {
 constexpr int kBinThreads = 1024;
 
 template <int P>
-__global__ void __launch_bounds__(kBinThreads) k_bin_count(CatDev cg, CatDev cr, int nbg, GeomDev g, int ntx,
-                                                           int ntiles, double* __restrict__ part,
+__global__ void __launch_bounds__(kBinThreads) k_bin_count(CatDev cg, CatDev cr, int nbg, GeomDev g, int two,
+                                                           GeomDev g2, int ntx, int ntiles, double* __restrict__ part,
                                                            int* __restrict__ bh, int* __restrict__ err) {
   const int is_ran = (int)blockIdx.x >= nbg;
   const CatDev& c = is_ran ? cr : cg;
@@ -128,6 +129,7 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_count(CatDev cg, CatDev cr,
       atomicAdd(hist + tile_of(cx, cy, cz, g.N, ntx), 1);
     else
       bad = true;
+    if (two && !centre_cell<P>(g2, __ldg(c.x + i), __ldg(c.y + i), __ldg(c.z + i), cx, cy, cz)) bad = true;
   }
   if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(err, 1);
   int* row = bh + (size_t)blockIdx.x * ntiles;
@@ -222,7 +224,8 @@ __global__ void __launch_bounds__(256) k_tile_prefix(int* __restrict__ bh, int n
 // and reach - kTile + 1 above, wrapped around a periodic box.
 __global__ void __launch_bounds__(1024) k_scan_tiles(const int* __restrict__ cnt, int ntiles, int* __restrict__ off,
                                                      int* __restrict__ items, int chunk, const int* __restrict__ more, int ntx,
-                                                     int N, int reach, int periodic, int* __restrict__ occ) {
+                                                     int N, int reach, int periodic, int* __restrict__ occ,
+                                                     int* __restrict__ occ2) {
   __shared__ int wsum[32], wsumi[32];
   __shared__ int ty0[32], ty1[32];  // per plane of tiles: first and last occupied tile row
   __shared__ int zfirst, zlast;
@@ -242,10 +245,22 @@ __global__ void __launch_bounds__(1024) k_scan_tiles(const int* __restrict__ cnt
     const int i = base + (int)threadIdx.x;
     const int cn = i + 1024 < ntiles ? cnt[i + 1024] : 0;
     const int ci = (c + chunk - 1) / chunk;
-    if (occ && i < ntiles && (c > 0 || (more && more[i] > 0))) {
-      const int q = i / ntx, tz = q / ntx, ty = q - tz * ntx;
-      if (ty < *(volatile int*)&ty0[tz]) atomicMin(&ty0[tz], ty);
-      if (ty > *(volatile int*)&ty1[tz]) atomicMax(&ty1[tz], ty);
+    if (occ) {
+      // lanes of one row of tiles speak through their first occupied lane
+      const bool full = i < ntiles && (c > 0 || (more && more[i] > 0));
+      const unsigned m = __ballot_sync(0xffffffffu, full);
+      const int q = i / ntx;
+      const int q0 = __shfl_up_sync(0xffffffffu, q, 1);
+      const unsigned starts = __ballot_sync(0xffffffffu, lane == 0 || q != q0);  // where a row begins in the warp
+      if (full) {
+        const unsigned upto = starts & (0xffffffffu >> (31 - lane));
+        const int first = 31 - __clz(upto);  // this row's first lane
+        if ((m & ((1u << lane) - 1u)) >> first == 0u) {
+          const int tz = q / ntx, ty = q - tz * ntx;
+          atomicMin(&ty0[tz], ty);
+          atomicMax(&ty1[tz], ty);
+        }
+      }
     }
     int s = c, si = ci;
 #pragma unroll
@@ -290,48 +305,59 @@ __global__ void __launch_bounds__(1024) k_scan_tiles(const int* __restrict__ cnt
     items[ntiles] = carryi;
   }
   if (!occ) return;
-  // plane z = threadIdx.x (N <= 512): the hull of the rows of the tile planes that reach it
-  const int z = threadIdx.x;
-  int y0 = N, y1 = 0;
-  if (z < N) {
-    for (int tz = 0; tz < ntx; ++tz) {
-      if (ty1[tz] < 0) continue;
-      const int a = tz * kTile - 1, b = tz * kTile + reach;
-      if (!((z >= a && z <= b) || (periodic && ((z - N >= a && z - N <= b) || (z + N >= a && z + N <= b))))) continue;
-      const int ya = ty0[tz] * kTile - 1, yb = ty1[tz] * kTile + reach;
-      if (periodic && (ya < 0 || yb >= N)) {
-        y0 = 0;
-        y1 = N;
-      } else {
-        y0 = min(y0, max(ya, 0));
-        y1 = max(y1, min(yb + 1, N));
+  // plane z = threadIdx.x (N <= 512): the hull of the rows of the tile planes
+  // that reach it.  The second grid of an interlaced pair is filled from the
+  // first grid's tiles, one cell further down (occ2).
+  for (int low = 1; low <= (occ2 ? 2 : 1); ++low) {
+    int* out = low == 1 ? occ : occ2;
+    const int z = threadIdx.x;
+    __syncthreads();
+    if (z == 0) {
+      zfirst = N;
+      zlast = -1;
+    }
+    __syncthreads();
+    int y0 = N, y1 = 0;
+    if (z < N) {
+      for (int tz = 0; tz < ntx; ++tz) {
+        if (ty1[tz] < 0) continue;
+        const int a = tz * kTile - low, b = tz * kTile + reach;
+        if (!((z >= a && z <= b) || (periodic && ((z - N >= a && z - N <= b) || (z + N >= a && z + N <= b))))) continue;
+        const int ya = ty0[tz] * kTile - low, yb = ty1[tz] * kTile + reach;
+        if (periodic && (ya < 0 || yb >= N)) {
+          y0 = 0;
+          y1 = N;
+        } else {
+          y0 = min(y0, max(ya, 0));
+          y1 = max(y1, min(yb + 1, N));
+        }
       }
+      if (y1 > y0) {
+        atomicMin(&zfirst, z);
+        atomicMax(&zlast, z);
+      } else {
+        y0 = y1 = 0;
+      }
+      out[4 + z] = y0 | (y1 << 16);
     }
-    if (y1 > y0) {
-      atomicMin(&zfirst, z);
-      atomicMax(&zlast, z);
-    } else {
-      y0 = y1 = 0;
-    }
-    occ[4 + z] = y0 | (y1 << 16);
-  }
-  const int len = z < N ? y1 - y0 : 0;
-  int sum = len;
+    const int len = z < N ? y1 - y0 : 0;
+    int sum = len;
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int v = __shfl_up_sync(0xffffffffu, sum, o);
-    if (lane >= o) sum += v;
-  }
-  if (lane == 31) wsum[warp] = sum;
-  __syncthreads();
-  int before = 0;
-  for (int w = 0; w < warp; ++w) before += wsum[w];
-  if (z < N) occ[4 + N + z] = before + sum - len;
-  if (z == N - 1) {
-    occ[0] = before + sum;
-    occ[1] = zlast < 0 ? 0 : zfirst;  // without objects: one plane of zeros
-    occ[2] = zlast < 0 ? 1 : zlast + 1;
-    occ[3] = 0;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, sum, o);
+      if (lane >= o) sum += v;
+    }
+    if (lane == 31) wsum[warp] = sum;
+    __syncthreads();
+    int before = 0;
+    for (int w = 0; w < warp; ++w) before += wsum[w];
+    if (z < N) out[4 + N + z] = before + sum - len;
+    if (z == N - 1) {
+      out[0] = before + sum;
+      out[1] = zlast < 0 ? 0 : zfirst;  // without objects: one plane of zeros
+      out[2] = zlast < 0 ? 1 : zlast + 1;
+      out[3] = 0;
+    }
   }
 }
 
@@ -475,13 +501,11 @@ __device__ __forceinline__ float object_moment(const GeomDev& g, const float4& o
   return ipow(hx, ea) * ipow(hy, eb) * ipow(hz, ec);
 }
 
-// Exponents (a, b, c) of the moment fields of a per-object plan (n = 0:
-// only F): blockIdx.y picks the field, gridded N^3 cells after the one before
+// Exponents (a, b, c) of the moment fields of a per-object plan: blockIdx.y picks the field, gridded N^3 cells after the one before
 // (one launch for all 16: on a small survey a launch per field leaves most
 // SMs idle, 128^3 and 2.2e5 objects 16 x 21 us).
 struct MomentExp {
-  int n = 0;
-  unsigned char e[kMaxFields][3];
+  unsigned long long a = 0, b = 0, c = 0;  // four bits per field
 };
 
 // One block per work item: up to chunk (<= kAccumChunk) objects of one tile (items in
@@ -502,8 +526,15 @@ struct MomentExp {
 // instead.  Both forms give the exact integer sum of the x, so the grid does
 // not depend on how the objects are split into items or in which order they
 // are added.
-template <int P, bool W2>
-__global__ void __launch_bounds__(kAccumThreads, W2 ? 2 : 4) k_tile_accum(GeomDev g, int ntx, int ntiles,
+//
+// SECOND: the second grid of an interlaced pair (geometry g; the tiles are
+// those of the first grid, whose origin is o1).  Its nodes lie half a cell
+// further, so an object's centre cell there is its centre cell in the first
+// grid or the one below: the region begins one cell lower, and the pair needs
+// one count, scan and scatter instead of two (360^3 PCS, 3.5e7 randoms: 1.1 ms
+// of 11.7).
+template <int P, bool W2, bool SECOND>
+__global__ void __launch_bounds__(kAccumThreads, W2 ? 2 : 4) k_tile_accum(GeomDev g, float3 o1, int ntx, int ntiles,
                                                                         const int* __restrict__ off,
                                                                         const int* __restrict__ items,
                                                                         const float4* __restrict__ xyzv,
@@ -527,9 +558,9 @@ __global__ void __launch_bounds__(kAccumThreads, W2 ? 2 : 4) k_tile_accum(GeomDe
   }
   // moment field of a per-object plan (0: F)
   const int fld = blockIdx.y;
-  const int ea = xe.n ? xe.e[fld][0] : 0, eb = xe.n ? xe.e[fld][1] : 0, ec = xe.n ? xe.e[fld][2] : 0;
+  const int ea = (int)(xe.a >> (4 * fld)) & 15, eb = (int)(xe.b >> (4 * fld)) & 15, ec = (int)(xe.c >> (4 * fld)) & 15;
   grid += (size_t)fld * g.N * g.N * g.N;
-  constexpr int kReg = reg_side<P>(), kReg3 = reg_cells<P>();
+  constexpr int kLow = SECOND ? 2 : 1, kReg = reg_side<P>(SECOND), kReg3 = kReg * kReg * kReg;
   static_assert(kAccumChunk * 262144ll < 2147483648ll, "the low words would wrap");
   extern __shared__ unsigned long long reg[];
   __shared__ int s_tile;
@@ -564,7 +595,7 @@ __global__ void __launch_bounds__(kAccumThreads, W2 ? 2 : 4) k_tile_accum(GeomDe
   const int a = off[t] + (item - items[t]) * chunk;
   const int b = min(off[t + 1], a + chunk);
   const int tx = t % ntx, ty = (t / ntx) % ntx, tz = t / (ntx * ntx);
-  const int lx0 = tx * kTile - 1, ly0 = ty * kTile - 1, lz0 = tz * kTile - 1;
+  const int lx0 = tx * kTile - kLow, ly0 = ty * kTile - kLow, lz0 = tz * kTile - kLow;
   // the item's objects are read twice: for the bounds, then for the taps
   float sa = 0.f, ma = 0.f;
   for (int i = a + threadIdx.x; i < b; i += kAccumThreads) {
@@ -595,7 +626,13 @@ __global__ void __launch_bounds__(kAccumThreads, W2 ? 2 : 4) k_tile_accum(GeomDe
     tap_weights<P>(uy, iy, wy);
     tap_weights<P>(uz, iz, wz);
     // taps relative to the region (periodic positions may lie one box away)
-    const int cx = ix + (P >= 3 ? 1 : 0), cy = iy + (P >= 3 ? 1 : 0), cz = iz + (P >= 3 ? 1 : 0);
+    int cx = ix + (P >= 3 ? 1 : 0), cy = iy + (P >= 3 ? 1 : 0), cz = iz + (P >= 3 ? 1 : 0);
+    if (SECOND) {  // the centre cell that chose the tile
+      const float sh = P == 3 ? 0.5f : 0.f;
+      cx = (int)floorf((o.x - o1.x) * g.invH + sh);
+      cy = (int)floorf((o.y - o1.y) * g.invH + sh);
+      cz = (int)floorf((o.z - o1.z) * g.invH + sh);
+    }
     const int rx = ix - (cx - wrapN(cx, N)) - lx0;
     const int ry = iy - (cy - wrapN(cy, N)) - ly0;
     const int rz = iz - (cz - wrapN(cz, N)) - lz0;
@@ -688,22 +725,23 @@ cudaError_t launch_combine_randoms(unsigned long long* grid, const unsigned long
 }
 
 // Both catalogs in one launch, nbg + nbr blocks (nbg = 0: no galaxies, nbr = 0:
-// the randoms are cached); part and bh: their nbg + nbr rows.
-cudaError_t launch_bin_count(const CatDev& gal, const CatDev& ran, int nbg, int nbr, const GeomDev& g, double* part,
-                             int* bh, int* err, cudaStream_t s) {
+// the randoms are cached); part and bh: their nbg + nbr rows; g2: NULL, or the
+// second grid of an interlaced pair, whose box limits are checked too.
+cudaError_t launch_bin_count(const CatDev& gal, const CatDev& ran, int nbg, int nbr, const GeomDev& g,
+                             const GeomDev* g2, double* part, int* bh, int* err, cudaStream_t s) {
   const int ntx = assign_tiles_per_axis(g.N);
   const int ntiles = ntx * ntx * ntx;
   const size_t sm = sizeof(int) * ntiles;
   const int nblk = nbg + nbr;
   if (g.assign == 2) {
     raise_smem_limit((const void*)k_bin_count<2>, sm);
-    k_bin_count<2><<<nblk, kBinThreads, sm, s>>>(gal, ran, nbg, g, ntx, ntiles, part, bh, err);
+    k_bin_count<2><<<nblk, kBinThreads, sm, s>>>(gal, ran, nbg, g, g2 ? 1 : 0, g2 ? *g2 : g, ntx, ntiles, part, bh, err);
   } else if (g.assign == 3) {
     raise_smem_limit((const void*)k_bin_count<3>, sm);
-    k_bin_count<3><<<nblk, kBinThreads, sm, s>>>(gal, ran, nbg, g, ntx, ntiles, part, bh, err);
+    k_bin_count<3><<<nblk, kBinThreads, sm, s>>>(gal, ran, nbg, g, g2 ? 1 : 0, g2 ? *g2 : g, ntx, ntiles, part, bh, err);
   } else {
     raise_smem_limit((const void*)k_bin_count<4>, sm);
-    k_bin_count<4><<<nblk, kBinThreads, sm, s>>>(gal, ran, nbg, g, ntx, ntiles, part, bh, err);
+    k_bin_count<4><<<nblk, kBinThreads, sm, s>>>(gal, ran, nbg, g, g2 ? 1 : 0, g2 ? *g2 : g, ntx, ntiles, part, bh, err);
   }
   return cudaGetLastError();
 }
@@ -727,9 +765,9 @@ int accum_chunk(long long nobj, int nsm) {
 }
 
 cudaError_t launch_scan_tiles(const int* cnt, int ntiles, int* off, int* items, int chunk, cudaStream_t s,
-                              const GeomDev& g, const int* more, int* occ) {
+                              const GeomDev& g, const int* more, int* occ, int* occ2) {
   k_scan_tiles<<<1, 1024, 0, s>>>(cnt, ntiles, off, items, chunk, more, assign_tiles_per_axis(g.N), g.N,
-                                  g.assign == 4 ? kTile + 1 : kTile, g.periodic, occ);
+                                  g.assign == 4 ? kTile + 1 : kTile, g.periodic, occ, occ2);
   return cudaGetLastError();
 }
 
@@ -754,18 +792,20 @@ cudaError_t launch_bin_scatter(const CatDev& gal, const CatDev& ran, int nbg, in
   return cudaGetLastError();
 }
 
+// first: NULL, or the first grid of the interlaced pair whose second grid is g;
 // nobj: the objects scattered into tile order (bounds the number of items);
 // mt: the moment table of a per-object plan, or NULL; lab: NULL, or where the
 // L^ab sums of the nlab rows of labpart go.
 cudaError_t launch_tile_accum(const GeomDev& g, const int* off, const int* items, long long nobj, int chunk,
                               const float4* xyzv, const float* vw2, unsigned long long* grid,
-                              unsigned long long* gridw, cudaStream_t s, const MomentTable* mt,
+                              unsigned long long* gridw, cudaStream_t s, const GeomDev* first, const MomentTable* mt,
                               const double* labpart, int nlab, double* lab) {
   MomentExp xe;
-  if (mt) {
-    xe.n = mt->nfields;
-    for (int q = 0; q < mt->nfields; ++q)
-      for (int a = 0; a < 3; ++a) xe.e[q][a] = mt->e[q][a];
+  static_assert(kMaxFields <= 16, "four bits per field in 64");
+  for (int q = 0; mt && q < mt->nfields; ++q) {
+    xe.a |= (unsigned long long)mt->e[q][0] << (4 * q);
+    xe.b |= (unsigned long long)mt->e[q][1] << (4 * q);
+    xe.c |= (unsigned long long)mt->e[q][2] << (4 * q);
   }
   const int ntx = assign_tiles_per_axis(g.N);
   const int ntiles = ntx * ntx * ntx;
@@ -775,20 +815,23 @@ cudaError_t launch_tile_accum(const GeomDev& g, const int* off, const int* items
   if (nitems > INT32_MAX) return cudaErrorInvalidValue;
   const bool w2 = gridw != nullptr;
   const dim3 blocks((unsigned)nitems, mt ? mt->nfields : 1);
-#define FKP_TA(PP, WW)                                                                                 \
-  do {                                                                                                 \
-    const size_t sm = sizeof(unsigned long long) * reg_cells<PP>() * (WW ? 2 : 1);                     \
-    raise_smem_limit((const void*)k_tile_accum<PP, WW>, sm);                                           \
-    k_tile_accum<PP, WW><<<blocks, kAccumThreads, sm, s>>>(g, ntx, ntiles, off, items, xyzv, vw2, grid, \
-                                                           gridw, chunk, xe, labpart, nlab, lab);      \
+#define FKP_TA(PP, WW, SS)                                                                               \
+  do {                                                                                                   \
+    const size_t sm = sizeof(unsigned long long) * reg_cells<PP>(SS) * (WW ? 2 : 1);                     \
+    raise_smem_limit((const void*)k_tile_accum<PP, WW, SS>, sm);                                         \
+    k_tile_accum<PP, WW, SS><<<blocks, kAccumThreads, sm, s>>>(g, o1, ntx, ntiles, off, items, xyzv, vw2, grid, \
+                                                               gridw, chunk, xe, labpart, nlab, lab);    \
   } while (0)
-  if (g.assign == 2) {
-    if (w2) FKP_TA(2, true); else FKP_TA(2, false);
-  } else if (g.assign == 3) {
-    if (w2) FKP_TA(3, true); else FKP_TA(3, false);
-  } else {
-    if (w2) FKP_TA(4, true); else FKP_TA(4, false);
-  }
+#define FKP_TAP(PP)                                                        \
+  do {                                                                     \
+    if (first) { if (w2) FKP_TA(PP, true, true); else FKP_TA(PP, false, true); } \
+    else { if (w2) FKP_TA(PP, true, false); else FKP_TA(PP, false, false); }     \
+  } while (0)
+  const float3 o1 = first ? make_float3(first->ox, first->oy, first->oz) : make_float3(0.f, 0.f, 0.f);
+  if (g.assign == 2) FKP_TAP(2);
+  else if (g.assign == 3) FKP_TAP(3);
+  else FKP_TAP(4);
+#undef FKP_TAP
 #undef FKP_TA
   return cudaGetLastError();
 }

@@ -105,3 +105,25 @@ def test_batch_of_mocks_in_different_places():
         one = plan.power(g, r)
         for k in ("P0", "P2", "P4", "P4b"):
             assert np.array_equal(b[k], one[k], equal_nan=True), k
+
+
+@pytest.mark.parametrize("assign", [2, 3, 4])
+@pytest.mark.parametrize("N,periodic", [(64, False), (64, True), (60, True)])
+def test_second_grid_of_a_pair_is_the_shifted_grid(N, periodic, assign):
+    """The second grid of an interlaced pair, filled from the first grid's
+    tiles, equals bit for bit the grid of a plan whose origin is half a cell
+    further (integer sums of the same rounded taps), with objects on both sides
+    of every tile face and, when periodic, around the box."""
+    import paper_1506_02729_gb300 as fkp
+    lo, hi = (0.0, 64.0) if periodic else (4.0, 59.0)
+    box = [_cell((lo,) * 3, (hi,) * 3, N=64)]
+    gal, ran = _cloud(box, 3000, 6), _cloud(box, 30000, 7)
+    g, r = to_device(gal), to_device(ran)
+    geom = dict(L=L, N=N, assign=assign, origin=(0.0, 0.0, 0.0), observer=(480.0, 480.0, 480.0), P_fkp=1e4,
+                periodic=periodic)
+    kf = 2 * math.pi / L
+    pair = fkp.Plan(dict(geom, interlace=True), (0.5 * kf, kf, 8), bshells=(3, 3, 3, 4), want=1 | 16)
+    half = 0.5 * L / N
+    one = fkp.Plan(dict(geom, origin=(half,) * 3), (0.5 * kf, kf, 8), bshells=(3, 3, 3, 4), want=1 | 16)
+    for a, b in zip(pair.grid(g, r, which=1, with_w=True), one.grid(g, r, with_w=True)):
+        assert np.array_equal(a, b)
