@@ -282,6 +282,7 @@ fkp::Plan::~Plan() {
   if (d_xyzv) cudaFree(d_xyzv);
   if (d_vw2) cudaFree(d_vw2);
   if (h_pinned) cudaFreeHost(h_pinned);
+  if (b_pinned) cudaFreeHost(b_pinned);
   if (batch_mem) cudaFree(batch_mem);
   for (auto& e : ev) if (e) cudaEventDestroy(e);
   if (ev_fork) cudaEventDestroy(ev_fork);
@@ -566,8 +567,8 @@ extern "C" int fkp_plan_create(void* vctx, const fkp_geometry_t* geom, const fkp
   P->reach_w.ztiles = d_ztiles + zt.size();
   P->d_scpart = (double*)A(sizeof(double) * SC_NSUM * 2 * P->nblk_cat);
   P->d_labpart = (double*)A(sizeof(double) * LAB_NSUM * P->nblk_cat);
-  P->d_ds = (double*)A(sizeof(double) * (DS_COUNT + LAB_NSUM + 8));
-  P->d_err = (int*)A(sizeof(int) * 4);
+  double* d_res = (double*)A(sizeof(double) * result_doubles(pb->nbins));
+  P->set_result(d_res);
   {
     const int ntx = assign_tiles_per_axis(N);
     P->ntiles = ntx * ntx * ntx;
@@ -578,8 +579,6 @@ extern "C" int fkp_plan_create(void* vctx, const fkp_geometry_t* geom, const fkp
   P->d_bhist = (int*)A(sizeof(int) * (size_t)P->ntiles * 2 * P->ctx->nsm);
   P->d_zpart = (double*)A(sizeof(double) * BQ_N * pb->nbins * (size_t)P->nblk_z);
   P->d_zpartc = (int*)A(sizeof(int) * pb->nbins * (size_t)P->nblk_z);
-  P->d_bins = (double*)A(sizeof(double) * BQ_N * pb->nbins);
-  P->d_binc = (long long*)A(sizeof(long long) * pb->nbins);
   if (!ok) {
     const size_t tot = P->bytes_total;
     delete P;
@@ -600,8 +599,7 @@ extern "C" int fkp_plan_create(void* vctx, const fkp_geometry_t* geom, const fkp
   CK(cudaMemcpy(d_ztiles, zt.data(), sizeof(int) * zt.size(), cudaMemcpyHostToDevice));
   CK(cudaMemcpy(d_ztiles + zt.size(), ztw.data(), sizeof(int) * ztw.size(), cudaMemcpyHostToDevice));
   CK(cudaMemcpy(P->d_hph, hph.data(), sizeof(float2) * N, cudaMemcpyHostToDevice));
-  const size_t hbytes = sizeof(double) * (BQ_N * pb->nbins + pb->nbins + DS_COUNT + LAB_NSUM + 8) + 64;
-  CK(cudaMallocHost(&P->h_pinned, hbytes));
+  CK(cudaMallocHost(&P->h_pinned, sizeof(double) * result_doubles(pb->nbins)));
   for (auto& e : P->ev) CK(cudaEventCreate(&e));
   CK(cudaEventCreateWithFlags(&P->ev_fork, cudaEventDisableTiming));
   CK(cudaEventCreateWithFlags(&P->ev_join, cudaEventDisableTiming));
@@ -937,19 +935,13 @@ int fkp::enqueue_fft_bin(Plan* P, const unsigned long long* gq, const float* gf,
   return FKP_OK;
 }
 
-// Copies bins and scalars back, synchronizes and fills out.
-int fkp::finish_power(Plan* P, cudaStream_t s, fkp_power_out* out, bool have_scalars, double I22u, double N0u) {
+// Fills out from the host copy h of a result block (Plan::set_result).
+static int fill_power(const Plan* P, const double* h, fkp_power_out* out, bool have_scalars, double I22u, double N0u) {
   const int nb = P->pb.nbins;
-  double* h = static_cast<double*>(P->h_pinned);
-  double* hb = h;
-  long long* hc = reinterpret_cast<long long*>(h + BQ_N * nb);
-  double* hds = h + BQ_N * nb + nb;
-  int* herr = reinterpret_cast<int*>(hds + DS_COUNT + LAB_NSUM + 8);
-  CK(cudaMemcpyAsync(hb, P->d_bins, sizeof(double) * BQ_N * nb, cudaMemcpyDeviceToHost, s));
-  CK(cudaMemcpyAsync(hc, P->d_binc, sizeof(long long) * nb, cudaMemcpyDeviceToHost, s));
-  CK(cudaMemcpyAsync(hds, P->d_ds, sizeof(double) * (DS_COUNT + LAB_NSUM), cudaMemcpyDeviceToHost, s));
-  CK(cudaMemcpyAsync(herr, P->d_err, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
-  CK(cudaStreamSynchronize(s));
+  const double* hb = h;
+  const long long* hc = reinterpret_cast<const long long*>(h + BQ_N * nb);
+  const double* hds = h + BQ_N * nb + nb;
+  const int* herr = reinterpret_cast<const int*>(hds + DS_COUNT + LAB_NSUM + 8);
   if (herr[1] != 0)
     return set_error(FKP_ETIMEOUT, "a bounded device-side wait for a tile copy gave up (flags 0x%x)", herr[1]);
   if (have_scalars && herr[0] != 0)
@@ -994,9 +986,19 @@ int fkp::finish_power(Plan* P, cudaStream_t s, fkp_power_out* out, bool have_sca
     if (out->P6b) out->P6b[b] = n > 0 && split ? 13.0 * s60 / n / I22 : nan;
     if (out->P8b) out->P8b[b] = n > 0 && split ? 17.0 * s80 / n / I22 : nan;
   }
-  float t = 0.f;
   for (int i = 0; i < 8; ++i) out->timing_ms[i] = 0.f;
   out->graph = 0;
+  return FKP_OK;
+}
+
+// Copies bins, scalars and flags back (one block, one copy: four copies cost
+// a small survey 15 us), synchronizes and fills out.
+int fkp::finish_power(Plan* P, cudaStream_t s, fkp_power_out* out, bool have_scalars, double I22u, double N0u) {
+  CK(cudaMemcpyAsync(P->h_pinned, P->d_bins, sizeof(double) * result_doubles(P->pb.nbins), cudaMemcpyDeviceToHost, s));
+  CK(cudaStreamSynchronize(s));
+  const int rc = fill_power(P, static_cast<const double*>(P->h_pinned), out, have_scalars, I22u, N0u);
+  if (rc || !out) return rc;
+  float t = 0.f;
   if (cudaEventElapsedTime(&t, P->ev[0], P->ev[1]) == cudaSuccess) out->timing_ms[0] = t;
   if (cudaEventElapsedTime(&t, P->ev[1], P->ev[2]) == cudaSuccess) out->timing_ms[1] = t;
   if (cudaEventElapsedTime(&t, P->ev[2], P->ev[3]) == cudaSuccess) out->timing_ms[2] = t;
@@ -1128,7 +1130,7 @@ extern "C" int fkp_grid(void* plan, const fkp_catalog_t* gal, const fkp_catalog_
 // Per-mock element counts of the fused batch workspace.
 namespace {
 struct BatchSizes {
-  size_t grid, s1, s2, zpart, zpartc, bins, binc, ds, err, occ;
+  size_t grid, s1, s2, zpart, zpartc, res, occ;
 };
 BatchSizes batch_sizes(const fkp::Plan* P) {
   const size_t N = (size_t)P->g.N, half = fkp::field_elems(P->g.N);
@@ -1138,10 +1140,7 @@ BatchSizes batch_sizes(const fkp::Plan* P) {
   z.s2 = half * P->mt.ngroups;
   z.zpart = (size_t)BQ_N * P->pb.nbins * P->nblk_z;
   z.zpartc = (size_t)P->pb.nbins * P->nblk_z;
-  z.bins = (size_t)BQ_N * P->pb.nbins;
-  z.binc = (size_t)P->pb.nbins;
-  z.ds = DS_COUNT + LAB_NSUM + 8;
-  z.err = 4;
+  z.res = result_doubles(P->pb.nbins);
   z.occ = occ_ints(P->g.N);
   return z;
 }
@@ -1154,9 +1153,8 @@ static int reserve_batch(fkp::Plan* P, int nmock) {
   if (P->batch_cap >= nmock) return FKP_OK;
   const BatchSizes z = batch_sizes(P);
   const size_t K = (size_t)nmock;
-  const size_t parts[10] = {align256(K * z.grid * 8),  align256(K * z.s1 * 8),     align256(K * z.s2 * 8),
-                           align256(K * z.zpart * 8), align256(K * z.zpartc * 4), align256(K * z.bins * 8),
-                           align256(K * z.binc * 8),  align256(K * z.ds * 8),     align256(K * z.err * 4),
+  const size_t parts[7] = {align256(K * z.grid * 8),  align256(K * z.s1 * 8),     align256(K * z.s2 * 8),
+                           align256(K * z.zpart * 8), align256(K * z.zpartc * 4), align256(K * z.res * 8),
                            align256(K * z.occ * 4)};
   size_t tot = 0;
   for (size_t b : parts) tot += b;
@@ -1167,6 +1165,13 @@ static int reserve_batch(fkp::Plan* P, int nmock) {
   P->batch_mem = nullptr;
   P->batch_cap = 0;
   P->batch_bytes = 0;
+  if (P->b_pinned) cudaFreeHost(P->b_pinned);
+  P->b_pinned = nullptr;
+  if (cudaMallocHost(&P->b_pinned, K * z.res * 8) != cudaSuccess) {
+    cudaGetLastError();
+    P->b_pinned = nullptr;
+    return set_error(FKP_ENOMEM, "cannot allocate the host buffer of a batch of %d mocks", nmock);
+  }
   if (cudaMalloc(&P->batch_mem, tot) != cudaSuccess) {
     cudaGetLastError();
     P->batch_mem = nullptr;
@@ -1178,10 +1183,7 @@ static int reserve_batch(fkp::Plan* P, int nmock) {
   P->b_S2 = reinterpret_cast<float2*>(m);                m += parts[2];
   P->b_zpart = reinterpret_cast<double*>(m);             m += parts[3];
   P->b_zpartc = reinterpret_cast<int*>(m);               m += parts[4];
-  P->b_bins = reinterpret_cast<double*>(m);              m += parts[5];
-  P->b_binc = reinterpret_cast<long long*>(m);           m += parts[6];
-  P->b_ds = reinterpret_cast<double*>(m);                m += parts[7];
-  P->b_err = reinterpret_cast<int*>(m);                  m += parts[8];
+  P->b_res = reinterpret_cast<double*>(m);               m += parts[5];
   P->b_occ = reinterpret_cast<int*>(m);
   P->batch_cap = nmock;
   P->batch_bytes = tot;
@@ -1205,8 +1207,7 @@ extern "C" int fkp_power_batch(void* plan, int nmock, const fkp_catalog_t* gals,
   // gridding, mock by mock (each launch shaped by its own catalogs), into the
   // mock's grid, scalars and flags
   unsigned long long* const grid0 = P->d_grid;
-  double* const ds0 = P->d_ds;
-  int* const err0 = P->d_err;
+  double* const res0 = P->d_bins;
   int* const occ0 = P->d_occ;
   CK(cudaEventRecord(P->ev[9], s));
   for (int k = 0; k < nmock; ++k) {
@@ -1215,19 +1216,21 @@ extern "C" int fkp_power_batch(void* plan, int nmock, const fkp_catalog_t* gals,
     if (!rc) rc = randoms_of(P, rans ? &rans[k] : nullptr, r, s);
     if (rc) return rc;
     P->d_grid = P->b_grid + k * z.grid;
-    P->d_ds = P->b_ds + k * z.ds;
-    P->d_err = P->b_err + k * z.err;
+    P->set_result(P->b_res + k * z.res);
     P->d_occ = P->b_occ + k * z.occ;
     rc = enqueue_grids(P, g, r, s);
     P->d_occ = occ0;
     P->d_grid = grid0;
-    P->d_ds = ds0;
-    P->d_err = err0;
+    P->set_result(res0);
     if (rc) return rc;
   }
   // the three FFT passes and the bin reduction: one launch each for all mocks
   // (blockIdx.z / blockIdx.y = mock); bounded-wait flags go to mock 0's word
-  int* perr = P->b_err + 1;
+  P->set_result(P->b_res);
+  int* perr = P->d_err + 1;
+  double* const bins = P->d_bins;
+  long long* const binc = P->d_binc;
+  P->set_result(res0);
   MockBatch mx;
   mx.n = nmock; mx.in = (long long)z.grid; mx.out = (long long)z.s1; mx.occ = (int)z.occ;
   CK(launch_xpass(P->b_grid, nullptr, P->g, P->mt, P->fp, P->d_tw, P->b_S1, P->ctx->nsm, s, P->reach, P->b_occ, P->sched.x_mult,
@@ -1245,31 +1248,21 @@ extern "C" int fkp_power_batch(void* plan, int nmock, const fkp_catalog_t* gals,
   CK(launch_zpass(P->b_S2, P->g, P->mt, P->fp, P->d_tw, zp, P->reach, P->b_zpart, P->b_zpartc, perr, s, P->ctx->nsm,
                   P->sched.z_threads, mz));
   CK(launch_reduce_bins(P->b_zpart, P->b_zpartc, zpass_blocks(P->reach, P->sched.z_threads, P->ctx->nsm), P->pb.nbins,
-                        P->b_bins, P->b_binc, s, nmock, (long long)z.zpart, (long long)z.zpartc));
+                        bins, binc, s, nmock, (long long)z.zpart, (long long)z.zpartc, (long long)z.res));
   CK(cudaEventRecord(P->ev[5], s));
-  // bins and scalars back, mock by mock
-  double* const bins0 = P->d_bins;
-  long long* const binc0 = P->d_binc;
+  // every mock's result block back in one copy
+  CK(cudaMemcpyAsync(P->b_pinned, P->b_res, (size_t)nmock * z.res * 8, cudaMemcpyDeviceToHost, s));
+  CK(cudaStreamSynchronize(s));
   float tg = 0.f, tx = 0.f, ty = 0.f, tz = 0.f, tt = 0.f;
+  cudaEventElapsedTime(&tg, P->ev[9], P->ev[2]);
+  cudaEventElapsedTime(&tx, P->ev[2], P->ev[3]);
+  cudaEventElapsedTime(&ty, P->ev[3], P->ev[4]);
+  cudaEventElapsedTime(&tz, P->ev[4], P->ev[5]);
+  cudaEventElapsedTime(&tt, P->ev[9], P->ev[5]);
+  cudaGetLastError();
   for (int k = 0; k < nmock; ++k) {
-    P->d_bins = P->b_bins + k * z.bins;
-    P->d_binc = P->b_binc + k * z.binc;
-    P->d_ds = P->b_ds + k * z.ds;
-    P->d_err = P->b_err + k * z.err;
-    rc = finish_power(P, s, outs ? &outs[k] : nullptr, true, 0, 0);
-    P->d_bins = bins0;
-    P->d_binc = binc0;
-    P->d_ds = ds0;
-    P->d_err = err0;
+    rc = fill_power(P, static_cast<const double*>(P->b_pinned) + k * z.res, outs ? &outs[k] : nullptr, true, 0, 0);
     if (rc) return rc;
-    if (k == 0) {
-      cudaEventElapsedTime(&tg, P->ev[9], P->ev[2]);
-      cudaEventElapsedTime(&tx, P->ev[2], P->ev[3]);
-      cudaEventElapsedTime(&ty, P->ev[3], P->ev[4]);
-      cudaEventElapsedTime(&tz, P->ev[4], P->ev[5]);
-      cudaEventElapsedTime(&tt, P->ev[9], P->ev[5]);
-      cudaGetLastError();
-    }
     if (outs) {
       // stage times of the whole batch
       float* t = outs[k].timing_ms;

@@ -30,6 +30,9 @@ struct Context {
   std::map<std::pair<int, int>, PassSchedule> schedules;  // (N, lmax) -> schedule
 };
 
+// 8-byte words of a plan's result block (Plan::set_result).
+inline size_t result_doubles(int nbins) { return (size_t)(BQ_N + 1) * nbins + DS_COUNT + LAB_NSUM + 8 + 2; }
+
 struct Plan {
   Context* ctx = nullptr;
   fkp_geometry_t geom{};
@@ -68,8 +71,16 @@ struct Plan {
   size_t sort_cap = 0;
   double* d_zpart = nullptr;
   int* d_zpartc = nullptr;
+  // result block, copied back whole: [BQ_N][nbins] bin sums, [nbins] counts,
+  // the scalars and L^ab sums (d_ds), four flag words (d_err)
   double* d_bins = nullptr;
   long long* d_binc = nullptr;
+  void set_result(double* base) {
+    d_bins = base;
+    d_binc = reinterpret_cast<long long*>(base + BQ_N * pb.nbins);
+    d_ds = base + (BQ_N + 1) * pb.nbins;
+    d_err = reinterpret_cast<int*>(d_ds + DS_COUNT + LAB_NSUM + 8);
+  }
 
   // bispectrum workspace and tables
   int ntri = 0;
@@ -122,9 +133,9 @@ struct Plan {
   size_t batch_bytes = 0;
   unsigned long long* b_grid = nullptr;
   float2 *b_S1 = nullptr, *b_S2 = nullptr;
-  double *b_zpart = nullptr, *b_bins = nullptr, *b_ds = nullptr;
-  int *b_zpartc = nullptr, *b_err = nullptr, *b_occ = nullptr;
-  long long* b_binc = nullptr;
+  double *b_zpart = nullptr, *b_res = nullptr;
+  int *b_zpartc = nullptr, *b_occ = nullptr;
+  void* b_pinned = nullptr;  // host copy of the result blocks
 
   std::vector<void*> buffers;
   size_t bytes_total = 0;
@@ -213,7 +224,7 @@ int zpass_blocks(const PassReach& pr, int nt, int nsm);
 std::vector<int> reach_tiles(int N, int r2, PassReach& pr);
 cudaError_t launch_reduce_bins(const double* part, const int* partc, int nblk, int nbins, double* out,
                                long long* outc, cudaStream_t s, int nmock = 1, long long pstride = 0,
-                               long long pcstride = 0);
+                               long long pcstride = 0, long long ostride = 0);
 
 // tensor-core triangle contraction (k_contract_tc.cu): a tile is 128 pairs
 // times a run of n field rows from r0 (its accumulator columns start at col

@@ -79,6 +79,7 @@ struct BispState {
   int nzjobs = 0, nyjobs = 0;
   int4 *d_zjobs = nullptr, *d_yjobs = nullptr;
   int* d_kmax = nullptr;
+  void* h_out = nullptr;             // host copy of d_T, d_shell, d_shellc (one allocation)
 };
 
 __device__ __forceinline__ int wrap_mode(int n, int N) { return n < 0 ? n + N : n; }
@@ -710,11 +711,11 @@ int bisp_plan_init(Plan* P) {
   st->d_I = (float*)A(sizeof(float) * (size_t)st->nl * S * N3);
   st->d_items = (ContractItem*)A(sizeof(ContractItem) * std::max<size_t>(1, st->items.size()));
   st->d_cpart = (double*)A(sizeof(double) * (size_t)st->nslices * std::max(1, ntri) * st->nq);
-  st->d_T = (double*)A(sizeof(double) * std::max(1, ntri) * st->nq);
+  st->d_T = (double*)A(sizeof(double) * (std::max(1, ntri) * st->nq + (BQ_N + 1) * S));
+  st->d_shell = st->d_T ? st->d_T + std::max(1, ntri) * st->nq : nullptr;
+  st->d_shellc = reinterpret_cast<long long*>(st->d_T ? st->d_shell + BQ_N * S : nullptr);
   st->d_spart = (double*)A(sizeof(double) * BQ_N * S * (size_t)P->nblk_z);
   st->d_spartc = (int*)A(sizeof(int) * S * (size_t)P->nblk_z);
-  st->d_shell = (double*)A(sizeof(double) * BQ_N * S);
-  st->d_shellc = (long long*)A(sizeof(long long) * S);
   if (st->tc_groups > 0) {
     st->d_pairs = (short2*)A(sizeof(short2) * tcp.pairs.size());
     st->d_groups = (TcGroup*)A(sizeof(TcGroup) * tcp.groups.size());
@@ -731,6 +732,7 @@ int bisp_plan_init(Plan* P) {
     tw[m] = make_float2((float)std::cos(a), (float)-std::sin(a));
   }
   BCK(cudaMemcpy(st->d_tw, tw.data(), sizeof(float2) * M, cudaMemcpyHostToDevice));
+  BCK(cudaMallocHost(&st->h_out, sizeof(double) * (std::max(1, ntri) * st->nq + (BQ_N + 1) * S)));
   BCK(cudaMemcpy(st->d_slut, slut.data(), st->nsh2, cudaMemcpyHostToDevice));
   if (!zj.empty()) BCK(cudaMemcpy(st->d_zjobs, zj.data(), sizeof(int4) * zj.size(), cudaMemcpyHostToDevice));
   if (!yj.empty()) BCK(cudaMemcpy(st->d_yjobs, yj.data(), sizeof(int4) * yj.size(), cudaMemcpyHostToDevice));
@@ -748,6 +750,7 @@ int bisp_plan_init(Plan* P) {
 
 void bisp_plan_free(Plan* P) {
   bisp_drop_graph(P);
+  if (P->bisp && static_cast<BispState*>(P->bisp)->h_out) cudaFreeHost(static_cast<BispState*>(P->bisp)->h_out);
   delete static_cast<BispState*>(P->bisp);
   P->bisp = nullptr;
 }
@@ -920,11 +923,10 @@ extern "C" int fkp_bispectrum(void* plan, const fkp_catalog_t* gal, const fkp_ca
   const int N = P->g.N, S = st->S;
   const long long N3 = (long long)N * N * N;
   const int ntri = P->ntri, nout = std::max(1, ntri) * st->nq;
-  std::vector<double> T(nout, 0.0), sh(BQ_N * S);
-  std::vector<long long> shc(S);
-  BCK(cudaMemcpyAsync(T.data(), st->d_T, sizeof(double) * nout, cudaMemcpyDeviceToHost, s));
-  BCK(cudaMemcpyAsync(sh.data(), st->d_shell, sizeof(double) * BQ_N * S, cudaMemcpyDeviceToHost, s));
-  BCK(cudaMemcpyAsync(shc.data(), st->d_shellc, sizeof(long long) * S, cudaMemcpyDeviceToHost, s));
+  // triangle sums and shell sums back in one copy, read after finish_power's synchronization
+  BCK(cudaMemcpyAsync(st->h_out, st->d_T, sizeof(double) * (nout + (BQ_N + 1) * S), cudaMemcpyDeviceToHost, s));
+  const double *T = static_cast<const double*>(st->h_out), *sh = T + nout;
+  const long long* shc = reinterpret_cast<const long long*>(sh + BQ_N * S);
   rc = finish_power(P, s, pout, true, 0, 0);
   if (rc) return rc;
   float t = 0.f;
@@ -935,8 +937,7 @@ extern "C" int fkp_bispectrum(void* plan, const fkp_catalog_t* gal, const fkp_ca
     if (cudaEventElapsedTime(&t, P->ev[0], P->ev[8]) == cudaSuccess) pout->timing_ms[7] = t;
   }
   // scalars for the finalize
-  double hds[DS_COUNT];
-  BCK(cudaMemcpy(hds, P->d_ds, sizeof(double) * DS_COUNT, cudaMemcpyDeviceToHost));
+  const double* hds = static_cast<const double*>(P->h_pinned) + (BQ_N + 1) * P->pb.nbins;
   const double I33 = hds[DS_I33], S3 = hds[DS_S3];
   if (!bout) return FKP_OK;
   bout->I33 = I33;

@@ -11,15 +11,15 @@ namespace fkp {
 
 // One block per (quantity, bin): fixed-order FP64 tree sum over the blocks.
 // blockIdx.y picks the mock of a fused launch (partials at pstride / pcstride,
-// bins contiguous per mock).
+// bins and counts at ostride, in 8-byte words).
 __global__ void __launch_bounds__(256) k_reduce_bins(const double* __restrict__ part, const int* __restrict__ partc,
                                                      int nblk, int nbins, double* __restrict__ out,
                                                      long long* __restrict__ outc, long long pstride,
-                                                     long long pcstride) {
+                                                     long long pcstride, long long ostride) {
   part += (long long)blockIdx.y * pstride;
   partc += (long long)blockIdx.y * pcstride;
-  out += (long long)blockIdx.y * BQ_N * nbins;
-  outc += (long long)blockIdx.y * nbins;
+  out += (long long)blockIdx.y * ostride;
+  outc += (long long)blockIdx.y * ostride;
   __shared__ double sh[32];
   const int row = blockIdx.x;  // 0 .. BQ_N*nbins (float rows) then nbins (count rows)
   double s = 0.0;
@@ -60,9 +60,9 @@ cudaError_t launch_wait_selftest(unsigned polls, int* flag, cudaStream_t s) {
 }
 
 cudaError_t launch_reduce_bins(const double* part, const int* partc, int nblk, int nbins, double* out, long long* outc,
-                               cudaStream_t s, int nmock, long long pstride, long long pcstride) {
+                               cudaStream_t s, int nmock, long long pstride, long long pcstride, long long ostride) {
   k_reduce_bins<<<dim3((BQ_N + 1) * nbins, nmock), 256, 0, s>>>(part, partc, nblk, nbins, out, outc, pstride,
-                                                                pcstride);
+                                                                pcstride, ostride);
   return cudaGetLastError();
 }
 
