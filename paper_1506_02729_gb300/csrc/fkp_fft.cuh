@@ -15,6 +15,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <utility>
+
 namespace fkp {
 
 struct FftPlan {
@@ -108,8 +110,67 @@ __device__ __forceinline__ void dft8(float2* v) {
   }
 }
 
+// Twiddles of the composite DFTs as constants: cos and sin of 2 pi m / R by
+// their power series in FP64, rounded to FP32.
+constexpr double cos_sin_series(double x, bool want_sin) {
+  double term = want_sin ? x : 1.0, sum = term;
+  for (int n = want_sin ? 1 : 0, k = 0; k < 18; ++k, n += 2) {
+    term *= -x * x / ((n + 1.0) * (n + 2.0));
+    sum += term;
+  }
+  return sum;
+}
+template <int R, int M>
+struct TwC {
+  static constexpr double a = 6.283185307179586476925 * (2 * M > R ? M - R : M) / R;  // in (-pi, pi]
+  static constexpr float c = (float)cos_sin_series(a, false), s = (float)cos_sin_series(a, true);
+};
+
+template <class F, int... I>
+__device__ __forceinline__ void static_for_(F&& f, std::integer_sequence<int, I...>) {
+  (f(std::integral_constant<int, I>{}), ...);
+}
+template <int N, class F>
+__device__ __forceinline__ void static_for(F&& f) {
+  static_for_(f, std::make_integer_sequence<int, N>{});
+}
+
+template <int R, int DIR>
+__device__ __forceinline__ void dftR(float2* v);
+
+// Length R1 R2 in registers: input n = R2 n1 + n2, output k = k1 + R1 k2.
+template <int R1, int R2, int DIR>
+__device__ __forceinline__ void dft_comp(float2* v) {
+  constexpr int R = R1 * R2;
+  static_for<R2>([&](auto i2) {
+    constexpr int n2 = decltype(i2)::value;
+    float2 u[R1];
+    static_for<R1>([&](auto i1) { u[decltype(i1)::value] = v[R2 * decltype(i1)::value + n2]; });
+    dftR<R1, DIR>(u);
+    static_for<R1>([&](auto i1) {
+      constexpr int k1 = decltype(i1)::value, m = (n2 * k1) % R;
+      v[R2 * k1 + n2] = m == 0 ? u[k1] : cmul(u[k1], make_float2(TwC<R, m>::c, DIR * TwC<R, m>::s));
+    });
+  });
+  float2 o[R];
+  static_for<R1>([&](auto i1) {
+    constexpr int k1 = decltype(i1)::value;
+    float2 t[R2];
+    static_for<R2>([&](auto i2) { t[decltype(i2)::value] = v[R2 * k1 + decltype(i2)::value]; });
+    dftR<R2, DIR>(t);
+    static_for<R2>([&](auto i2) { o[k1 + R1 * decltype(i2)::value] = t[decltype(i2)::value]; });
+  });
+  static_for<R>([&](auto i) { v[decltype(i)::value] = o[decltype(i)::value]; });
+}
+
 template <int R, int DIR>
 __device__ __forceinline__ void dftR(float2* v) {
+  if constexpr (R == 12) { dft_comp<3, 4, DIR>(v); return; }
+  if constexpr (R == 15) { dft_comp<3, 5, DIR>(v); return; }
+  if constexpr (R == 16) { dft_comp<4, 4, DIR>(v); return; }
+  if constexpr (R == 24) { dft_comp<3, 8, DIR>(v); return; }
+  if constexpr (R == 32) { dft_comp<4, 8, DIR>(v); return; }
+  if constexpr (R > 8) return;
   if (R == 2) dft2<DIR>(v);
   else if (R == 3) dft3<DIR>(v);
   else if (R == 4) dft4<DIR>(v);
@@ -357,6 +418,41 @@ __device__ __forceinline__ void fft_ct_fused(float2* a, float2* b, const float2*
 #pragma unroll
     for (int r = 0; r < R; ++r) f((j0 + r * NS) / JT, v[r]);
   }
+}
+
+// A transform of N = R0 R1 in two stages with both radices in registers: P
+// interleaved pencils, thread (p, j).  The first stage takes elements j + r R1
+// (r < R0, j < R1) and leaves its results in buf, the second (j < R0) reads
+// those and gives the transform's elements j + r R0 (r < R1): one crossing of
+// shared memory, where radix 8, 5 and 3 stages make two or three.
+// For even R0 rows 2i and 2i + 1 of buf swap when the butterfly that wrote them
+// is odd: butterflies j and j + 1 of a half-warp then write rows of both
+// parities (both halves of the banks).
+template <int N>
+struct TwoStage {
+  static constexpr int R0 = N == 360 ? 15 : (N == 192 ? 12 : (N <= 128 ? 8 : 16)), R1 = N / R0;
+  static constexpr int kTY = R1 > R0 ? R1 : R0;
+};
+template <int N, int P, int DIR>
+__device__ __forceinline__ void two_stage_first(float2* v, float2* buf, int p, int j) {
+  constexpr int R0 = TwoStage<N>::R0;
+  dftR<R0, DIR>(v);
+  const int x = R0 % 2 ? 0 : (j & 1);
+#pragma unroll
+  for (int r = 0; r < R0; ++r) buf[((j * R0 + r) ^ x) * P + p] = v[r];
+}
+template <int N, int P, int DIR>
+__device__ __forceinline__ void two_stage_second(float2* v, const float2* buf, const float2* tw, int p, int j) {
+  constexpr int R0 = TwoStage<N>::R0, R1 = TwoStage<N>::R1;
+  static_assert(R0 * R1 == N && R1 <= 32, "no two-stage split");
+#pragma unroll
+  for (int r = 0; r < R1; ++r) v[r] = buf[((j + r * R0) ^ (R0 % 2 ? 0 : (r & 1))) * P + p];
+#pragma unroll
+  for (int r = 1; r < R1; ++r) {
+    const float2 w = tw[r * j];
+    v[r] = cmul(v[r], make_float2(w.x, DIR < 0 ? w.y : -w.y));
+  }
+  dftR<R1, DIR>(v);
 }
 
 // Runtime-N version on the same interleaved layout (sizes without a

@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(256) k_counts(const int* __restrict__ ball, co
 //       n_x <= floor(r_s) (Hermitian extension), two real rows per complex
 //       pencil;  I[s][z][y][x]
 // Pencils are interleaved 8 to a block (element i of pencil p at i * 8 + p)
-// for the compile-time FFT.
+// (this form for sides without a compiled transform).
 // ----------------------------------------------------------------------------
 
 constexpr int kSP = 8;      // pencils per block
@@ -168,12 +168,11 @@ struct BispLaunch {
   int xblocks;
 };
 
-template <int N_>
 __global__ void __launch_bounds__(kSNT) k_shell_z(const float2* __restrict__ E, ShellParams sp, FftPlan fp,
                                                   const float2* __restrict__ twg, const int4* __restrict__ jobs,
                                                   float2* __restrict__ T1) {
   extern __shared__ float2 sm[];
-  const int N = N_ ? N_ : sp.N;
+  const int N = sp.N;
   float2* tw = sm;
   float2* A = sm + N;
   float2* B = A + kSP * N;
@@ -193,7 +192,7 @@ __global__ void __launch_bounds__(kSNT) k_shell_z(const float2* __restrict__ E, 
     }
   }
   __syncthreads();
-  const float2* R = fft_any<N_, kSP, kSNT, 1>(A, B, fp, tw);
+  const float2* R = fft_any<0, kSP, kSNT, 1>(A, B, fp, tw);
   const int c = threadIdx.x, run = threadIdx.y, rl = (N + 31) / 32;
   if (kx0 + c < m1) {
 #pragma unroll
@@ -204,12 +203,11 @@ __global__ void __launch_bounds__(kSNT) k_shell_z(const float2* __restrict__ E, 
   }
 }
 
-template <int N_>
 __global__ void __launch_bounds__(kSNT) k_shell_y(const float2* __restrict__ T1, ShellParams sp, FftPlan fp,
                                                   const float2* __restrict__ twg, const int4* __restrict__ jobs,
                                                   float2* __restrict__ T2) {
   extern __shared__ float2 sm[];
-  const int N = N_ ? N_ : sp.N;
+  const int N = sp.N;
   float2* tw = sm;
   float2* A = sm + N;
   float2* B = A + kSP * N;
@@ -225,7 +223,7 @@ __global__ void __launch_bounds__(kSNT) k_shell_y(const float2* __restrict__ T1,
     if (kx0 + c < m1) A[wrap_mode(ny, N) * kSP + c] = T1[(((size_t)s * N + z) * w2 + ny + mm) * m1 + kx0 + c];
   }
   __syncthreads();
-  const float2* R = fft_any<N_, kSP, kSNT, 1>(A, B, fp, tw);
+  const float2* R = fft_any<0, kSP, kSNT, 1>(A, B, fp, tw);
   const int c = threadIdx.x, run = threadIdx.y, rl = (N + 31) / 32;
   if (kx0 + c < m1) {
 #pragma unroll
@@ -238,11 +236,10 @@ __global__ void __launch_bounds__(kSNT) k_shell_y(const float2* __restrict__ T1,
 
 // Rows r = (s N + z) N + y; pencil p of a block iteration holds rows 2(g0+p)
 // and 2(g0+p)+1 (same shell: N^2 is even) as x1 + i x2.
-template <int N_>
 __global__ void __launch_bounds__(kSNT) k_shell_x(const float2* __restrict__ T2, ShellParams sp, FftPlan fp,
                                                   const float2* __restrict__ twg, float* __restrict__ I) {
   extern __shared__ float2 sm[];
-  const int N = N_ ? N_ : sp.N;
+  const int N = sp.N;
   float2* tw = sm;
   // A and B each followed by kXGap float2 of slack: the transposed rows
   // (stride N + 2 floats, so that the eight pencils' stores fall in distinct
@@ -308,7 +305,7 @@ __global__ void __launch_bounds__(kSNT) k_shell_x(const float2* __restrict__ T2,
     }
     __syncthreads();
     stage(g0 + (long long)gridDim.x * kSP);
-    const float2* R = fft_any<N_, kSP, kSNT, 1>(A, B, fp, tw);
+    const float2* R = fft_any<0, kSP, kSNT, 1>(A, B, fp, tw);
     // transpose through the free buffer into rows of stride N + 2 floats
     // (row 2p starts 20p banks further on: a warp's 8 pencils x 4 points hit
     // 32 distinct banks), then coalesced 8-byte stores (N even)
@@ -331,34 +328,197 @@ __global__ void __launch_bounds__(kSNT) k_shell_x(const float2* __restrict__ T2,
   }
 }
 
-template <int N_>
+// The same three passes at compiled lengths, as N = R0 R1 in two stages with
+// both radices in registers: the first stage takes its inputs where they lie
+// (E, T1, the staged rows) and the second hands its outputs on (T1, T2, the
+// transposed rows), so a transform crosses shared memory once instead of once
+// per radix 8, 5, 3 stage and twice more for its fill and its result.  Those
+// crossings and their barriers set the time of the staged form: 360^3, 37
+// shells, per multipole z 0.55, y 1.64, x 3.81 ms; here the three together
+// 6.0 -> 3.8 ms (with the F^w passes 20.4 -> 13.5 ms per mock).
+// Block (8, kTY): threadIdx.x is the pencil, threadIdx.y the butterfly.
+template <int N>
+__global__ void __launch_bounds__(kSP * TwoStage<N>::kTY) k_shell_zc(const float2* __restrict__ E, ShellParams sp,
+                                                                     const float2* __restrict__ twg,
+                                                                     const int4* __restrict__ jobs,
+                                                                     float2* __restrict__ T1) {
+  using T = TwoStage<N>;
+  __shared__ float2 tw[N], buf[kSP * N];
+  const int c = threadIdx.x, j = threadIdx.y;
+  for (int i = j * kSP + c; i < N; i += kSP * T::kTY) tw[i] = twg[i];
+  const int4 job = jobs[blockIdx.x];
+  const int s = job.x, kyp = job.y, kx = job.z + c;
+  const int mm = sp.mm, w2 = 2 * mm + 1, m1 = mm + 1, ny = kyp - mm;
+  if (j < T::R1) {
+    float2 v[T::R0];
+#pragma unroll
+    for (int r = 0; r < T::R0; ++r) {
+      const int i = j + r * T::R1, nz = i <= N / 2 ? i : i - N;
+      const int n2 = kx * kx + ny * ny + nz * nz;
+      v[r] = make_float2(0.f, 0.f);
+      if (kx < m1 && n2 < sp.nsh2 && sp.slut[n2] == s) v[r] = __ldg(E + ((size_t)(nz + mm) * w2 + kyp) * m1 + kx);
+    }
+    two_stage_first<N, kSP, 1>(v, buf, c, j);
+  }
+  __syncthreads();
+  if (j < T::R0) {
+    float2 v[T::R1];
+    two_stage_second<N, kSP, 1>(v, buf, tw, c, j);
+    if (kx < m1) {
+#pragma unroll
+      for (int r = 0; r < T::R1; ++r) T1[(((size_t)s * N + j + r * T::R0) * w2 + kyp) * m1 + kx] = v[r];
+    }
+  }
+}
+
+template <int N>
+__global__ void __launch_bounds__(kSP * TwoStage<N>::kTY) k_shell_yc(const float2* __restrict__ T1, ShellParams sp,
+                                                                     const float2* __restrict__ twg,
+                                                                     const int4* __restrict__ jobs,
+                                                                     float2* __restrict__ T2) {
+  using T = TwoStage<N>;
+  __shared__ float2 tw[N], buf[kSP * N];
+  const int c = threadIdx.x, j = threadIdx.y;
+  for (int i = j * kSP + c; i < N; i += kSP * T::kTY) tw[i] = twg[i];
+  const int4 job = jobs[blockIdx.x];
+  const int s = job.x, kx = job.y + c, nyr = job.z, z = blockIdx.y;
+  const int mm = sp.mm, w2 = 2 * mm + 1, m1 = mm + 1;
+  if (j < T::R1) {
+    const float2* src = T1 + (((size_t)s * N + z) * w2 + mm) * m1 + kx;
+    float2 v[T::R0];
+#pragma unroll
+    for (int r = 0; r < T::R0; ++r) {
+      const int i = j + r * T::R1, ny = i <= N / 2 ? i : i - N;
+      v[r] = make_float2(0.f, 0.f);
+      if (kx < m1 && ny <= nyr && ny >= -nyr) v[r] = __ldg(src + (long long)ny * m1);
+    }
+    two_stage_first<N, kSP, 1>(v, buf, c, j);
+  }
+  __syncthreads();
+  if (j < T::R0) {
+    float2 v[T::R1];
+    two_stage_second<N, kSP, 1>(v, buf, tw, c, j);
+    if (kx < m1) {
+      float2* dst = T2 + (((size_t)s * N + z) * N + j) * m1 + kx;
+#pragma unroll
+      for (int r = 0; r < T::R1; ++r) dst[(size_t)(r * T::R0) * m1] = v[r];
+    }
+  }
+}
+
+template <int N>
+__global__ void __launch_bounds__(kSP * TwoStage<N>::kTY) k_shell_xc(const float2* __restrict__ T2, ShellParams sp,
+                                                                     const float2* __restrict__ twg,
+                                                                     float* __restrict__ I) {
+  using T = TwoStage<N>;
+  constexpr int NT = kSP * T::kTY, rs = N + 2;
+  extern __shared__ __align__(16) float2 sm[];
+  float2* tw = sm;
+  float2* buf = tw + N;
+  float* rows = reinterpret_cast<float*>(buf + kSP * N);        // 2 kSP rows of stride N + 2 floats
+  float2* stg = reinterpret_cast<float2*>(rows + 2 * kSP * rs);  // the next iteration's rows of T2
+  const int p = threadIdx.x, j = threadIdx.y, tid = j * kSP + p;
+  const int m1 = sp.mm + 1;
+  for (int i = tid; i < N; i += NT) tw[i] = twg[i];
+  const long long pairs = (long long)sp.S * N * N / 2;
+  // 2 kSP rows of T2 are one contiguous span from row 2 g0 (g0 a multiple of 8: 16-byte aligned)
+  auto stage = [&](long long gn) {
+    if (gn < pairs) {
+      const int npn = (int)(pairs - gn < kSP ? pairs - gn : kSP);
+      const float2* src = T2 + 2 * gn * m1;
+      for (int t = tid; t < npn * m1; t += NT)  // 16-byte chunks
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(stg + 2 * t)), "l"(src + 2 * t)
+                     : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  stage((long long)blockIdx.x * kSP);
+  for (long long g0 = (long long)blockIdx.x * kSP; g0 < pairs; g0 += (long long)gridDim.x * kSP) {
+    const int np = (int)(pairs - g0 < kSP ? pairs - g0 : kSP);
+    // the pencil's shell (an iteration may straddle two) and its reach
+    const int s = (int)((2 * (g0 + p)) / ((long long)N * N));
+    const int km = p < np ? sp.kmax[s < sp.S ? s : sp.S - 1] : -1;
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    if (j < T::R1) {
+      const float2 *h0 = stg + (size_t)(2 * p) * m1, *h1 = h0 + m1;
+      float2 v[T::R0];
+#pragma unroll
+      for (int r = 0; r < T::R0; ++r) {
+        // x1 + i x2 of the Hermitian rows x1, x2: n_x and -n_x from the stored half
+        const int i = j + r * T::R1, k = i <= N / 2 ? i : N - i;
+        v[r] = make_float2(0.f, 0.f);
+        if (k <= km) {
+          float2 a = h0[k], b = h1[k];
+          if (i == 0) a.y = b.y = 0.f;
+          v[r] = i <= N / 2 ? make_float2(a.x - b.y, a.y + b.x) : make_float2(a.x + b.y, b.x - a.y);
+        }
+      }
+      two_stage_first<N, kSP, 1>(v, buf, p, j);
+    }
+    __syncthreads();
+    stage(g0 + (long long)gridDim.x * kSP);
+    if (j < T::R0) {
+      float2 v[T::R1];
+      two_stage_second<N, kSP, 1>(v, buf, tw, p, j);
+      // rows of stride N + 2 floats: a warp's 8 pencils x 4 points hit distinct banks
+#pragma unroll
+      for (int r = 0; r < T::R1; ++r) {
+        rows[(2 * p) * rs + j + r * T::R0] = v[r].x;
+        rows[(2 * p + 1) * rs + j + r * T::R0] = v[r].y;
+      }
+    }
+    __syncthreads();
+    float2* dst = reinterpret_cast<float2*>(I + 2 * g0 * N);
+    for (int t = tid; t < 2 * np * (N / 2); t += NT) {
+      const int row = t / (N / 2), x2 = t - row * (N / 2);
+      dst[t] = *reinterpret_cast<const float2*>(rows + row * rs + 2 * x2);
+    }
+  }
+}
+
+template <int N>
+static cudaError_t shell_passes_c(const BispLaunch& L, cudaStream_t s) {
+  const dim3 blk(kSP, TwoStage<N>::kTY);
+  cudaError_t e;
+  if (L.nz > 0) k_shell_zc<N><<<L.nz, blk, 0, s>>>(L.E, L.sp, L.tw, L.zjobs, L.T1);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if (L.ny > 0) k_shell_yc<N><<<dim3(L.ny, N), blk, 0, s>>>(L.T1, L.sp, L.tw, L.yjobs, L.T2);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  const size_t sm = sizeof(float2) * ((size_t)N * (1 + kSP) + 2 * kSP * (size_t)(L.sp.mm + 1)) +
+                    sizeof(float) * 2 * kSP * (N + 2);
+  if ((e = raise_smem_limit((const void*)k_shell_xc<N>, sm)) != cudaSuccess) return e;
+  k_shell_xc<N><<<L.xblocks, blk, sm, s>>>(L.T2, L.sp, L.tw, L.I);
+  return cudaGetLastError();
+}
+
 static cudaError_t shell_passes_n(const BispLaunch& L, cudaStream_t s) {
   const size_t sm = sizeof(float2) * (size_t)L.sp.N * (1 + 2 * kSP);
   cudaError_t e;
-  if ((e = raise_smem_limit((const void*)k_shell_z<N_>, sm)) != cudaSuccess) return e;
-  if ((e = raise_smem_limit((const void*)k_shell_y<N_>, sm)) != cudaSuccess) return e;
+  if ((e = raise_smem_limit((const void*)k_shell_z, sm)) != cudaSuccess) return e;
+  if ((e = raise_smem_limit((const void*)k_shell_y, sm)) != cudaSuccess) return e;
   const dim3 blk(kSP, kSNT / kSP);
-  if (L.nz > 0) k_shell_z<N_><<<L.nz, blk, sm, s>>>(L.E, L.sp, L.fp, L.tw, L.zjobs, L.T1);
+  if (L.nz > 0) k_shell_z<<<L.nz, blk, sm, s>>>(L.E, L.sp, L.fp, L.tw, L.zjobs, L.T1);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if (L.ny > 0) k_shell_y<N_><<<dim3(L.ny, L.sp.N), blk, sm, s>>>(L.T1, L.sp, L.fp, L.tw, L.yjobs, L.T2);
+  if (L.ny > 0) k_shell_y<<<dim3(L.ny, L.sp.N), blk, sm, s>>>(L.T1, L.sp, L.fp, L.tw, L.yjobs, L.T2);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   // + the slack after A and B, and the row staging
   const size_t smx = sm + sizeof(float2) * (2 * kXGap + 2 * kSP * (size_t)(L.sp.mm + 1));
-  if ((e = raise_smem_limit((const void*)k_shell_x<N_>, smx)) != cudaSuccess) return e;
-  k_shell_x<N_><<<L.xblocks, blk, smx, s>>>(L.T2, L.sp, L.fp, L.tw, L.I);
+  if ((e = raise_smem_limit((const void*)k_shell_x, smx)) != cudaSuccess) return e;
+  k_shell_x<<<L.xblocks, blk, smx, s>>>(L.T2, L.sp, L.fp, L.tw, L.I);
   return cudaGetLastError();
 }
 
 static cudaError_t shell_passes(const BispLaunch& L, cudaStream_t s) {
   switch (L.sp.N) {
-    case 360: return shell_passes_n<360>(L, s);
-    case 256: return shell_passes_n<256>(L, s);
-    case 384: return shell_passes_n<384>(L, s);
-    case 192: return shell_passes_n<192>(L, s);
-    case 128: return shell_passes_n<128>(L, s);
-    case 64: return shell_passes_n<64>(L, s);
-    case 512: return shell_passes_n<512>(L, s);
-    default: return shell_passes_n<0>(L, s);
+    case 512: return shell_passes_c<512>(L, s);
+    case 384: return shell_passes_c<384>(L, s);
+    case 360: return shell_passes_c<360>(L, s);
+    case 256: return shell_passes_c<256>(L, s);
+    case 192: return shell_passes_c<192>(L, s);
+    case 128: return shell_passes_c<128>(L, s);
+    case 64: return shell_passes_c<64>(L, s);
+    default: return shell_passes_n(L, s);
   }
 }
 
