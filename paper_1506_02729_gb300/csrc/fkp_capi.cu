@@ -99,6 +99,7 @@ bool fkp::radix_plan(int n, FftPlan& p) {
   while (m % 2 == 0) { if (!push(2)) return false; m /= 2; }
   while (m % 5 == 0) { if (!push(5)) return false; m /= 5; }
   while (m % 3 == 0) { if (!push(3)) return false; m /= 3; }
+  p.set_magic();
   return m == 1;
 }
 

@@ -90,6 +90,7 @@ bool na_radix(int n, FftPlan& p) {
       p.radix[p.nst++] = r;
       m /= r;
     }
+  p.set_magic();
   return m == 1;
 }
 
