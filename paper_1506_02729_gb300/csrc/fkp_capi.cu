@@ -646,7 +646,8 @@ int fkp::stage_catalog(Plan* P, const fkp_catalog_t* c, int slot, CatDev& out, c
     out.x = c->x; out.y = c->y; out.z = c->z; out.w = c->w; out.nbar = c->nbar;
     return FKP_OK;
   }
-  const size_t need = (size_t)c->n * sizeof(float) * 5;
+  const size_t n = (size_t)c->n, stride = (n + 3) & ~(size_t)3;  // arrays on 16-byte boundaries
+  const size_t need = stride * sizeof(float) * 5;
   if (P->staging_bytes[slot] < need) {
     if (P->staging[slot]) cudaFree(P->staging[slot]);
     P->staging[slot] = nullptr;
@@ -656,12 +657,11 @@ int fkp::stage_catalog(Plan* P, const fkp_catalog_t* c, int slot, CatDev& out, c
     P->staging_bytes[slot] = need;
   }
   float* base = static_cast<float*>(P->staging[slot]);
-  const size_t n = (size_t)c->n;
   const float* src[5] = {c->x, c->y, c->z, c->w, c->nbar};
   const float* dst[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
   for (int a = 0; a < 5; ++a) {
     if (!src[a]) continue;
-    float* d = base + a * n;
+    float* d = base + a * stride;
     CK(cudaMemcpyAsync(d, src[a], n * sizeof(float), cudaMemcpyHostToDevice, s));
     dst[a] = d;
   }

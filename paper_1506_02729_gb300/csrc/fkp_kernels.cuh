@@ -198,11 +198,6 @@ __device__ __forceinline__ double block_sum_f64(double v, double* sh) {
   return r;
 }
 
-// FKP weight w = 1/(1 + nbar P_FKP) unless the catalog carries weights.
-__device__ __forceinline__ float fkp_weight(const CatDev& c, long long i, float Pfkp) {
-  return c.w ? __ldg(c.w + i) : 1.0f / (1.0f + __ldg(c.nbar + i) * Pfkp);
-}
-
 // Double-single ("float-float") arithmetic for the scalar sums: a value is an
 // unevaluated pair hi + lo of FP32 numbers (about 48 significant bits), with
 // Knuth's TwoSum for exact additions and the FMA-based TwoProduct for exact
@@ -238,9 +233,8 @@ struct FFSum {
 // exactly as a pair, the FP32 reciprocal r0 of its leading part, and one
 // Newton-Raphson step w = r0 + r0 (1 - d r0) with the residual formed by FMA
 // (relative error about 2^-46).  Weights given with the catalog are exact.
-__device__ __forceinline__ FF fkp_weight_ff(const CatDev& c, long long i, float Ph, float Pl) {
-  if (c.w) return {__ldg(c.w + i), 0.f};
-  const float nb = __ldg(c.nbar + i);
+__device__ __forceinline__ FF fkp_weight_ff(bool given, float w, float nb, float Ph, float Pl) {
+  if (given) return {w, 0.f};
   const float p = nb * Ph;
   const float pe = fmaf(nb, Ph, -p) + nb * Pl;  // nbar P = p + pe
   const FF d = ff_two_sum(1.f, p);               // 1 + p = d.hi + d.lo

@@ -127,3 +127,30 @@ def test_second_grid_of_a_pair_is_the_shifted_grid(N, periodic, assign):
     one = fkp.Plan(dict(geom, origin=(half,) * 3), (0.5 * kf, kf, 8), bshells=(3, 3, 3, 4), want=1 | 16)
     for a, b in zip(pair.grid(g, r, which=1, with_w=True), one.grid(g, r, with_w=True)):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("n", [1, 3, 4, 5, 4095, 8193])
+@pytest.mark.parametrize("shift", [0, 1, 3])
+def test_catalog_lengths_and_alignments(n, shift):
+    """The count launch reads four objects at a time where all arrays start on
+    16-byte boundaries: lengths around multiples of four and of a block's share,
+    and views that start off those boundaries, give the grid and the scalars of
+    an aligned copy (the scalars to the FP64 rounding of another order of sums:
+    n terms, 1e-12)."""
+    import paper_1506_02729_gb300 as fkp
+    N = 64
+    box = [_cell((8, 8, 8), (56, 56, 56), N=64)]
+    geom = dict(L=L, N=N, assign=3, origin=(0.0, 0.0, 0.0), observer=(480.0, 480.0, 480.0), P_fkp=1e4)
+    kf = 2 * math.pi / L
+    plan = fkp.Plan(geom, (0.5 * kf, kf, 8))
+    base = _cloud(box, n + shift, 8)
+    base["w"] = np.linspace(0.5, 1.5, n + shift).astype(np.float32)
+    ran = to_device(_cloud(box, 5000, 9))
+    whole = to_device(base)
+    view = {k: v[shift:] for k, v in whole.items()}
+    copy = {k: v.clone() for k, v in view.items()}
+    assert np.array_equal(plan.grid(view, ran), plan.grid(copy, ran))
+    a, b = plan.power(view, ran), plan.power(copy, ran)
+    for k in ("alpha", "I22", "N0", "S3", "W_g"):
+        assert abs(a[k] / b[k] - 1) < 1e-12, k
+    assert abs(a["W_g"] / float(copy["w"].double().sum()) - 1) < 1e-12
