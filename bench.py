@@ -427,8 +427,8 @@ def run_gpu(args):
                     "d2h_bytes_per_step": d2h, "path": f"fkp_server_submit/wait, {args.e2e_slots} slots"
                     if args.e2e_slots > 1 else "fkp_power, one call at a time",
                     "one_call_at_a_time": job_rate(world, sync_s)},
-            # per step: 2 counts, scalars, tile totals, scan, 2 scatters, L^ab, tiles, x, y, z, bins
-            "gpu_launches": 13 * args.steps,
+            # per step: count, tile totals with the scalars, scan, scatter, tiles with L^ab, x, y, z, bins
+            "gpu_launches": 9 * args.steps,
             "roofline": roof,
             "fft_schedule": plan.schedule(),
             "clocks": ck}

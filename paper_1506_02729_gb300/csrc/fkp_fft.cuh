@@ -1,7 +1,7 @@
 // fkp_fft.cuh - batched shared-memory FFT building blocks for sm_103a.
 //
-// A batch of complex pencils of length n (n = 2^a 3^b 5^c <= 512) lives in
-// shared memory, pencil p at base + p*stride.  Each radix stage reads one
+// A batch of complex pencils of length n (n = 2^a 3^b 5^c <= 512) lives
+// interleaved in shared memory.  Each radix stage reads one
 // buffer and writes the other (self-sorting Stockham order, so the result is
 // in natural order without a bit-reversal pass).  For a stage of radix R
 // after stages whose radices multiply to ns, butterfly j (0 <= j < n/R)
