@@ -122,12 +122,14 @@ __global__ void __launch_bounds__(32 * ((nfields_of(LMAX) + 1) / 2), LMAX < 4 ? 
     __syncthreads();
     const float2* R;
     const int ncol = nxt * kT;
-    if constexpr (N_ > 0 && N_ < 512 && NP == 8) {
+    if constexpr (N_ >= 256 && N_ < 512 && NP == 8 && !PO) {
       // compiled lengths: two stages (TwoStage); the result goes back to A, only
       // the elements the unpack reads (k and N - k of the stored columns).  360^3
       // 0.95 -> 0.86 ms, 256^3 0.42 -> 0.37 ms.  At 512 the radix-32 stage keeps
       // half of the threads busy with 64 registers of data: 1.88 against 1.83 ms
-      // for twice the rounding error, so that length stays at 8 x 8 x 8.
+      // for twice the rounding error, so that length stays at 8 x 8 x 8, and so
+      // do the lengths below 256 and the per-object fields (8 x 16 at 128 read
+      // 1.7e-6 for 1.4e-6 against FP64 in P_4).
       using T = TwoStage<N_>;
       const int p = threadIdx.x, j = threadIdx.y;
       if (j < T::R1) {
