@@ -44,28 +44,39 @@ __host__ __device__ constexpr int reg_cells(bool second) { return reg_side<P>(se
 
 int assign_tiles_per_axis(int N) { return (N + kTile - 1) / kTile; }
 
-// Centre cell of an object: TSC taps c-1..c+1 around c = floor(u + 1/2);
-// CIC taps c, c+1 with c = floor(u); PCS taps c-1..c+2 with c = floor(u).
-// Returns false when a tap would leave [1, N-2] (non-periodic) or the
-// position is not finite.
+// Centre cell of an object along one axis, u = (x - origin)/H: TSC taps
+// c-1..c+1 around c = floor(u + 1/2); CIC taps c, c+1 with c = floor(u); PCS
+// taps c-1..c+2 with c = floor(u).  The count, the scatter and the accumulation
+// of an object must agree on its cell (its taps lie in its tile's region), also
+// where u + 1/2 is within a rounding of a whole number, so every kernel takes it
+// from here, with the roundings written out: left to the compiler, the product
+// may join the sum in one FMA in one kernel and not in another.
+template <int P>
+__device__ __forceinline__ int centre_index(float x, float origin, float invH) {
+  const float r = __fsub_rn(x, origin);
+  return (int)floorf(P == 3 ? __fmaf_rn(r, invH, 0.5f) : __fmul_rn(r, invH));
+}
+
+// The centre cell along the three axes.  Returns false when a tap would leave
+// [1, N-2] (non-periodic) or the position is not finite.
 template <int P>
 __device__ __forceinline__ bool centre_cell(const GeomDev& g, float px, float py, float pz, int& cx, int& cy,
                                             int& cz) {
   const float ux = (px - g.ox) * g.invH, uy = (py - g.oy) * g.invH, uz = (pz - g.oz) * g.invH;
-  const float sh = P == 3 ? 0.5f : 0.f;
   const int N = g.N;
+  auto cells = [&] {
+    cx = centre_index<P>(px, g.ox, g.invH);
+    cy = centre_index<P>(py, g.oy, g.invH);
+    cz = centre_index<P>(pz, g.oz, g.invH);
+  };
   if (!g.periodic) {
     if (!(ux >= 0.f && ux < (float)N && uy >= 0.f && uy < (float)N && uz >= 0.f && uz < (float)N)) return false;
-    cx = (int)floorf(ux + sh);
-    cy = (int)floorf(uy + sh);
-    cz = (int)floorf(uz + sh);
+    cells();
     const int lo = P == 2 ? 1 : 2, hi = P == 4 ? N - 4 : N - 3;
     return cx >= lo && cy >= lo && cz >= lo && cx <= hi && cy <= hi && cz <= hi;
   }
   if (!(fabsf(ux) < 1e8f && fabsf(uy) < 1e8f && fabsf(uz) < 1e8f)) return false;
-  cx = (int)floorf(ux + sh);
-  cy = (int)floorf(uy + sh);
-  cz = (int)floorf(uz + sh);
+  cells();
   return true;
 }
 
@@ -458,27 +469,24 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_scatter(CatDev cg, CatDev c
   }
 }
 
+// Taps of an object along one axis: the first of its P cells and their weights,
+// from its distance d = u - c to its centre cell c.
 template <int P>
-__device__ __forceinline__ void tap_weights(float u, int& i0, float* wt) {
+__device__ __forceinline__ void tap_weights(float x, float origin, float invH, int& i0, float* wt) {
+  const int c = centre_index<P>(x, origin, invH);
+  const float r = __fsub_rn(x, origin);
+  const float d = P == 3 ? __fmaf_rn(r, invH, -(float)c) : __fsub_rn(__fmul_rn(r, invH), (float)c);
+  i0 = P == 2 ? c : c - 1;
   if (P == 2) {
-    const float f = floorf(u);
-    const float d = u - f;
-    i0 = (int)f;
     wt[0] = 1.f - d;
     wt[1] = d;
   } else if (P == 3) {
-    const float f = floorf(u + 0.5f);
-    const float d = u - f;
-    i0 = (int)f - 1;
     const float a = 0.5f - d, b = 0.5f + d;
     wt[0] = 0.5f * a * a;
     wt[1] = 0.75f - d * d;
     wt[2] = 0.5f * b * b;
   } else {
     // PCS: the cubic B-spline at distances 1 + d, d, 1 - d, 2 - d
-    const float f = floorf(u);
-    const float d = u - f;
-    i0 = (int)f - 1;
     const float e = 1.f - d, d2 = d * d, d3 = d2 * d;
     wt[0] = e * e * e * (1.f / 6.f);
     wt[1] = (4.f - 6.f * d2 + 3.f * d3) * (1.f / 6.f);
@@ -643,19 +651,17 @@ __global__ void __launch_bounds__(kAccumThreads, W2 ? 2 : 4) k_tile_accum(GeomDe
     float4 o = xyzv[i];
     const float wv = W2 ? vw2[i] : 0.f;
     if (fld > 0) o.w *= object_moment(g, o, ea, eb, ec);  // |x^ products| <= 1: the bounds hold
-    const float ux = (o.x - g.ox) * g.invH, uy = (o.y - g.oy) * g.invH, uz = (o.z - g.oz) * g.invH;
     int ix, iy, iz;
     float wx[P], wy[P], wz[P];
-    tap_weights<P>(ux, ix, wx);
-    tap_weights<P>(uy, iy, wy);
-    tap_weights<P>(uz, iz, wz);
+    tap_weights<P>(o.x, g.ox, g.invH, ix, wx);
+    tap_weights<P>(o.y, g.oy, g.invH, iy, wy);
+    tap_weights<P>(o.z, g.oz, g.invH, iz, wz);
     // taps relative to the region (periodic positions may lie one box away)
     int cx = ix + (P >= 3 ? 1 : 0), cy = iy + (P >= 3 ? 1 : 0), cz = iz + (P >= 3 ? 1 : 0);
     if (SECOND) {  // the centre cell that chose the tile
-      const float sh = P == 3 ? 0.5f : 0.f;
-      cx = (int)floorf((o.x - o1.x) * g.invH + sh);
-      cy = (int)floorf((o.y - o1.y) * g.invH + sh);
-      cz = (int)floorf((o.z - o1.z) * g.invH + sh);
+      cx = centre_index<P>(o.x, o1.x, g.invH);
+      cy = centre_index<P>(o.y, o1.y, g.invH);
+      cz = centre_index<P>(o.z, o1.z, g.invH);
     }
     const int rx = ix - (cx - wrapN(cx, N)) - lx0;
     const int ry = iy - (cy - wrapN(cy, N)) - ly0;

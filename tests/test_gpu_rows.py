@@ -154,3 +154,35 @@ def test_catalog_lengths_and_alignments(n, shift):
     for k in ("alpha", "I22", "N0", "S3", "W_g"):
         assert abs(a[k] / b[k] - 1) < 1e-12, k
     assert abs(a["W_g"] / float(copy["w"].double().sum()) - 1) < 1e-12
+
+
+@pytest.mark.parametrize("assign", [2, 3, 4])
+@pytest.mark.parametrize("interlace", [False, True], ids=["plain", "pair"])
+def test_half_a_cell_outside_a_periodic_box(assign, interlace):
+    """Objects within a few roundings of u = -1/2 and u = N - 1/2, where a
+    rounding of u + 1/2 decides between the first cell and the last: every
+    launch takes the same one, so all of their weight lies in the cells around
+    the corner (three axes of up to four weights that each round to 2^-23 or
+    better: 2e-6 of it) and no other cell is touched."""
+    import paper_1506_02729_gb300 as fkp
+    N, H = 64, 15.625
+    edge = np.float32(-3 * H) + np.float32([-0.5 * H, (N - 0.5) * H])
+    near = [edge]
+    for to in (-1e9, 1e9):
+        e = edge
+        for _ in range(3):
+            e = np.nextafter(e, np.float32(to), dtype=np.float32)
+            near.append(e)
+    near = np.concatenate(near)
+    gen = np.random.default_rng(12)
+    gal = {k: gen.choice(near, 3000) for k in "xyz"} | {"nbar": np.full(3000, 1e-4, np.float32)}
+    ran = {k: np.full(100, (32 - 3) * H, np.float32) for k in "xyz"} | {"nbar": np.full(100, 1e-4, np.float32)}
+    geom = dict(L=N * H, N=N, assign=assign, origin=(-3 * H,) * 3, observer=(0.0, 0.0, 0.0), P_fkp=1e4, periodic=True)
+    kf = 2 * math.pi / (N * H)
+    plan = fkp.Plan(dict(geom, interlace=interlace), (0.5 * kf, kf, 8))
+    F = plan.grid(to_device(gal), to_device(ran), which=1 if interlace else 0)
+    corner = np.ix_(*[[-3, -2, -1, 0, 1, 2]] * 3)
+    middle = np.ix_(*[range(28, 37)] * 3)
+    W = 3000 * 0.5  # w = 1/(1 + nbar P) = 1/2
+    assert abs(F[corner].sum() * 2.0 ** -40 / W - 1) < 2e-6
+    assert np.count_nonzero(F) == np.count_nonzero(F[corner]) + np.count_nonzero(F[middle])
