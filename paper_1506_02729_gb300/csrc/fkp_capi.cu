@@ -745,7 +745,7 @@ static int grid_pass(Plan* P, const CatDev& gal, const CatDev& ran, cudaStream_t
                         geo.alpha_mode, P->d_ds, s));
   const int chunk = accum_chunk(ntot * ngrid, nb);
   CK(launch_scan_tiles(P->d_tcnt, P->ntiles, P->d_toff, P->d_titem, chunk, s, geo,
-                       cached ? P->rc_tcnt : nullptr, P->d_occ, P->d_occ2));
+                       cached ? P->rc_tcnt : nullptr, P->d_occ, P->d_occ2, P->d_err));
   CK(record_stage(P->ev[1], s));
   CK(cudaStreamWaitEvent(s, P->ev_join, 0));
   float* vw2 = gridw ? P->d_vw2 : nullptr;
@@ -804,7 +804,7 @@ static int cache_randoms(Plan* P, const CatDev& ran, cudaStream_t s) {
     }
     P->rc_part = (double*)P->alloc(sizeof(double) * SC_NSUM * nb);
     P->rc_lab = (double*)P->alloc(sizeof(double) * LAB_NSUM);
-    P->rc_tcnt = (int*)P->alloc(sizeof(int) * P->ntiles);
+    P->rc_tcnt = (int*)P->alloc(sizeof(int) * (P->ntiles + 1));
     if (!P->rc_grid || (P->d_gridw && !P->rc_gridw) || !P->rc_part || !P->rc_lab || !P->rc_tcnt ||
         (P->interlace && (!P->rc_grid2 || (P->d_gridw && !P->rc_gridw2))))
       return set_error(FKP_ENOMEM, "cannot allocate the cached random grids");
@@ -826,8 +826,10 @@ static int cache_randoms(Plan* P, const CatDev& ran, cudaStream_t s) {
   CK(launch_bin_count(ran, ran, 0, nbr, P->g, P->interlace ? &P->g2 : nullptr, P->rc_part, P->d_bhist, P->d_err, s));
   CK(launch_tile_prefix(P->d_bhist, nbr, P->ntiles, P->d_tcnt, nullptr, 0, 0, 0, 0, 0, nullptr, s));
   const int chunk = accum_chunk(ran.n, nb);
-  CK(launch_scan_tiles(P->d_tcnt, P->ntiles, P->d_toff, P->d_titem, chunk, s, P->g, nullptr, nullptr, nullptr));
+  CK(launch_scan_tiles(P->d_tcnt, P->ntiles, P->d_toff, P->d_titem, chunk, s, P->g, nullptr, nullptr, nullptr,
+                       P->d_err));
   CK(cudaMemcpyAsync(P->rc_tcnt, P->d_tcnt, sizeof(int) * P->ntiles, cudaMemcpyDeviceToDevice, s));
+  CK(cudaMemcpyAsync(P->rc_tcnt + P->ntiles, P->d_err + kErrApart, sizeof(int), cudaMemcpyDeviceToDevice, s));
   CK(launch_bin_scatter(ran, ran, 0, nbr, P->g, P->geom.observer, P->d_ds, P->d_toff, P->d_bhist, P->d_xyzv, vw2,
                         P->d_labpart, s, 1));
   for (int which = 0; which < (P->interlace ? 2 : 1); ++which) {

@@ -72,7 +72,8 @@ struct Plan {
   double* d_zpart = nullptr;
   int* d_zpartc = nullptr;
   // result block, copied back whole: [BQ_N][nbins] bin sums, [nbins] counts,
-  // the scalars and L^ab sums (d_ds), four flag words (d_err)
+  // the scalars and L^ab sums (d_ds), four flag words (d_err: [0] an object out
+  // of the box, [1] a bounded wait gave up, [kErrApart])
   double* d_bins = nullptr;
   long long* d_binc = nullptr;
   void set_result(double* base) {
@@ -101,7 +102,7 @@ struct Plan {
   bool rc_valid = false;
   unsigned long long *rc_grid = nullptr, *rc_gridw = nullptr;
   double *rc_part = nullptr, *rc_lab = nullptr;
-  int* rc_tcnt = nullptr;  // its tile counts
+  int* rc_tcnt = nullptr;  // its tile counts, and its flag kErrApart behind them
   int rc_nblk = 0;
   long long rc_n = 0;
 
@@ -185,10 +186,15 @@ cudaError_t launch_bin_count(const CatDev& gal, const CatDev& ran, int nbg, int 
 cudaError_t launch_tile_prefix(int* bh, int nrows, int ntiles, int* cnt, const double* part, int nbg, int nbr,
                                long long ng, long long nr, int alpha_mode, double* ds, cudaStream_t s);
 int accum_chunk(long long nobj, int nsm);
+// Flag word (Plan::d_err) that the count launch sets when an object's centre
+// cells in the two grids of an interlaced pair are neither the same nor
+// neighbours (k_tile_accum).
+constexpr int kErrApart = 2;
 // occ: NULL, or the plan's list of occupied rows; more: NULL, or the tile
-// counts of a cached random catalog.
+// counts of a cached random catalog with its flag kErrApart behind them; err:
+// the flags of this call.
 cudaError_t launch_scan_tiles(const int* cnt, int ntiles, int* off, int* items, int chunk, cudaStream_t s,
-                              const GeomDev& g, const int* more, int* occ, int* occ2);
+                              const GeomDev& g, const int* more, int* occ, int* occ2, const int* err);
 cudaError_t launch_bin_scatter(const CatDev& gal, const CatDev& ran, int nbg, int nbr, const GeomDev& g,
                                const double obs[3], const double* ds, const int* off, const int* bpref, float4* xyzv,
                                float* vw2, double* labpart, cudaStream_t s, int raw = 0);

@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_count(CatDev cg, CatDev cr,
   for (int t = threadIdx.x; t < ntiles; t += blockDim.x) hist[t] = 0;
   __syncthreads();
   FFSum s_w, s_w2, s_w3, s_nw2, s_n2w3;
-  bool bad = false;
+  bool bad = false, apart = false;
   const int nblk = is_ran ? (int)gridDim.x - nbg : nbg, blk = is_ran ? (int)blockIdx.x - nbg : (int)blockIdx.x;
   const long long chunk = ((c.n + nblk - 1) / nblk + 3) & ~3ll;
   const long long i0 = blk * chunk < c.n ? blk * chunk : c.n;
@@ -163,13 +163,19 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_count(CatDev cg, CatDev cr,
       s_n2w3.add(ff_mul(ff_mul(w3, nb), nb));
     }
     int cx, cy, cz;
-    if (centre_cell<P>(g, px, py, pz, cx, cy, cz))
+    const bool in = centre_cell<P>(g, px, py, pz, cx, cy, cz);
+    if (in)
       atomicAdd(hist + tile_of(cx, cy, cz, g.N, ntx), 1);
     else
       bad = true;
-    if (two && !centre_cell<P>(g2, px, py, pz, cx, cy, cz)) bad = true;
+    if (two) {
+      int dx, dy, dz;
+      if (!in || !centre_cell<P>(g2, px, py, pz, dx, dy, dz)) bad = true;
+      else if ((unsigned)(cx - dx) > 1u || (unsigned)(cy - dy) > 1u || (unsigned)(cz - dz) > 1u) apart = true;
+    }
   });
   if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(err, 1);
+  if (two && __syncthreads_or(apart) && threadIdx.x == 0) atomicOr(err + kErrApart, 1);
   int* row = bh + (size_t)blockIdx.x * ntiles;
   for (int t = threadIdx.x; t < ntiles; t += blockDim.x) row[t] = hist[t];
   double* out = part + (size_t)blockIdx.x * SC_NSUM;
@@ -259,11 +265,13 @@ __global__ void __launch_bounds__(256) k_tile_prefix(int* __restrict__ bh, int n
 // occ (if not null) receives the rows that the occupied tiles reach (OccView),
 // a tile counting as occupied when cnt or more (the cached random catalog's
 // counts, or null) says so: a tile's objects reach its cells, one cell below
-// and reach - kTile + 1 above, wrapped around a periodic box.
+// and reach - kTile + 1 above, wrapped around a periodic box.  apart (with
+// occ2): the flag of objects whose second-grid cells lie anywhere; the cached
+// catalog's follows its counts.  The second grid then counts every row.
 __global__ void __launch_bounds__(1024) k_scan_tiles(const int* __restrict__ cnt, int ntiles, int* __restrict__ off,
                                                      int* __restrict__ items, int chunk, const int* __restrict__ more, int ntx,
                                                      int N, int reach, int periodic, int* __restrict__ occ,
-                                                     int* __restrict__ occ2) {
+                                                     int* __restrict__ occ2, const int* __restrict__ apart) {
   __shared__ int wsum[32], wsumi[32];
   __shared__ int ty0[32], ty1[32];  // per plane of tiles: first and last occupied tile row
   __shared__ int zfirst, zlast;
@@ -348,6 +356,7 @@ __global__ void __launch_bounds__(1024) k_scan_tiles(const int* __restrict__ cnt
   // first grid's tiles, one cell further down (occ2).
   for (int low = 1; low <= (occ2 ? 2 : 1); ++low) {
     int* out = low == 1 ? occ : occ2;
+    const bool all = low == 2 && (*apart || (more && more[ntiles]));
     const int z = threadIdx.x;
     __syncthreads();
     if (z == 0) {
@@ -369,6 +378,10 @@ __global__ void __launch_bounds__(1024) k_scan_tiles(const int* __restrict__ cnt
           y0 = min(y0, max(ya, 0));
           y1 = max(y1, min(yb + 1, N));
         }
+      }
+      if (all) {
+        y0 = 0;
+        y1 = N;
       }
       if (y1 > y0) {
         atomicMin(&zfirst, z);
@@ -564,7 +577,10 @@ struct MomentExp {
 // further, so an object's centre cell there is its centre cell in the first
 // grid or the one below: the region begins one cell lower, and the pair needs
 // one count, scan and scatter instead of two (360^3 PCS, 3.5e7 randoms: 1.1 ms
-// of 11.7).
+// of 11.7).  A periodic box takes positions up to 1e8 cells away, where the two
+// FP32 coordinates round apart (from 2^22 cells on their spacing is half a cell
+// and more) and the second grid's cell may lie further down: such an object's
+// taps go to the grid directly.
 template <int P, bool W2, bool SECOND>
 __global__ void __launch_bounds__(kAccumThreads, W2 ? 2 : 4) k_tile_accum(GeomDev g, float3 o1, int ntx, int ntiles,
                                                                         const int* __restrict__ off,
@@ -597,7 +613,7 @@ __global__ void __launch_bounds__(kAccumThreads, W2 ? 2 : 4) k_tile_accum(GeomDe
   extern __shared__ unsigned long long reg[];
   __shared__ int s_tile;
   __shared__ float s_abs;
-  __shared__ int s_max;
+  __shared__ int s_max, s_apart;
   unsigned long long* regw = reg + kReg3;
   int* L = reinterpret_cast<int*>(reg);
   int* H = L + kReg3;
@@ -616,6 +632,7 @@ __global__ void __launch_bounds__(kAccumThreads, W2 ? 2 : 4) k_tile_accum(GeomDe
     s_tile = lo;
     s_abs = 0.f;
     s_max = 0;
+    s_apart = 0;
   }
   const int N = g.N;
   for (int i = threadIdx.x; i < kReg3; i += blockDim.x) {
@@ -645,6 +662,11 @@ __global__ void __launch_bounds__(kAccumThreads, W2 ? 2 : 4) k_tile_accum(GeomDe
     atomicMax(&s_max, __float_as_int(ma));  // non-negative: ordered as integers (NaN above +inf)
   }
   __syncthreads();
+  // whether the P taps from (x, y, z) of the region lie in it
+  auto inside = [](int x, int y, int z) {
+    constexpr unsigned kLast = kReg - P;
+    return (unsigned)x <= kLast && (unsigned)y <= kLast && (unsigned)z <= kLast;
+  };
   // the bounds, with room for the rounding of the FP32 sums above
   const bool split = s_abs < 1000.f && __int_as_float(s_max) < 2.f;
   for (int i = a + threadIdx.x; i < b; i += kAccumThreads) {
@@ -666,6 +688,10 @@ __global__ void __launch_bounds__(kAccumThreads, W2 ? 2 : 4) k_tile_accum(GeomDe
     const int rx = ix - (cx - wrapN(cx, N)) - lx0;
     const int ry = iy - (cy - wrapN(cy, N)) - ly0;
     const int rz = iz - (cz - wrapN(cz, N)) - lz0;
+    if (SECOND && !inside(rx, ry, rz)) {
+      s_apart = 1;  // left for the loop below
+      continue;
+    }
     if (split) {
 #pragma unroll
       for (int p = 0; p < P; ++p) {
@@ -706,6 +732,36 @@ __global__ void __launch_bounds__(kAccumThreads, W2 ? 2 : 4) k_tile_accum(GeomDe
     }
   }
   __syncthreads();
+  if (SECOND && s_apart) {
+#pragma unroll 1
+    for (int i = a + threadIdx.x; i < b; i += kAccumThreads) {
+      const float4 o = xyzv[i];
+      const float wv = W2 ? vw2[i] : 0.f;
+      int ix, iy, iz;
+      float wx[P], wy[P], wz[P];
+      tap_weights<P>(o.x, g.ox, g.invH, ix, wx);
+      tap_weights<P>(o.y, g.oy, g.invH, iy, wy);
+      tap_weights<P>(o.z, g.oz, g.invH, iz, wz);
+      const int cx = centre_index<P>(o.x, o1.x, g.invH), cy = centre_index<P>(o.y, o1.y, g.invH),
+                cz = centre_index<P>(o.z, o1.z, g.invH);
+      if (inside(ix - (cx - wrapN(cx, N)) - lx0, iy - (cy - wrapN(cy, N)) - ly0, iz - (cz - wrapN(cz, N)) - lz0))
+        continue;
+#pragma unroll
+      for (int p = 0; p < P; ++p)
+#pragma unroll
+        for (int q = 0; q < P; ++q) {
+          const float wzy = wz[p] * wy[q];
+          const size_t row = ((size_t)wrapN(iz + p, N) * N + wrapN(iy + q, N)) * N;
+#pragma unroll
+          for (int r = 0; r < P; ++r) {
+            const float tw = wzy * wx[r];
+            const size_t gi = row + wrapN(ix + r, N);
+            atomicAdd(grid + gi, (unsigned long long)__float2ll_rn(o.w * tw * kFixScaleF));
+            if (W2) atomicAdd(gridw + gi, (unsigned long long)__float2ll_rn(wv * tw * kFixScaleF));
+          }
+        }
+    }
+  }
   for (int i = threadIdx.x; i < kReg3; i += blockDim.x) {
     unsigned long long v, vw = 0ull;
     if (split) {
@@ -795,9 +851,9 @@ int accum_chunk(long long nobj, int nsm) {
 }
 
 cudaError_t launch_scan_tiles(const int* cnt, int ntiles, int* off, int* items, int chunk, cudaStream_t s,
-                              const GeomDev& g, const int* more, int* occ, int* occ2) {
+                              const GeomDev& g, const int* more, int* occ, int* occ2, const int* err) {
   k_scan_tiles<<<1, 1024, 0, s>>>(cnt, ntiles, off, items, chunk, more, assign_tiles_per_axis(g.N), g.N,
-                                  g.assign == 4 ? kTile + 1 : kTile, g.periodic, occ, occ2);
+                                  g.assign == 4 ? kTile + 1 : kTile, g.periodic, occ, occ2, err + kErrApart);
   return cudaGetLastError();
 }
 

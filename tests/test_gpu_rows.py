@@ -186,3 +186,78 @@ def test_half_a_cell_outside_a_periodic_box(assign, interlace):
     W = 3000 * 0.5  # w = 1/(1 + nbar P) = 1/2
     assert abs(F[corner].sum() * 2.0 ** -40 / W - 1) < 2e-6
     assert np.count_nonzero(F) == np.count_nonzero(F[corner]) + np.count_nonzero(F[middle])
+
+
+# origins whose sums with far positions are ties of the FP32 spacing there (32,
+# 64, 128, that is 2, 4, 8 cells), so that the two grids of a pair round apart
+FAR = dict(L=1024.0, N=64, origin=(-48.0, -32.0, -64.0), observer=(480.0, 480.0, 480.0), P_fkp=1e4, periodic=True)
+FAR_EXP = (28, 29, 30)
+
+
+def _far(n, seed, axes, cells=(0, 64)):
+    """n objects, on the given axes 2^28 to 2^31 away, elsewhere in the box, all with
+    their first-grid cell in [cells) modulo the box; exact weights; and the
+    largest distance between an object's two cells."""
+    g = np.random.default_rng(seed)
+    cat, apart = {}, 0
+    for a, k in enumerate("xyz"):
+        lo = np.float32(FAR["origin"][a])
+        if a in axes:
+            ulp = 2.0 ** (FAR_EXP[a] - 23)
+            x = (2.0 ** FAR_EXP[a] + ulp * g.integers(1, 2 ** 21, 400 * n)).astype(np.float32)
+            x *= g.choice(np.float32([-1, 1]), x.size)
+        else:
+            x = (lo + 1024 * g.random(400 * n)).astype(np.float32)
+        c1 = np.floor((x - lo) * np.float32(1 / 16)).astype(np.int64)
+        c2 = np.floor((x - (lo + np.float32(8))) * np.float32(1 / 16)).astype(np.int64)
+        keep = np.nonzero((c1 % 64 >= cells[0]) & (c1 % 64 < cells[1]))[0][:n]
+        assert len(keep) == n
+        cat[k] = x[keep]
+        apart = max(apart, int((c1 - c2)[keep].max()))
+    cat["nbar"] = np.full(n, 1e-4, np.float32)
+    cat["w"] = (g.integers(1, 1024, n) / 1024.0).astype(np.float32)
+    return cat, apart
+
+
+@pytest.mark.parametrize("assign", [2, 3, 4])
+@pytest.mark.parametrize("axes", [(0,), (1,), (2,), (0, 1, 2)], ids=["x", "y", "z", "xyz"])
+def test_pair_takes_positions_many_boxes_away(assign, axes):
+    """A periodic box takes positions up to 1e8 cells away.  There the two FP32
+    coordinates of an interlaced pair round apart, and an object's cell in the
+    second grid may lie several below its cell in the first: the second grid is
+    still, bit for bit, the grid of a plan whose origin is half a cell further."""
+    import paper_1506_02729_gb300 as fkp
+    (gal, da), (ran, dr) = _far(3000, 1, axes), _far(9000, 2, axes)
+    assert max(da, dr) > 1
+    geom = dict(FAR, assign=assign)
+    kf = 2 * math.pi / 1024.0
+    pair = fkp.Plan(dict(geom, interlace=True), (0.5 * kf, kf, 8), bshells=(3, 3, 3, 4), want=1 | 16)
+    one = fkp.Plan(dict(geom, origin=tuple(o + 8.0 for o in FAR["origin"])), (0.5 * kf, kf, 8), bshells=(3, 3, 3, 4),
+                   want=1 | 16)
+    g, r = to_device(gal), to_device(ran)
+    for a, b in zip(pair.grid(g, r, which=1, with_w=True), one.grid(g, r, with_w=True)):
+        assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("cached", [False, True], ids=["both", "cached_randoms"])
+@pytest.mark.parametrize("far", ["galaxies", "randoms", "none"])
+def test_rows_of_a_pair_with_positions_many_boxes_away(far, cached):
+    """Such objects may reach rows of the second grid that no tile of the first
+    grid announces: the spectra are those of the same survey with a weightless
+    galaxy in every tile, which makes every row count."""
+    import paper_1506_02729_gb300 as fkp
+    gal = _far(500, 3, (0, 1, 2) if far == "galaxies" else (), cells=(16, 32))[0]
+    ran = _far(2000, 4, (0, 1, 2) if far == "randoms" else (), cells=(16, 32))[0]
+    t = np.stack(np.meshgrid(*[np.arange(8.5, 64, 16)] * 3), -1).reshape(-1, 3)
+    fill = {k: np.concatenate([gal[k], (FAR["origin"][a] + 16 * t[:, a]).astype(np.float32)]) for a, k in enumerate("xyz")}
+    fill["nbar"] = np.full(len(fill["x"]), 1e-4, np.float32)
+    fill["w"] = np.concatenate([gal["w"], np.zeros(len(t), np.float32)])
+    kf = 2 * math.pi / 1024.0
+    plan = fkp.Plan(dict(FAR, assign=3, interlace=True), (0.5 * kf, kf, 24))
+    g, f, r = to_device(gal), to_device(fill), to_device(ran)
+    if cached:
+        plan.cache_randoms(r)
+        r = None
+    got, ref = plan.power(g, r), plan.power(f, r)
+    for k in ("P0", "P2", "P4", "P4b", "nmodes"):
+        assert np.array_equal(got[k], ref[k], equal_nan=True), k
