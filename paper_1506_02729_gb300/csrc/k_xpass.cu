@@ -120,39 +120,14 @@ __global__ void __launch_bounds__(32 * ((nfields_of(LMAX) + 1) / 2), LMAX < 4 ? 
       build_pairs<NP, NF, 0, SWZ>(rowF[x], hx, hy, hz, A, x);
     }
     __syncthreads();
-    const float2* R;
+    // Radix 8, 4, 2, 5, 3 stages at every length.  Two register stages (TwoStage,
+    // as the shell transforms run) take 0.37 for 0.42 ms at 256^3 and 0.86 for 0.95
+    // ms at 360^3, but against FP64 they are not as good everywhere: their errors
+    // over these are, in the mean of 12 survey mocks each, 1.07 +- 0.03 in P_0 at
+    // 256^3, 1.21 +- 0.09 in P_0 at 360^3 and 1.6 +- 0.2 in P_4 at 384^3 (FP32
+    // constants w_16, w_24 that meet every row alike).
     const int ncol = nxt * kT;
-    if constexpr (N_ >= 256 && N_ < 512 && NP == 8 && !PO) {
-      // compiled lengths: two stages (TwoStage); the result goes back to A, only
-      // the elements the unpack reads (k and N - k of the stored columns).  360^3
-      // 0.95 -> 0.86 ms, 256^3 0.42 -> 0.37 ms.  At 512 the radix-32 stage keeps
-      // half of the threads busy with 64 registers of data: 1.88 against 1.83 ms
-      // for twice the rounding error, so that length stays at 8 x 8 x 8, and so
-      // do the lengths below 256 and the per-object fields (8 x 16 at 128 read
-      // 1.7e-6 for 1.4e-6 against FP64 in P_4).
-      using T = TwoStage<N_>;
-      const int p = threadIdx.x, j = threadIdx.y;
-      if (j < T::R1) {
-        float2 v[T::R0];
-#pragma unroll
-        for (int r = 0; r < T::R0; ++r) v[r] = A[ilv<NP, SWZ>(j + r * T::R1, p)];
-        two_stage_first<N_, NP, -1>(v, B, p, j);
-      }
-      __syncthreads();
-      if (j < T::R0) {
-        float2 v[T::R1];
-        two_stage_second<N_, NP, -1>(v, B, tw, p, j);
-#pragma unroll
-        for (int r = 0; r < T::R1; ++r) {
-          const int k = j + r * T::R0;
-          if (k < ncol || k > N - ncol) A[ilv<NP, SWZ>(k, p)] = v[r];
-        }
-      }
-      __syncthreads();
-      R = A;
-    } else {
-      R = fft_any<N_, NP, NTX, -1, SWZ>(A, B, fp, tw);
-    }
+    const float2* R = fft_any<N_, NP, NTX, -1, SWZ>(A, B, fp, tw);
     // unpack: warp p takes pencil p (the block has NP warps), consecutive lanes
     // consecutive k_x, so the stores into the tile-major layout are 64-byte
     // contiguous runs; only the k_x tiles that hold a wanted mode are stored
