@@ -101,27 +101,38 @@ __device__ __forceinline__ int tile_of(int cx, int cy, int cz, int N, int ntx) {
 // 2e4 galaxies and 2e5 randoms took 19 + 26 us one after the other).  Each
 // block owns a contiguous chunk of objects (the same chunks as the scatter
 // launch on the same catalogs): its counts go to a shared-memory histogram
-// over all tiles, written out whole as the block's row of bh.
+// over all tiles, written out whole as the block's row of bh.  TWO: the objects'
+// cells in the second grid g2 of an interlaced pair are checked too.
 constexpr int kBinThreads = 1024;
 
 // f(x, y, z, nbar, w or 0) for the objects of [i0, i1).  WIDE: in runs of four
-// per thread when every array of the catalog starts on a 16-byte boundary (one
-// 16-byte load per array instead of four of 4 bytes; chunks start at multiples
-// of four), one by one otherwise.  3.57e7 objects, 512^3: the count launch and
-// the scans behind it 0.55 -> 0.40 ms; the scatter gains nothing (four objects
-// of a thread go to four places one after the other: 1.59 -> 1.64 ms with the
-// accumulation) and takes them one by one.
+// per thread, one 16-byte load per array where every array of the catalog starts
+// on a 16-byte boundary (chunks start at multiples of four) and four loads of 4
+// bytes otherwise: the objects come to each thread in the same order either way,
+// so its sums do not depend on where the caller's arrays lie.  Otherwise one by
+// one.  3.57e7 objects, 512^3: the count launch and the scans behind it 0.55 ->
+// 0.41 ms; the scatter gains nothing (four objects of a thread go to four places
+// one after the other: 1.59 -> 1.64 ms with the accumulation) and takes them one
+// by one.
 template <bool WIDE, class F>
 __device__ __forceinline__ void each_object(const CatDev& c, long long i0, long long i1, F&& f) {
-  const unsigned long long al = (unsigned long long)c.x | (unsigned long long)c.y | (unsigned long long)c.z |
-                                (unsigned long long)c.nbar | (unsigned long long)c.w;  // c.w may be null
-  if (WIDE && (al & 15) == 0) {
+  if (WIDE) {
     const long long n4 = i0 + ((i1 - i0) & ~3ll);
-    auto load4 = [](const float* p, long long i) { return __ldg(reinterpret_cast<const float4*>(p + i)); };
+    const unsigned long long al = (unsigned long long)c.x | (unsigned long long)c.y | (unsigned long long)c.z |
+                                  (unsigned long long)c.nbar | (unsigned long long)c.w;  // c.w may be null
+    const bool wide = (al & 15) == 0;
+    auto load4 = [](const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); };
+    auto load1 = [](const float* p) { return make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3)); };
 #pragma unroll 1
     for (long long i = i0 + 4 * (long long)threadIdx.x; i < n4; i += 4 * (long long)blockDim.x) {
-      const float4 x = load4(c.x, i), y = load4(c.y, i), z = load4(c.z, i), nb = load4(c.nbar, i);
-      const float4 w = c.w ? load4(c.w, i) : make_float4(0.f, 0.f, 0.f, 0.f);
+      float4 x, y, z, nb, w = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (wide) {
+        x = load4(c.x + i); y = load4(c.y + i); z = load4(c.z + i); nb = load4(c.nbar + i);
+        if (c.w) w = load4(c.w + i);
+      } else {
+        x = load1(c.x + i); y = load1(c.y + i); z = load1(c.z + i); nb = load1(c.nbar + i);
+        if (c.w) w = load1(c.w + i);
+      }
       f(x.x, y.x, z.x, nb.x, w.x);
       f(x.y, y.y, z.y, nb.y, w.y);
       f(x.z, y.z, z.z, nb.z, w.z);
@@ -134,9 +145,9 @@ __device__ __forceinline__ void each_object(const CatDev& c, long long i0, long 
     f(__ldg(c.x + i), __ldg(c.y + i), __ldg(c.z + i), __ldg(c.nbar + i), c.w ? __ldg(c.w + i) : 0.f);
 }
 
-template <int P>
-__global__ void __launch_bounds__(kBinThreads) k_bin_count(CatDev cg, CatDev cr, int nbg, GeomDev g, int two,
-                                                           GeomDev g2, int ntx, int ntiles, double* __restrict__ part,
+template <int P, bool TWO>
+__global__ void __launch_bounds__(kBinThreads) k_bin_count(CatDev cg, CatDev cr, int nbg, GeomDev g, GeomDev g2,
+                                                           int ntx, int ntiles, double* __restrict__ part,
                                                            int* __restrict__ bh, int* __restrict__ err) {
   const int is_ran = (int)blockIdx.x >= nbg;
   const CatDev& c = is_ran ? cr : cg;
@@ -168,14 +179,14 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_count(CatDev cg, CatDev cr,
       atomicAdd(hist + tile_of(cx, cy, cz, g.N, ntx), 1);
     else
       bad = true;
-    if (two) {
+    if (TWO) {
       int dx, dy, dz;
       if (!in || !centre_cell<P>(g2, px, py, pz, dx, dy, dz)) bad = true;
       else if ((unsigned)(cx - dx) > 1u || (unsigned)(cy - dy) > 1u || (unsigned)(cz - dz) > 1u) apart = true;
     }
   });
   if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(err, 1);
-  if (two && __syncthreads_or(apart) && threadIdx.x == 0) atomicOr(err + kErrApart, 1);
+  if (TWO && __syncthreads_or(apart) && threadIdx.x == 0) atomicOr(err + kErrApart, 1);
   int* row = bh + (size_t)blockIdx.x * ntiles;
   for (int t = threadIdx.x; t < ntiles; t += blockDim.x) row[t] = hist[t];
   double* out = part + (size_t)blockIdx.x * SC_NSUM;
@@ -819,16 +830,20 @@ cudaError_t launch_bin_count(const CatDev& gal, const CatDev& ran, int nbg, int 
   const int ntiles = ntx * ntx * ntx;
   const size_t sm = sizeof(int) * ntiles;
   const int nblk = nbg + nbr;
-  if (g.assign == 2) {
-    raise_smem_limit((const void*)k_bin_count<2>, sm);
-    k_bin_count<2><<<nblk, kBinThreads, sm, s>>>(gal, ran, nbg, g, g2 ? 1 : 0, g2 ? *g2 : g, ntx, ntiles, part, bh, err);
-  } else if (g.assign == 3) {
-    raise_smem_limit((const void*)k_bin_count<3>, sm);
-    k_bin_count<3><<<nblk, kBinThreads, sm, s>>>(gal, ran, nbg, g, g2 ? 1 : 0, g2 ? *g2 : g, ntx, ntiles, part, bh, err);
-  } else {
-    raise_smem_limit((const void*)k_bin_count<4>, sm);
-    k_bin_count<4><<<nblk, kBinThreads, sm, s>>>(gal, ran, nbg, g, g2 ? 1 : 0, g2 ? *g2 : g, ntx, ntiles, part, bh, err);
-  }
+#define FKP_BC(PP, TWO)                                                                                             \
+  do {                                                                                                              \
+    raise_smem_limit((const void*)k_bin_count<PP, TWO>, sm);                                                        \
+    k_bin_count<PP, TWO><<<nblk, kBinThreads, sm, s>>>(gal, ran, nbg, g, g2 ? *g2 : g, ntx, ntiles, part, bh, err); \
+  } while (0)
+#define FKP_BCP(PP)                                \
+  do {                                             \
+    if (g2) FKP_BC(PP, true); else FKP_BC(PP, false); \
+  } while (0)
+  if (g.assign == 2) FKP_BCP(2);
+  else if (g.assign == 3) FKP_BCP(3);
+  else FKP_BCP(4);
+#undef FKP_BCP
+#undef FKP_BC
   return cudaGetLastError();
 }
 
