@@ -166,7 +166,9 @@ typedef struct {
 /* Contraction of the triangle sums (eq. Factorize):
  *   FP32   CUDA cores, FP32 products, compensated FP32 sums, FP64 across slices;
  *   BF16X3 tcgen05 tensor cores, operands split v = hi + lo in BF16, products
- *          hi*hi + hi*lo + lo*hi, FP32 accumulation in tensor memory;
+ *          hi*hi + hi*lo + lo*hi, FP32 accumulation in tensor memory (where the
+ *          triangle sums are formed on fewer than N^3 points: as BF16X6, so that
+ *          they are no less exact than over N^3);
  *   BF16X6 tcgen05 tensor cores, 3-way split hi + mid + lo, the six products of
  *          order <= 2^-16: per-term error near FP32 rounding.
  * The tensor-core modes need (number of multipoles) x (shells) <= 128. */

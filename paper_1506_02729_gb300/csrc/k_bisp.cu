@@ -982,9 +982,13 @@ static int enqueue_bisp(Plan* P, const CatDev& g, const CatDev& r, int contracti
   // contraction
   const int ntri = P->ntri, nout = std::max(1, ntri) * st->nq;
   if (tensor && st->d_pairs) {
+    // The hi/lo split's dropped terms average over the points of the sum grid.
+    // On one smaller than the plan's its T_4 was further from FP64 than sums over
+    // N^3 points (400^3 -> 216^3, 22 shells: 1.9e-6 -> 2.4e-6; 300^3, 16 shells: 1.9e-6
+    // -> 2.4e-6), so there it takes the six products of the 3-way split too (1.2e-6).
+    const int nsplit = contraction == FKP_CONTRACT_BF16X3 && M == P->g.N ? 2 : 3;
     BCK(launch_contract_tc(st->d_I, N3, S, st->nl, st->d_groups, st->tc_groups, st->d_pairs, st->tc_ncols,
-                           st->d_tcpart, P->d_err + 1, st->tc_slices, st->tc_chunks,
-                           contraction == FKP_CONTRACT_BF16X3 ? 2 : 3, s));
+                           st->d_tcpart, P->d_err + 1, st->tc_slices, st->tc_chunks, nsplit, s));
     BCK(launch_tc_reduce(st->d_tcpart, st->tc_slices, st->tc_ncols, st->d_off, nout, st->d_T, s));
   } else if (!st->items.empty()) {
     const int nf = st->nl * S;

@@ -50,3 +50,19 @@ def test_tiling_edges_match_fp32(N, S, want, mode):
             # graded as B_l is: by the noise-free scale of all triangles of these shells
             d = np.maximum(np.maximum(np.abs(ref[k][m]), mono), np.median(mono))
             assert np.max(np.abs(got[k][m] - ref[k][m]) / d) < tol, k
+
+
+@pytest.mark.parametrize("N,coarser", [(128, False), (160, True)])
+def test_hi_lo_split_on_a_coarser_sum_grid(N, coarser):
+    """The hi/lo split's dropped terms average over the points of the sum grid:
+    where that is smaller than the plan's (160 -> 128) its sums are those of the
+    3-way split, on the plan's own grid they are not."""
+    import paper_1506_02729_gb300 as fkp
+    sv = mockgen.survey_small(N=N, assign=3)
+    gal, ran = mockgen.catalog(sv, 5)
+    kf = 2 * math.pi / sv.L
+    plan = fkp.Plan(sv.geometry(), (0.5 * kf, kf, 8), bshells=(3, 3, 3, 6), want=1 | B0 | B2 | B4)
+    g, r = to_device(gal), to_device(ran)
+    b3, b6 = (plan.bispectrum(g, r, contraction=c)[1] for c in (1, 2))
+    for k in ("T0", "T2", "T4"):
+        assert np.array_equal(b3[k], b6[k]) == coarser, k
