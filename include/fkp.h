@@ -197,8 +197,9 @@ int fkp_plan_sizes(const void *plan, int *nbins, int *ntriangles, size_t *worksp
  * per SM = resident blocks x x_mult: 1, 2, 4 or 8), and the threads per block
  * of the y- and z-passes (256 or 512).  The first plan of a given grid and
  * multipole order in a context times the x- and y-pass candidates on its own
- * workspace (about 12 launches of each pass) and keeps the fastest; later
- * plans of that kind reuse the choice.  The z-pass shape is fixed per grid
+ * workspace (about 12 launches of each pass, every mode carried whatever the
+ * plan's bins) and keeps the fastest; later plans of that kind reuse the
+ * choice.  The z-pass shape is fixed per grid
  * (256 threads up to N = 256, 512 above): it sets how the bin sums are
  * split into FP32 runs, so with it fixed every result is the same bit for bit
  * whatever the tuning picks (every reduction of the path has a fixed order or

@@ -298,8 +298,10 @@ int fkp::z_threads_for(int N) { return N <= 256 ? 256 : 512; }
 // Times the candidate launch schedules of the three FFT passes on the plan's
 // own workspace (zeroed: the passes' cost does not depend on the values) and
 // keeps the fastest of each; the choice is shared by later plans of the same
-// grid and multipole order in this context.  About 12 launches of each pass,
-// once per (N, lmax).
+// grid and multipole order in this context, whatever their bins and shells, so
+// the passes are timed carrying every mode and not those of the plan that
+// happens to come first.  (A per-object plan shares the choice too, made on the
+// x-pass from a grid.)  About 12 launches of each pass, once per (N, lmax).
 static int tune_schedule(Plan* P) {
   const std::pair<int, int> key{P->g.N, P->lmax};
   std::lock_guard<std::mutex> lk(P->ctx->tune_mu);
@@ -314,11 +316,17 @@ static int tune_schedule(Plan* P) {
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   CK(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
   int rc = FKP_OK;
+  PassReach all;
+  const std::vector<int> zt = reach_tiles(N, 3 * (N / 2) * (N / 2), all);
+  int* d_zt = nullptr;
   auto fail = [&](cudaError_t e, const char* what) {
     if (e != cudaSuccess && rc == FKP_OK) rc = set_error(FKP_ECUDA, "schedule tuning (%s): %s", what, cudaGetErrorString(e));
     return e != cudaSuccess;
   };
-  if (!fail(cudaEventCreate(&e0), "event") && !fail(cudaEventCreate(&e1), "event")) {
+  if (!fail(cudaEventCreate(&e0), "event") && !fail(cudaEventCreate(&e1), "event") &&
+      !fail(cudaMalloc(&d_zt, sizeof(int) * zt.size()), "tiles")) {
+    all.ztiles = d_zt;
+    fail(cudaMemcpyAsync(d_zt, zt.data(), sizeof(int) * zt.size(), cudaMemcpyHostToDevice, s), "tiles");
     fail(cudaMemsetAsync(P->d_grid, 0, N3 * 8, s), "memset");
     fail(cudaMemsetAsync(P->d_S1, 0, half * P->mt.nfields, s), "memset");
     fail(cudaMemsetAsync(P->d_S2, 0, half * P->mt.ngroups, s), "memset");
@@ -344,19 +352,19 @@ static int tune_schedule(Plan* P) {
     float bx = 1e30f, by = 1e30f, bz = 1e30f;
     for (int xm : {1, 2, 4, 8}) {
       const float t = timed([&] { return launch_xpass(P->d_grid, nullptr, P->g, P->mt, P->fp, P->d_tw, P->d_S1,
-                                                      P->ctx->nsm, s, P->reach, nullptr, xm); }, "x-pass");
+                                                      P->ctx->nsm, s, all, nullptr, xm); }, "x-pass");
       if (t < bx) { bx = t; best.x_mult = xm; }
     }
     for (int nt : {256, 512}) {
       const float t = timed([&] { return launch_ypass(P->d_S1, P->d_grid, nullptr, P->g, P->mt, P->fp, P->d_tw,
-                                                      P->d_S2, P->d_err + 1, s, P->reach, nullptr, nt); }, "y-pass");
+                                                      P->d_S2, P->d_err + 1, s, all, nullptr, nt); }, "y-pass");
       if (t < by) { by = t; best.y_threads = nt; }
     }
     // the z-pass block shape sets the partition of each k_z column into the
     // FP32 runs of the bin sums, so it is fixed per grid rather than tuned:
     // results then do not depend on the tuning (bit for bit)
     best.z_threads = z_threads_for(N);
-    bz = timed([&] { return launch_zpass(P->d_S2, P->g, P->mt, P->fp, P->d_tw, zp, P->reach, P->d_zpart, P->d_zpartc,
+    bz = timed([&] { return launch_zpass(P->d_S2, P->g, P->mt, P->fp, P->d_tw, zp, all, P->d_zpart, P->d_zpartc,
                                          P->d_err + 1, s, P->ctx->nsm, best.z_threads); }, "z-pass");
     best.ms[0] = bx;
     best.ms[1] = by;
@@ -371,6 +379,7 @@ static int tune_schedule(Plan* P) {
   if (e1) cudaEventDestroy(e1);
   cudaStreamSynchronize(s);
   cudaStreamDestroy(s);
+  if (d_zt) cudaFree(d_zt);
   return rc;
 }
 

@@ -46,3 +46,20 @@ def test_bins_that_hold_no_mode(N=64):
     kf = 2 * math.pi / sv.L
     got = fkp.Plan(sv.geometry(), (0.0, 0.1 * kf, 5)).power(to_device(gal), to_device(ran))
     assert not got["nmodes"].any() and np.isnan(got["P0"]).all()
+
+
+def test_schedule_does_not_depend_on_the_first_plans_bins(N=256):
+    """Later plans of a grid reuse the schedule that the first one timed, so it
+    is timed with every mode carried: a context whose first plan bins the
+    lowest modes only (one k_x tile of 16) reads the y-pass time of one whose
+    first plan bins to the corner (within a factor of 3; that plan's own y-pass
+    takes a tenth of it)."""
+    import paper_1506_02729_gb300 as fkp
+    sv = mockgen.survey_small(N=N, assign=2)
+    kf = 2 * math.pi / sv.L
+    full = int(math.ceil(math.sqrt(3) * N / 2))
+    ms = {}
+    for i, nb in enumerate((1, full)):  # another budget, another context
+        ms[nb] = fkp.Plan(sv.geometry(), (0.5 * kf, kf, nb), budget=(100 << 30) + i).schedule()["tuned_ms"]
+    assert ms[1][1] > ms[full][1] / 3, ms
+    assert ms[1][2] > ms[full][2] / 3, ms
