@@ -161,24 +161,56 @@ class Clocks:
 
 # ---------------------------------------------------------------------------
 # algorithmic bytes of one mock of the power step: the least traffic the
-# method needs (catalog read once, the real grid F written once and read
-# once, the k_z-power groups that carry the moment fields through the
-# z-FFT written once and read once; half = one half-spectrum field of
-# N^2 (N/2 + 1) complex FP32 values), split by stage.  The design's own
-# extra traffic (the fixed-point grid is 8 bytes per node, the x-pass spills
-# every moment half spectrum for the y-pass to read) is not algorithmic: it
-# shows in the measured DRAM `traffic` instead.
+# method needs (catalog read once, the real grid F written once and read once
+# on the rows that hold objects, the k_z-power groups that carry the moment
+# fields through the z-FFT written once and read once: on the (k_x, k_y)
+# pencils that meet a bin and the planes that hold objects, complex FP32),
+# split by stage.  The design's own extra traffic (the fixed-point grid is 8
+# bytes per node, the x-pass spills every moment half spectrum for the y-pass
+# to read) is not algorithmic: it shows in the measured DRAM `traffic` instead.
 # ---------------------------------------------------------------------------
 
-def algorithmic_bytes(N, ngroups, n_obj, cat_bytes=16):
-    half = N * N * (N // 2 + 1) * 8
-    grid = 4 * N ** 3
+def reached_pencils(N, n_max2):
+    """(k_x >= 0, k_y) pencils, off the Nyquist rows, of the modes |n|^2 <= n_max2."""
+    ky = np.arange(-(N // 2) + 1, N // 2, dtype=np.int64)
+    kx = np.arange(N // 2, dtype=np.int64)
+    return int(np.count_nonzero(kx[:, None] ** 2 + ky[None, :] ** 2 <= n_max2))
+
+
+def largest_n2(k_max, L):
+    """The largest |n|^2 with k = 2 pi |n| / L below k_max."""
+    return math.ceil((k_max * L / (2 * math.pi)) ** 2) - 1
+
+
+def occupied_rows(cats, geom):
+    """Grid rows (z, y) that the assignment taps of the catalogs' objects
+    reach, and planes z among them (numpy arrays or tensors)."""
+    N, p = int(geom["N"]), int(geom["assign"])
+    H = float(geom["L"]) / N
+    rows = np.zeros((N, N), dtype=bool)
+    for c in cats:
+        y, z = ((np.asarray(c[k].cpu() if hasattr(c[k], "cpu") else c[k], np.float64) - geom["origin"][a]) / H
+                for a, k in ((1, "y"), (2, "z")))
+        first = [np.floor(v + 0.5).astype(np.int64) - 1 if p == 3 else np.floor(v).astype(np.int64) - (p == 4)
+                 for v in (y, z)]
+        hit = np.zeros(N * N, dtype=bool)
+        hit[first[1] % N * N + first[0] % N] = True
+        cell = np.flatnonzero(hit)
+        for dz in range(p):
+            for dy in range(p):
+                rows[(cell // N + dz) % N, (cell % N + dy) % N] = True
+    return int(rows.sum()), int(rows.any(axis=1).sum())
+
+
+def algorithmic_bytes(N, ngroups, n_obj, pencils, rows, planes, cat_bytes=16):
+    grid = 4 * N * rows
+    groups = 8 * ngroups * pencils * planes
     return {
         "count": 0,                                  # reads the catalog, but the step reads it once: counted below
         "assign": cat_bytes * n_obj + grid,          # catalog (x, y, z, nbar) read once; F written once
         "xpass": grid,                               # F read once
-        "ypass": ngroups * half,                     # the k_z-power groups written once
-        "zpass": ngroups * half,                     # the groups read once (bins are negligible)
+        "ypass": groups,                             # the k_z-power groups written once
+        "zpass": groups,                             # the groups read once (bins are negligible)
     }
 
 
@@ -405,7 +437,9 @@ def run_gpu(args):
     # the launching stream between the stages of every timed step)
     st = np.mean(np.array(stage), axis=0)
     names = {"count": st[0], "assign": st[1], "xpass": st[2], "ypass": st[3], "zpass": st[4]}
-    ab = algorithmic_bytes(sv.N, 9, n_obj)  # 9 k_z-power groups carry P_0,2,4 (and P_4b)
+    rows, planes = occupied_rows((gal, ran), geom)
+    pencils = reached_pencils(sv.N, largest_n2(BINS[0] + BINS[1] * BINS[2], sv.L))
+    ab = algorithmic_bytes(sv.N, 9, n_obj, pencils, rows, planes)  # 9 k_z-power groups carry P_0,2,4 (and P_4b)
     dom = max(names, key=names.get)
     pk, src = peaks()
     achieved = ab[dom] / (names[dom] * 1e-3) / 1e9
@@ -415,6 +449,8 @@ def run_gpu(args):
             "algorithmic_bytes": ab[dom], "peak_source": src,
             "stage_ms": {k: float(v) for k, v in names.items()},
             "stage_algorithmic_bytes": ab,
+            "carried": {"pencils": pencils, "of_pencils": sv.N * (sv.N // 2 + 1), "rows": rows, "of_rows": sv.N ** 2,
+                        "planes": planes},
             "stage_frac": {k: ab[k] / (names[k] * 1e-3) / 1e9 / pk["hbm_gbs"] for k in names},
             "step": {"algorithmic_bytes": step_bytes, "ms": ms_all,
                      "frac": step_bytes / (ms_all * 1e-3) / 1e9 / pk["hbm_gbs"]}}
@@ -613,9 +649,10 @@ def run_bisp(args, gal, ran, dg, dr, stream):
     # useful tensor work, 2 x (triangles x 3 multipoles) x N^3 multiply-adds
     # times the BF16 products per term (3 hi/lo, 6 for the 3-way split),
     # against the sustained BF16 peak; the rest of the step's algorithmic bytes
-    # (catalog 20 B per object, the F and F^w grids written and read, the k_z
-    # groups of both pass sets written and read, the 3 S shell fields of both
-    # the fields' shell IFFTs written and read) against HBM
+    # (catalog 20 B per object, the F and F^w grids written and read on the rows
+    # that hold objects, the k_z groups of both pass sets written and read on the
+    # pencils that meet a bin or shell and the planes that hold objects, the 3 S
+    # shell fields of both the fields' shell IFFTs written and read) against HBM
     pk, src = peaks()
     N = args.bisp_grid
     N3 = float(N) ** 3
@@ -628,10 +665,13 @@ def run_bisp(args, gal, ran, dg, dr, stream):
         roof[name] = {"bound": "tensor", "kernel": "contraction", "useful_flop": fl, "achieved": ach,
                       "peak": pk["bf16_tflops_sustained"], "unit": "TFLOP/s",
                       "frac": ach / pk["bf16_tflops_sustained"], "peak_source": src}
-    half = N * N * (N // 2 + 1) * 8.0
     nmax = int(3 * args.bisp_nshells + 1.5)
     nobj = int(len(gal["x"]) + len(ran["x"]))
-    bts = (20.0 * nobj + 2 * 2 * 4 * N3 + 2 * (2 * 9 * half)
+    rows, planes = occupied_rows((gal, ran), sv.geometry())
+    n2w = math.ceil((3 * args.bisp_nshells + 1.5) ** 2) - 1
+    n2 = max(n2w, largest_n2(BINS[0] + BINS[1] * BINS[2], sv.L))
+    bts = (20.0 * nobj + 2 * 2 * 4 * N * rows
+           + 2 * 9 * 8.0 * planes * (reached_pencils(N, n2) + reached_pencils(N, n2w))
            + 2 * 3 * args.bisp_nshells * ((nmax + 1) * N * N * 8.0))
     st = out["modes"]["bf16x6_tcgen05"]["stage_ms"]
     oms = st["grids"] + st["F_passes"] + st["Fw_passes_and_shell_ifft"]
