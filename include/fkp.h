@@ -213,10 +213,10 @@ int fkp_plan_set_schedule(void *plan, int x_mult, int y_threads, int z_threads);
 /* CUDA graphs of the power path (default on).  With device catalogs, the
  * second fkp_power call on a plan with the same catalog pointers and sizes
  * captures the gridding, FFT passes and binning into a graph; later calls
- * with those catalogs replay it (one launch instead of about twenty).  A
- * different catalog runs the plain launches; host catalogs never use the
- * graph.  enable = 0 frees the graph and keeps plain launches.  Results
- * are the same either way. */
+ * with those catalogs replay it (one launch instead of nine kernels and
+ * their memsets).  A different catalog runs the plain launches; host catalogs
+ * never use the graph.  enable = 0 frees the graph and keeps plain launches.
+ * Results are the same either way. */
 int fkp_plan_set_graphs(void *plan, int enable);
 
 /* Random catalog shared by many mocks (Sec. III.C, Performance: gridding

@@ -705,10 +705,10 @@ static std::map<std::vector<int>, std::vector<long long>> g_count_cache;
 // transforms' random rounding averages over M^3 points only, so no grid is
 // made smaller than 128^3, where the sums cost little.  A side with a compiled
 // transform is taken up to 1.35 times the points of the smallest smooth side:
-// the runtime-size passes take about 1.5 times as long per point and are a
-// third of the work.  27 shells on 512^3: M = 256 (250 is the smallest), the
-// whole mock
-// 102 -> 18 ms; 37 shells on 360^3: M = 360 as before.
+// the runtime-size passes take 2.4 times as long per point (27 shells x 3: 6.8 ms
+// on 250^3, 3.0 on 256^3, beside 3.4 and 3.7 ms of contraction, so up to 1.6 times
+// the points would pay there).  27 shells on 512^3: M = 256 (250 is the smallest),
+// the whole mock 102 -> 18 ms; 37 shells on 360^3: M = 360 as before.
 int sum_grid(int N, int mm) {
   auto smooth = [](int n) {
     for (int f : {2, 3, 5}) while (n % f == 0) n /= f;
